@@ -334,14 +334,18 @@ apm_status apm_set_deposit_tiles(apm_ctx* ctx, int32_t on);
  *             passes, 4..32 kx columns for the y/z passes, 2..32 in FP64),
  *             halved while the CTA needs more than 200 KB of shared memory;
  *  threads[p] the runtime-planned pass's CTA size, 128 or 256;
- *  plan[p]    0: FP32 grids whose length has a compile-time plan (every
- *             {2,3,5,7}-smooth length from 36 to 84, and 128, 150, 256, 512)
- *             run the kernel specialised for it (16 lines per CTA); 1: every
- *             grid runs the runtime-planned kernel; 2 (x forward and x inverse only): as 0,
- *             and grids with M0 = M1 whose M x (M/2 + 1) plane fits 200 KB run
- *             the x and y transforms of a whole z plane in one kernel (the y
- *             pass then has no work for them; the inverse needs the window no
- *             taller than M1, which excludes a periodic root);
+ *  plan[p]    0: grids whose length has a compile-time plan run the kernel
+ *             specialised for it (16 lines per CTA, FP64 8): FP32 every
+ *             {2,3,5,7}-smooth length from 36 to 150 and 160, 168, 180, 192,
+ *             200, 216, 224, 240, 250, 256, 288, 300, 320, 360, 384, 400, 480
+ *             and 512, FP64 the same ones from 70 up; FP32 grids with
+ *             M0 = M1 from 70 to 192 run the x and y transforms of a whole z
+ *             plane in one kernel (the y pass then has no work for them; the
+ *             inverse needs the window no taller than M1, which excludes a
+ *             periodic root); 1: every grid runs the runtime-planned kernel;
+ *             2 (x forward and x inverse only): as 0, with the plane kernels
+ *             for every FP32 grid with M0 = M1 whose M x (M/2 + 1) plane fits
+ *             200 KB;
  *  max_radix  the largest stage radix of the runtime plans: 16 (FP32
  *             default; composite radices in registers) or 8 (FP64: always 8);
  *  packing    0: the grids of a level enter each work list in hierarchy order;

@@ -19,14 +19,17 @@ LIB = os.path.join(OUT_DIR, "libapm.so")
 BOUNDS_DIR = os.path.join(HERE, "_build_bounds")
 
 # (source, object, extra flags): k_fft_col.cu is compiled once per precision
-# and column pass, k_fft_fast.cu once per pass
+# and column pass, k_fft_fast.cu once per kernel, precision and group of lengths
+# (longest compilations first)
 SOURCES = [("apm_api.cu", "apm_api.o", []), ("k_green.cu", "k_green.o", []),
            ("k_deposit.cu", "k_deposit.o", []), ("k_fft_x.cu", "k_fft_x.o", []),
            ("k_field.cu", "k_field.o", []), ("k_evolve.cu", "k_evolve.o", []),
            ("apm_noalloc.cu", "apm_noalloc.o", []), ("k_order.cu", "k_order.o", [])] + [
     ("k_fft_col.cu", f"k_fft_col_{p}_{m}.o", [f"-DAPM_COL_FP64={1 if p == 'f64' else 0}", f"-DAPM_COL_MODE={m}"])
     for p in ("f32", "f64") for m in (0, 1, 2, 3)] + [
-    ("k_fft_fast.cu", f"k_fft_fast_{m}.o", [f"-DAPM_FAST_MODE={m}"]) for m in (0, 1, 2, 3, 4, 5)]
+    ("k_fft_fast.cu", f"k_fft_fast_{m}_{p}_{g}.o",
+     [f"-DAPM_FAST_MODE={m}", f"-DAPM_FAST_FP64={p}", f"-DAPM_FAST_GROUP={g}"])
+    for g in (3, 2, 1, 0) for p in (1, 0) for m in (1, 5, 0, 2, 3, 4, 6, 7) if not (p and (g == 0 or m > 5))]
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 COMMON = ["-O3", "-lineinfo", "-std=c++17", "-Xcompiler", "-fPIC", "-I", INCLUDE, "-I", CSRC,
           "--expt-relaxed-constexpr"]

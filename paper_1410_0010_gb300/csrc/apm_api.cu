@@ -53,7 +53,7 @@ struct Profiler {
 // grid's lines per CTA, the threads per CTA, and the resulting work list.
 // One launch of a pass: a contiguous range of the work list whose grids all
 // run the same kernel (fast_L = 0: the runtime-planned kernel; otherwise the
-// FP32 kernel with the compile-time plan of that length).
+// kernel with the compile-time plan of that length; negative: fused planes).
 struct PassSeg {
     int first = 0, count = 0;
     int fast_L = 0;
@@ -233,8 +233,7 @@ long long floor_div(long long a, long long b) {
     return q;
 }
 
-// the FP32 column passes use the compile-time plans of fft_fast.cuh where a
-// length has one (APM_FFT_FAST=0 keeps every pass on the runtime-planned
+// the passes use the compile-time plans of fft_fast.cuh where a length has one (APM_FFT_FAST=0 keeps every pass on the runtime-planned
 // kernels, for comparison)
 bool fft_fast_enabled() {
     const char* v = std::getenv("APM_FFT_FAST");
@@ -341,6 +340,19 @@ void build_csr(const std::vector<std::pair<std::array<long long, 3>, std::array<
 
 apm_status cuda_status(cudaError_t e) { return e == cudaSuccess ? APM_OK : APM_E_CUDA; }
 
+// the compile-time-planned kernel of pass q in a segment of kind `kind` (L, or
+// -L for the fused plane kernels), for component comp of a spectral gradient
+int fast_kernel(int q, int kind, int comp) {
+    if (kind < 0) return q == kPassXf ? kFastXy : kFastYx;
+    switch (q) {
+        case kPassXf: return kFastXf;
+        case kPassYf: return kFastYf;
+        case kPassZ: return comp > 0 ? kFastZg : kFastZ;   // the table times -i D_comp
+        case kPassYi: return kFastYi;
+        default: return kFastXi;
+    }
+}
+
 // Work list of FFT pass q over the grids of a level for a buffer budget and a
 // CTA size: each grid's lines per CTA (halved until the CTA fits its shared
 // memory), one chunk per CTA.  The lines batch whole lines, so the shape never
@@ -354,33 +366,36 @@ apm_status build_pass(apm_ctx* c, const Level& L, int q, int budget, int threads
     P.count.assign(ng, 0);
     P.seg_of.assign(ng, 0);
     P.seg.clear();
-    // the kernel of each grid: a compile-time plan for the FP32 passes of its
-    // length, if there is one (not for the x-forward pass while its bulk-copy
+    // the kernel of each grid: the compile-time plan of its length, if there is
+    // one (not for the x-forward pass while its bulk-copy
     // wait is made to run out); a spectral gradient's components run the z pass
     // on the same work list (k_col_fast MODE 3, or k_col MODE 3)
     std::vector<int> fast(ng, 0), lens(ng, 0);
     const bool row = q == kPassXf || q == kPassXi;
-    // with plan 2 on the x-forward pass, a grid with M0 = M1 whose plane fits
-    // runs the fused x + y forward (k_xy_fast) as its x-forward segment (kind
+    // with plan 2 on the x-forward pass (or plan 0 and a length of
+    // fast_xy_default), a grid with M0 = M1 whose plane fits runs the fused x + y forward (k_xy_fast) as its x-forward segment (kind
     // -L) and has no y-forward work (kind kSkip); other grids run plan 0
     constexpr int kSkip = INT_MIN;
+    auto fuses = [&](int x_pass, int len) {
+        return L.plan[x_pass] == 2 || (L.plan[x_pass] == 0 && fast_xy_default(len));
+    };
     // (the kernel stores row pair p in plane rows 2p, 2p + 1: an odd G1 needs
     // G1 < M1, so that the pairs fit the M1 rows of the plane)
     auto fused_xy = [&](const GridDev& g) {
-        return !f64 && L.plan[kPassXf] == 2 && fft_fast_enabled() && !fault_wait() && g.M[0] == g.M[1] &&
+        return !f64 && fuses(kPassXf, g.M[0]) && fft_fast_enabled() && !fault_wait() && g.M[0] == g.M[1] &&
                fast_xy_length(g.M[0]) && 2 * ((g.G[1] + 1) / 2) <= g.M[1];
     };
     // ... and the fused y + x inverse (k_yx_fast) as its x-inverse segment when
     // the window's row pairs are distinct rows of the transform (2 ceil(W1/2)
     // <= M1: a periodic root, whose window is taller than M1, is excluded)
     auto fused_yx = [&](const GridDev& g) {
-        return !f64 && L.plan[kPassXi] == 2 && fft_fast_enabled() && g.M[0] == g.M[1] && fast_xy_length(g.M[0]) &&
+        return !f64 && fuses(kPassXi, g.M[0]) && fft_fast_enabled() && g.M[0] == g.M[1] && fast_xy_length(g.M[0]) &&
                2 * ((g.W[1] + 1) / 2) <= g.M[1];
     };
     for (int k = 0; k < ng; ++k) {
         const GridDev& g = L.hg[k];
         lens[k] = row ? g.M[0] : (q == kPassZ ? g.M[2] : g.M[1]);
-        if (!f64 && L.plan[q] != 1 && fft_fast_enabled() && fast_length(lens[k]) &&
+        if (L.plan[q] != 1 && fft_fast_enabled() && fast_length(lens[k], f64) &&
             !(q == kPassXf && fault_wait()))
             fast[k] = lens[k];
         if ((q == kPassXf || q == kPassYf) && fused_xy(g)) fast[k] = q == kPassXf ? -lens[k] : kSkip;
@@ -400,7 +415,7 @@ apm_status build_pass(apm_ctx* c, const Level& L, int q, int budget, int threads
         if (kind == kSkip) {            // fused into the x-forward segment: no chunks
             for (int k = 0; k < ng; ++k)
                 if (fast[k] == kSkip) {
-                    P.lines[k] = kFastTx;
+                    P.lines[k] = fast_lines(f64);
                     P.first[k] = 0;
                     P.count[k] = 0;
                     P.seg_of[k] = 0;
@@ -415,7 +430,7 @@ apm_status build_pass(apm_ctx* c, const Level& L, int q, int budget, int threads
             const GridDev& g = L.hg[k];
             const int len = lens[k];
             if (kind < 0) {             // fused x + y passes: one chunk per z (window) plane
-                P.lines[k] = kFastNp;
+                P.lines[k] = fast_lines(f64);
                 P.first[k] = (int)list.size();
                 P.seg_of[k] = (int)P.seg.size();
                 sg.smem = fast_xy_smem(len);
@@ -426,8 +441,8 @@ apm_status build_pass(apm_ctx* c, const Level& L, int q, int budget, int threads
             }
             int lines;
             if (kind) {
-                lines = row ? kFastNp : kFastTx;
-                sg.smem = row ? fast_row_smem(len) : fast_col_smem(len);
+                lines = fast_lines(f64);
+                sg.smem = row ? fast_row_smem(len, f64) : fast_col_smem(len, f64);
             } else {
                 lines = fft_pass_lines(q, len, budget, f64);
                 while (lines > 1 && fft_pass_smem(q, len, lines, csz, g.G[0]) > (size_t)kFftSmemLimit) lines /= 2;
@@ -450,6 +465,12 @@ apm_status build_pass(apm_ctx* c, const Level& L, int q, int budget, int threads
             P.count[k] = (int)list.size() - P.first[k];
         }
         sg.count = (int)list.size() - sg.first;
+        if (kind) {
+            cudaError_t e = configure_fft_fast(fast_kernel(q, kind, 0), f64, std::abs(kind));
+            if (e == cudaSuccess && q == kPassZ && c->cfg.gradient == APM_GRAD_SPECTRAL)
+                e = configure_fft_fast(fast_kernel(q, kind, 1), f64, std::abs(kind));
+            if (e != cudaSuccess) return APM_E_CUDA;
+        }
         P.seg.push_back(sg);
     }
     P.budget = budget;
@@ -503,19 +524,9 @@ cudaError_t run_seg(apm_ctx* c, const Level& L, int q, const PassPlan& P, const 
     a.inject_wait = fault_wait() ? 1 : 0;
     a.comp = comp;
     if (c->cfg.gradient == APM_GRAD_SPECTRAL && (q == kPassYi || q == kPassXi)) a.wsB = c->wsC;
-    if (sg.fast_L < 0)
-        return q == kPassXf ? launch_fft_xy_fast(-sg.fast_L, a, (const int64_t* const*)d_gmf, s)
-                            : launch_fft_yx_fast(-sg.fast_L, a, d_phis, s);
-    if (sg.fast_L) {
-        switch (q) {
-            case kPassYf: return launch_fft_yf_fast(sg.fast_L, a, s);
-            case kPassZ:   // component comp > 0 of a spectral gradient: the table times -i D_comp
-                return comp > 0 ? launch_fft_zgrad_fast(sg.fast_L, a, s) : launch_fft_z_fast(sg.fast_L, a, s);
-            case kPassYi: return launch_fft_yi_fast(sg.fast_L, a, s);
-            case kPassXf: return launch_fft_xf_fast(sg.fast_L, a, (const int64_t* const*)d_gmf, s);
-            default: return launch_fft_xi_fast(sg.fast_L, a, d_phis, s);
-        }
-    }
+    if (sg.fast_L)
+        return launch_fft_fast(fast_kernel(q, sg.fast_L, comp), f64, std::abs(sg.fast_L), a,
+                               (const int64_t* const*)d_gmf, d_phis, s);
     switch (q) {
         case kPassXf:
             return f64 ? launch_fft_xf<double>(a, (const int64_t* const*)d_gmf, s)
@@ -1460,7 +1471,7 @@ apm_status apm_autotune_level(apm_ctx* c, int32_t level, const int64_t* const* g
             for (int k = 0; k < (int)L.hg.size(); ++k) {
                 const GridDev& g = L.hg[k];
                 const int len = (q == kPassXf || q == kPassXi) ? g.M[0] : (q == kPassZ ? g.M[2] : g.M[1]);
-                any_fast = any_fast || fast_length(len);
+                any_fast = any_fast || fast_length(len, f64);
             }
             if (any_fast && fft_fast_enabled())
                 st = try_knob([&] { L.plan[q] = 0; }, [&] { L.plan[q] = 1; });

@@ -140,43 +140,72 @@ inline void fft_plan_reversed(const FftPlan1D& f, FftPlan1D* r) {
     }
 }
 
-// ---- FP32 transforms with compile-time plans (fft_fast.cuh) ------------------
+// ---- transforms with compile-time plans (fft_fast.cuh) -----------------------
 // Lengths with a compile-time radix plan: X(L, R1, R2, R3); R3 = 1 for two
-// stages.  Every radix is one the FP32 butterflies compute in registers.
-#define APM_FAST_LENGTHS(X) \
+// stages.  Every radix is one the butterflies compute in registers.  They
+// cover every {2,3,5,7}-smooth length from 36 to 150 (a refined grid of N cells
+// takes the smallest one >= N + 20; an isolated root of N cells takes 2 N) and
+// the usual longer ones; the rest runs the runtime-planned kernels.  The lists
+// are four groups so that they compile in parallel.  FP64 takes groups 1 to 3:
+// below 70 points a transform is too short for the FP64 pipe to bound it.
+#define APM_FAST_LENGTHS_0(X) \
     X(36, 6, 6, 1) X(40, 8, 5, 1) X(42, 7, 6, 1) X(45, 9, 5, 1) X(48, 8, 6, 1) X(49, 7, 7, 1) \
-    X(50, 10, 5, 1) X(54, 9, 6, 1) X(56, 8, 7, 1) X(60, 10, 6, 1) X(63, 9, 7, 1) X(64, 8, 8, 1) \
+    X(50, 10, 5, 1) X(54, 9, 6, 1) X(56, 8, 7, 1) X(60, 10, 6, 1) X(63, 9, 7, 1) X(64, 8, 8, 1)
+#define APM_FAST_LENGTHS_1(X) \
     X(70, 10, 7, 1) X(72, 9, 8, 1) X(75, 15, 5, 1) X(80, 10, 8, 1) X(81, 9, 9, 1) X(84, 12, 7, 1) \
-    X(128, 16, 8, 1) X(150, 15, 10, 1) X(256, 16, 16, 1) X(512, 8, 8, 8)
-constexpr int kFastTx = 16;   // kx columns per CTA of a fast column pass
-constexpr int kFastNp = 16;   // complex lines (row pairs) per CTA of a fast x pass
+    X(90, 10, 9, 1) X(96, 12, 8, 1) X(98, 14, 7, 1) X(100, 10, 10, 1) X(105, 15, 7, 1) X(108, 12, 9, 1)
+#define APM_FAST_LENGTHS_2(X) \
+    X(112, 14, 8, 1) X(120, 12, 10, 1) X(125, 5, 5, 5) X(126, 14, 9, 1) X(128, 16, 8, 1) X(135, 15, 9, 1) \
+    X(140, 14, 10, 1) X(144, 12, 12, 1) X(147, 7, 7, 3) X(150, 15, 10, 1)
+#define APM_FAST_LENGTHS_3(X) \
+    X(160, 16, 10, 1) X(168, 14, 12, 1) X(180, 15, 12, 1) X(192, 16, 12, 1) X(200, 10, 5, 4) X(216, 6, 6, 6) \
+    X(224, 16, 14, 1) X(240, 16, 15, 1) X(250, 10, 5, 5) X(256, 16, 16, 1) X(288, 8, 6, 6) X(300, 10, 6, 5) \
+    X(320, 8, 8, 5) X(360, 10, 6, 6) X(384, 8, 8, 6) X(400, 10, 8, 5) X(480, 10, 8, 6) X(512, 8, 8, 8)
+constexpr int kFastGroups = 4;
+// lines per CTA: kx columns of a column pass, complex lines (row pairs) of an
+// x pass; 128 bytes of each HBM row in both precisions
+constexpr int fast_lines(bool f64) { return f64 ? 8 : 16; }
 
-constexpr int fast_gcd(int a, int b) { return b == 0 ? a : fast_gcd(b, a % b); }
-// threads of a fast pass CTA for `lines` lines: lines x the gcd of the stages'
-// butterfly counts (so the trips divide evenly), brought into [64, 256] by
-// powers of two
+// threads of a fast pass CTA for `lines` lines: whole warps, and among 96, 128,
+// 160 and 192 (64 where every stage has fewer items) the one whose stages leave
+// the fewest threads without a butterfly in their last trip
 constexpr int fast_threads(int r1, int r2, int r3, int lines) {
     const int L = r1 * r2 * r3;
-    int g = fast_gcd(L / r1, L / r2);
-    if (r3 > 1) g = fast_gcd(g, L / r3);
-    int nt = lines * g;
-    while (nt < 64) nt *= 2;
-    while (nt > 256 && nt % 2 == 0) nt /= 2;
-    return nt;
+    const int items[3] = {L / r1 * lines, L / r2 * lines, r3 > 1 ? L / r3 * lines : 0};
+    int best = 64, best_cost = 1 << 30;
+    for (int nt = 64; nt <= 192; nt += 32) {
+        int cost = 0;
+        for (int k = 0; k < 3; ++k) cost += (items[k] + nt - 1) / nt * nt;
+        if (cost < best_cost || (cost == best_cost && nt <= 160)) {
+            best = nt;
+            best_cost = cost;
+        }
+    }
+    return best;
 }
-// 1 when length L has a compile-time plan
-inline bool fast_length(int L) {
-#define APM_FAST_CASE(LL, A, B, C) if (L == LL) return true;
-    APM_FAST_LENGTHS(APM_FAST_CASE)
+// the group of length L's compile-time plan, -1 without one
+inline int fast_group(int L, bool f64) {
+#define APM_FAST_CASE(LL, A, B, C) if (L == LL) return g;
+    int g = 0;
+    if (!f64) { APM_FAST_LENGTHS_0(APM_FAST_CASE) }
+    g = 1;
+    APM_FAST_LENGTHS_1(APM_FAST_CASE)
+    g = 2;
+    APM_FAST_LENGTHS_2(APM_FAST_CASE)
+    g = 3;
+    APM_FAST_LENGTHS_3(APM_FAST_CASE)
 #undef APM_FAST_CASE
-    return false;
+    return -1;
 }
+inline bool fast_length(int L, bool f64) { return fast_group(L, f64) >= 0; }
+constexpr size_t fast_csz(bool f64) { return f64 ? sizeof(double2) : sizeof(float2); }
 // dynamic shared memory of a fast column-pass CTA: the buffer and the twiddles
-inline size_t fast_col_smem(int L) { return (size_t)(L * kFastTx + L) * sizeof(float2); }
-// ... and of a fast x-pass CTA (rows padded to kFastNp + 1 lines)
-// (the x-inverse pads its lines by one element every R_last positions: at
-// most L / 2 more)
-inline size_t fast_row_smem(int L) { return (size_t)(L * (kFastNp + 1) + L / 2 + L) * sizeof(float2); }
+constexpr size_t fast_col_smem(int L, bool f64) { return (size_t)(L * fast_lines(f64) + L) * fast_csz(f64); }
+// ... and of a fast x-pass CTA (rows padded to one line more; the x-inverse
+// pads its lines by one element every R_last positions: at most L / 2 more)
+constexpr size_t fast_row_smem(int L, bool f64) {
+    return (size_t)(L * (fast_lines(f64) + 1) + L / 2 + L) * fast_csz(f64);
+}
 
 // Column-pass chunks carry (kx tile, line index of the other axis) as
 // (kt << 20) | other: other < 2^20, kt < 2^11.
@@ -521,26 +550,32 @@ template <typename T>
 cudaError_t launch_fft_zgrad(const FftArgs& a, cudaStream_t s);
 template <typename T>
 cudaError_t launch_fft_xi(const FftArgs& a, void* const* phis, cudaStream_t s);
-// FP32 column passes of length L with a compile-time plan (fast_length(L)):
-// yf, z (with the table) and yi; a.chunks hold kFastTx columns per CTA
-cudaError_t launch_fft_yf_fast(int L, const FftArgs& a, cudaStream_t s);
-cudaError_t launch_fft_z_fast(int L, const FftArgs& a, cudaStream_t s);
-cudaError_t launch_fft_zgrad_fast(int L, const FftArgs& a, cudaStream_t s);   // spectral component a.comp
-cudaError_t launch_fft_yi_fast(int L, const FftArgs& a, cudaStream_t s);
-// the fused x + y forward over one z plane (k_xy_fast) of a grid with
-// M0 = M1 = L: the plane (L rows x L/2 + 1 columns) and the twiddles
+// The passes with a compile-time plan of length L (fast_length), by kernel:
+// the y forward, z (with the table) and y inverse column passes, the x forward
+// and x inverse, the z pass of spectral component a.comp, and (FP32) the fused
+// plane kernels: x + y forward over one z plane (k_xy_fast) of a grid with
+// M0 = M1 = L, and y + x inverse over one window plane (k_yx_fast) for grids
+// whose window fits the transform (W1 <= M1).
+enum { kFastYf = 0, kFastZ, kFastYi, kFastXf, kFastXi, kFastZg, kFastXy, kFastYx, kFastKernels };
 constexpr int kFastXyThreads = 384;
-inline size_t fast_xy_smem(int L) { return (size_t)(L * (L / 2 + 1) + L) * sizeof(float2); }
-inline bool fast_xy_length(int L) { return fast_length(L) && fast_xy_smem(L) <= (size_t)kFftSmemLimit; }
-cudaError_t launch_fft_xy_fast(int L, const FftArgs& a, const int64_t* const* gmf, cudaStream_t s);
-// ... and its inverse, the fused y + x inverse over one window plane
-// (k_yx_fast), for grids whose window fits the transform (W1 <= M1)
-cudaError_t launch_fft_yx_fast(int L, const FftArgs& a, void* const* phis, cudaStream_t s);
-
-// FP32 x passes of length M0 = L with a compile-time plan: kFastNp row pairs
-// per CTA (both use fast_row_smem)
-cudaError_t launch_fft_xf_fast(int L, const FftArgs& a, const int64_t* const* gmf, cudaStream_t s);
-cudaError_t launch_fft_xi_fast(int L, const FftArgs& a, void* const* phis, cudaStream_t s);
+// the plane (L rows x L/2 + 1 columns) and the twiddles
+constexpr size_t fast_xy_smem(int L) { return (size_t)(L * (L / 2 + 1) + L) * sizeof(float2); }
+inline bool fast_xy_length(int L) { return fast_length(L, false) && fast_xy_smem(L) <= (size_t)kFftSmemLimit; }
+// plan 0 runs the fused planes for M0 = M1 = L from 70 to 192 (plan 2: wherever
+// a plane fits).  Measured, unfused against fused, one level's five passes in
+// us: 8 grids of L = 84 65.8 / 51.2, 27 of them 166.5 / 165.1, 8 of 120 148.9 /
+// 133.5, 1 of 150 63.7 / 43.1, 27 of 150 1028 / 765, 8 of 160 451 / 319, 8 of
+// 192 766 / 678, an isolated 96^3 root (192) 71.8 / 53.4.  Above 192 one plane
+// fills an SM and the passes one by one are faster (8 of 216: 950 / 1047, a
+// periodic 200^3 root 127 / 157).  Below 70 plan 0 keeps its separate passes,
+// as it always had, although the planes are faster there too (1 of 45: 26.6 /
+// 16.5): plan 2 asks for them.
+inline bool fast_xy_default(int L) { return L >= 70 && L <= 192; }
+cudaError_t launch_fft_fast(int kernel, bool f64, int L, const FftArgs& a, const int64_t* const* gmf,
+                            void* const* phis, cudaStream_t s);
+// allows the kernel its shared memory (once per kernel and device before its
+// first launch; not inside a stream capture)
+cudaError_t configure_fft_fast(int kernel, bool f64, int L);
 
 // accelerations + parent carry for the four-point and spectral gradients (the
 // two-point one runs launch_accel), on launch_accel's block work list

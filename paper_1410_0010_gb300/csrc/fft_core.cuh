@@ -174,7 +174,20 @@ template <typename T, int DIR> struct Dft<T, DIR, 8> {
     }
 };
 
-// odd prime R (3, 5, 7): with a_k = v_k + v_{R-k}, b_k = v_k - v_{R-k}
+template <typename T, int DIR> struct Dft<T, DIR, 3> {
+    // as the general form below, with the one sine product folded into the
+    // output sums (an FMA each)
+    __device__ static void run(C<T>* v) {
+        constexpr T c = (T)ct_cs(1, 3, false), sn = (T)(DIR * ct_cs(1, 3, true));
+        const C<T> a = add<T>(v[1], v[2]), b = sub<T>(v[1], v[2]), x0 = v[0];
+        const C<T> re = mk<T>(x0.x + c * a.x, x0.y + c * a.y);
+        v[0] = add<T>(x0, a);
+        v[1] = mk<T>(re.x - sn * b.y, re.y + sn * b.x);
+        v[2] = mk<T>(re.x + sn * b.y, re.y - sn * b.x);
+    }
+};
+
+// odd prime R (5, 7; 3 above): with a_k = v_k + v_{R-k}, b_k = v_k - v_{R-k}
 // (k = 1 .. (R-1)/2),
 //   X_0     = v_0 + sum_k a_k
 //   X_q     = v_0 + sum_k cos(2 pi qk/R) a_k + DIR i sum_k sin(2 pi qk/R) b_k
@@ -213,35 +226,58 @@ template <typename T, int DIR, int R> struct Dft {
     }
 };
 
-// Composite radix R = R1 R2 in registers (Cooley-Tukey inside the butterfly):
-// with n = R2 n1 + n2 and k = k1 + R1 k2,
+// Composite radix R = R1 R2 in registers.
+// Coprime R1, R2 (6, 10, 12, 14, 15): the prime-factor form (Good 1958, Thomas
+// 1963).  With n = R2 n1 + R1 n2 and k = k1 mod R1 = k2 mod R2 (both mod R),
+//   X[k] = sum_n2 w_R2^(n2 k2) sum_n1 v[n] w_R1^(n1 k1)
+// exactly: no twiddles between the two steps.  The index maps are
+// compile-time, so it is the same adds with fewer multiplies (radix 15: 8
+// complex constant products less, a fifth of its arithmetic).
+// Otherwise (9, 16) Cooley-Tukey inside the butterfly: with n = R2 n1 + n2 and
+// k = k1 + R1 k2,
 //   X[k1 + R1 k2] = sum_n2 w_R2^(n2 k2) w_R^(n2 k1) sum_n1 v[R2 n1 + n2] w_R1^(n1 k1),
 // w_m = exp(DIR 2 pi i / m); every w_R^(n2 k1) is a compile-time constant.
+constexpr int ct_gcd(int a, int b) { return b == 0 ? a : ct_gcd(b, a % b); }
+constexpr int ct_inverse(int a, int m) {   // a^-1 mod m
+    for (int x = 1; x < m; ++x)
+        if (a % m * x % m == 1) return x;
+    return 0;
+}
 template <typename T, int DIR, int R1, int R2>
 struct DftC {
     __device__ static void run(C<T>* v) {
         constexpr int R = R1 * R2;
+        constexpr bool PFA = ct_gcd(R1, R2) == 1;
         sfor<R2>([&](auto n2i) {
             constexpr int n2 = decltype(n2i)::value;
             C<T> t[R1];
-#pragma unroll
-            for (int n1 = 0; n1 < R1; ++n1) t[n1] = v[R2 * n1 + n2];
+            sfor<R1>([&](auto n1i) {
+                constexpr int n1 = decltype(n1i)::value;
+                t[n1] = v[PFA ? (R2 * n1 + R1 * n2) % R : R2 * n1 + n2];
+            });
             Dft<T, DIR, R1>::run(t);
             sfor<R1>([&](auto k1i) {
                 constexpr int k1 = decltype(k1i)::value;
-                v[R2 * k1 + n2] = mul_root<T, DIR, n2 * k1, R>(t[k1]);
+                if constexpr (PFA) v[(R2 * k1 + R1 * n2) % R] = t[k1];
+                else v[R2 * k1 + n2] = mul_root<T, DIR, n2 * k1, R>(t[k1]);
             });
         });
         C<T> out[R];
-#pragma unroll
-        for (int k1 = 0; k1 < R1; ++k1) {
+        sfor<R1>([&](auto k1i) {
+            constexpr int k1 = decltype(k1i)::value;
             C<T> t[R2];
-#pragma unroll
-            for (int n2 = 0; n2 < R2; ++n2) t[n2] = v[R2 * k1 + n2];
+            sfor<R2>([&](auto n2i) {
+                constexpr int n2 = decltype(n2i)::value;
+                t[n2] = v[PFA ? (R2 * k1 + R1 * n2) % R : R2 * k1 + n2];
+            });
             Dft<T, DIR, R2>::run(t);
-#pragma unroll
-            for (int k2 = 0; k2 < R2; ++k2) out[k1 + R1 * k2] = t[k2];
-        }
+            sfor<R2>([&](auto k2i) {
+                constexpr int k2 = decltype(k2i)::value;
+                constexpr int k = PFA ? (R2 * ct_inverse(R2, R1) * k1 + R1 * ct_inverse(R1, R2) * k2) % R
+                                      : k1 + R1 * k2;
+                out[k] = t[k2];
+            });
+        });
 #pragma unroll
         for (int q = 0; q < R; ++q) v[q] = out[q];
     }

@@ -1,7 +1,7 @@
-// fft_fast.cuh -- FP32 FFT passes with the transform length and its radices
-// fixed at compile time (the lengths of fast_radices()), for the same five
-// passes, work lists and data layout as fft_core.cuh's runtime-planned
-// kernels, which remain the path for every other length and for FP64.
+// fft_fast.cuh -- FFT passes with the transform length and its radices fixed at
+// compile time (APM_FAST_LENGTHS), for the same five passes, work lists and
+// data layout as fft_core.cuh's runtime-planned kernels, which remain the path
+// for every other length (and for the short FP64 ones, fast_length()).
 //
 // A length L = R1 R2 (R3) is transformed in place in ONE shared-memory
 // buffer, element-major (line fastest):
@@ -28,14 +28,14 @@ namespace {
 
 // DFT of radix R in registers: the building blocks of fft_core.cuh (direct
 // radices 2, 3, 4, 5, 7, 8 and composites R1 x R2)
-template <int DIR, int R> struct FastDft;
+template <typename T, int DIR, int R> struct FastDft;
 #define APM_FAST_DFT_DIRECT(R) \
-    template <int DIR> struct FastDft<DIR, R> { \
-        __device__ __forceinline__ static void run(float2* v) { Dft<float, DIR, R>::run(v); } \
+    template <typename T, int DIR> struct FastDft<T, DIR, R> { \
+        __device__ __forceinline__ static void run(C<T>* v) { Dft<T, DIR, R>::run(v); } \
     };
 #define APM_FAST_DFT_COMPOSITE(R, A, B) \
-    template <int DIR> struct FastDft<DIR, R> { \
-        __device__ __forceinline__ static void run(float2* v) { DftC<float, DIR, A, B>::run(v); } \
+    template <typename T, int DIR> struct FastDft<T, DIR, R> { \
+        __device__ __forceinline__ static void run(C<T>* v) { DftC<T, DIR, A, B>::run(v); } \
     };
 APM_FAST_DFT_DIRECT(2)
 APM_FAST_DFT_DIRECT(3)
@@ -88,9 +88,9 @@ template <int A, int B, int Cc> struct FastPlan {
 //  IN_G: the inputs come from global memory (natural index = position)
 //  OUT_G: the outputs go to global memory (natural index from the digits;
 //         only for the last stage, whose digits are complete)
-template <class P, int S_, int TX, int NT, bool IN_G, bool OUT_G, class GIN, class GOUT, int PITCH = TX,
+template <typename T, class P, int S_, int TX, int NT, bool IN_G, bool OUT_G, class GIN, class GOUT, int PITCH = TX,
           int DIR = -1>
-__device__ __forceinline__ void fast_dif_stage(float2* buf, const float2* __restrict__ tw, const GIN& gin,
+__device__ __forceinline__ void fast_dif_stage(C<T>* buf, const C<T>* __restrict__ tw, const GIN& gin,
                                                const GOUT& gout) {
     constexpr int R = P::radix(S_), S = P::inner(S_), L = P::L;
     constexpr int NB = L / R, ITEMS = NB * TX, TRIPS = (ITEMS + NT - 1) / NT;
@@ -102,16 +102,16 @@ __device__ __forceinline__ void fast_dif_stage(float2* buf, const float2* __rest
         const int line = i % TX, b = i / TX;
         const int hi = b / S, lo = b - hi * S;
         const int base = hi * R * S + lo;
-        float2 v[R];
+        C<T> v[R];
 #pragma unroll
         for (int k = 0; k < R; ++k) {
             if constexpr (IN_G) v[k] = gin.ld(base + k * S);
             else v[k] = buf[(base + k * S) * PITCH + line];
         }
-        FastDft<DIR, R>::run(v);
+        FastDft<T, DIR, R>::run(v);
         if constexpr (S > 1) {
 #pragma unroll
-            for (int k = 1; k < R; ++k) v[k] = mul<float>(v[k], twid<float, DIR>(tw, lo * k * TWS));
+            for (int k = 1; k < R; ++k) v[k] = mul<T>(v[k], twid<T, DIR>(tw, lo * k * TWS));
         }
         static_assert(!OUT_G || S == 1, "global output only from the last stage");
         const int nat0 = OUT_G ? P::natural(base) : 0;
@@ -130,8 +130,8 @@ __device__ __forceinline__ void fast_dif_stage(float2* buf, const float2* __rest
 //        only for the first inverse stage, the last digit)
 //  OUT_G: the outputs go to global memory (the first digit's stage: the
 //         positions are then natural indices)
-template <class P, int S_, int TX, int NT, bool IN_G, bool OUT_G, class GIN, class GOUT, int PITCH = TX>
-__device__ __forceinline__ void fast_dit_stage(float2* buf, const float2* __restrict__ tw, const GIN& gin,
+template <typename T, class P, int S_, int TX, int NT, bool IN_G, bool OUT_G, class GIN, class GOUT, int PITCH = TX>
+__device__ __forceinline__ void fast_dit_stage(C<T>* buf, const C<T>* __restrict__ tw, const GIN& gin,
                                                const GOUT& gout) {
     constexpr int R = P::radix(S_), S = P::inner(S_), L = P::L;
     constexpr int NB = L / R, ITEMS = NB * TX, TRIPS = (ITEMS + NT - 1) / NT;
@@ -143,7 +143,7 @@ __device__ __forceinline__ void fast_dit_stage(float2* buf, const float2* __rest
         const int line = i % TX, b = i / TX;
         const int hi = b / S, lo = b - hi * S;
         const int base = hi * R * S + lo;
-        float2 v[R];
+        C<T> v[R];
         static_assert(!IN_G || S == 1, "global input only to the first inverse stage");
         const int nat0 = IN_G ? P::natural(base) : 0;
 #pragma unroll
@@ -153,9 +153,9 @@ __device__ __forceinline__ void fast_dit_stage(float2* buf, const float2* __rest
         }
         if constexpr (S > 1) {
 #pragma unroll
-            for (int k = 1; k < R; ++k) v[k] = mul<float>(v[k], twid<float, 1>(tw, lo * k * TWS));
+            for (int k = 1; k < R; ++k) v[k] = mul<T>(v[k], twid<T, 1>(tw, lo * k * TWS));
         }
-        FastDft<1, R>::run(v);
+        FastDft<T, 1, R>::run(v);
 #pragma unroll
         for (int k = 0; k < R; ++k) {
             if constexpr (OUT_G) gout.st(base + k * S, v[k]);
@@ -166,8 +166,8 @@ __device__ __forceinline__ void fast_dit_stage(float2* buf, const float2* __rest
 
 // The z pass's middle: the forward's last stage (S = 1), the table multiply at
 // the natural index, and the inverse's first stage on the same registers.
-template <class P, int TX, int NT, class TAB>
-__device__ __forceinline__ void fast_mid_stage(float2* buf, const TAB& tabf) {
+template <typename T, class P, int TX, int NT, class TAB>
+__device__ __forceinline__ void fast_mid_stage(C<T>* buf, const TAB& tabf) {
     constexpr int SL = P::NST - 1;
     constexpr int R = P::radix(SL), L = P::L;
     constexpr int NB = L / R, ITEMS = NB * TX, TRIPS = (ITEMS + NT - 1) / NT;
@@ -177,15 +177,15 @@ __device__ __forceinline__ void fast_mid_stage(float2* buf, const TAB& tabf) {
         if (ITEMS % NT != 0 && i >= ITEMS) break;
         const int line = i % TX, hi = i / TX;
         const int base = hi * R;
-        float2 v[R];
+        C<T> v[R];
 #pragma unroll
         for (int k = 0; k < R; ++k) v[k] = buf[(base + k) * TX + line];
-        FastDft<-1, R>::run(v);
+        FastDft<T, -1, R>::run(v);
         // natural index of output k: the digits of hi, then k as the last digit
         const int k0 = P::natural(base);
 #pragma unroll
         for (int k = 0; k < R; ++k) v[k] = tabf.apply(k0 + k * (L / R), v[k]);
-        FastDft<1, R>::run(v);
+        FastDft<T, 1, R>::run(v);
 #pragma unroll
         for (int k = 0; k < R; ++k) buf[(base + k) * TX + line] = v[k];
     }
@@ -194,22 +194,22 @@ __device__ __forceinline__ void fast_mid_stage(float2* buf, const TAB& tabf) {
 // Global element n of this thread's line: p[n stride] for n < n_in (zero
 // beyond: the padding); nothing for a dead line (kx >= Hx).  Offsets stay
 // 32-bit (lines of at most 1024 elements, strides below 1024 x 513).
-struct FastIn {
-    const float2* __restrict__ p;
+template <typename T> struct FastIn {
+    const C<T>* __restrict__ p;
     int stride, n;
     bool live;
-    __device__ __forceinline__ float2 ld(int i) const {
-        return (live && i < n) ? p[i * stride] : make_float2(0.f, 0.f);
+    __device__ __forceinline__ C<T> ld(int i) const {
+        return (live && i < n) ? p[i * stride] : mk<T>(T(0), T(0));
     }
 };
 // Output element i at window index w = (i - s0) mod L, written when w < n, and
 // again at w + L when that is inside the window too (a periodic root's window
 // N + 4 exceeds M = N).
-template <int L> struct FastOut {
-    float2* __restrict__ p;
+template <typename T, int L> struct FastOut {
+    C<T>* __restrict__ p;
     int stride, n, s0;
     bool live;
-    __device__ __forceinline__ void st(int i, float2 v) const {
+    __device__ __forceinline__ void st(int i, C<T> v) const {
         if (!live) return;
         int w = i - s0;
         if (w < 0) w += L;
@@ -219,11 +219,11 @@ template <int L> struct FastOut {
 };
 
 // Output element i of a pass with no window (the y forward: all L outputs)
-struct FastOutAll {
-    float2* __restrict__ p;
+template <typename T> struct FastOutAll {
+    C<T>* __restrict__ p;
     int stride;
     bool live;
-    __device__ __forceinline__ void st(int i, float2 v) const {
+    __device__ __forceinline__ void st(int i, C<T> v) const {
         if (live) p[i * stride] = v;
     }
 };
@@ -232,14 +232,14 @@ struct FastOutAll {
 // (the level's lines for this pass) and NT threads; the same work list and
 // layout as k_col (MODE 0 yf, 1 z with the table, 2 yi, 3 z with the table
 // times -i D_comp of spectral-gradient component comp).
-template <class P, int AX, int MODE, int TX, int NT>
+template <class P, int AX, int MODE, int TX, int NT, typename T>
 __global__ void __launch_bounds__(NT) k_col_fast(const GridDev* __restrict__ grids, const Chunk* __restrict__ chunks,
-                                                 const float2* __restrict__ tw_arena, const float* __restrict__ tab,
-                                                 float2* __restrict__ wsA, float2* __restrict__ wsB, int comp) {
+                                                 const C<T>* __restrict__ tw_arena, const T* __restrict__ tab,
+                                                 C<T>* __restrict__ wsA, C<T>* __restrict__ wsB, int comp) {
     constexpr int L = P::L;
     extern __shared__ __align__(16) unsigned char smem_fast[];
-    float2* buf = reinterpret_cast<float2*>(smem_fast);
-    float2* tw = buf + L * TX;
+    C<T>* buf = reinterpret_cast<C<T>*>(smem_fast);
+    C<T>* tw = buf + L * TX;
     const Chunk ch = chunks[blockIdx.x];
     const GridDev& g = grids[ch.grid];
     const int Hx = g.Hx;
@@ -254,8 +254,8 @@ __global__ void __launch_bounds__(NT) k_col_fast(const GridDev* __restrict__ gri
     static_assert(NT % TX == 0, "NT must be a multiple of TX");
     const int line = threadIdx.x % TX;
     const bool live = kx0 + line < Hx;
-    FastIn gin;
-    FastOut<L> gout;
+    FastIn<T> gin;
+    FastOut<T, L> gout;
     gin.live = gout.live = live;
     if (AX == 1 && MODE == 0) {
         gin.p = wsA + (g.wsA + (long long)other * g.G[1] * Hx + kx0 + line);
@@ -277,29 +277,29 @@ __global__ void __launch_bounds__(NT) k_col_fast(const GridDev* __restrict__ gri
 
     if constexpr (MODE == 0) {
         // the y forward writes all M1 outputs: no window test
-        const FastOutAll gall{gout.p, gout.stride, live};
+        const FastOutAll<T> gall{gout.p, gout.stride, live};
         if constexpr (P::NST == 2) {
-            fast_dif_stage<P, 0, TX, NT, true, false>(buf, tw, gin, gall);
+            fast_dif_stage<T, P, 0, TX, NT, true, false>(buf, tw, gin, gall);
             __syncthreads();
-            fast_dif_stage<P, 1, TX, NT, false, true>(buf, tw, gin, gall);
+            fast_dif_stage<T, P, 1, TX, NT, false, true>(buf, tw, gin, gall);
         } else {
-            fast_dif_stage<P, 0, TX, NT, true, false>(buf, tw, gin, gall);
+            fast_dif_stage<T, P, 0, TX, NT, true, false>(buf, tw, gin, gall);
             __syncthreads();
-            fast_dif_stage<P, 1, TX, NT, false, false>(buf, tw, gin, gall);
+            fast_dif_stage<T, P, 1, TX, NT, false, false>(buf, tw, gin, gall);
             __syncthreads();
-            fast_dif_stage<P, 2, TX, NT, false, true>(buf, tw, gin, gall);
+            fast_dif_stage<T, P, 2, TX, NT, false, true>(buf, tw, gin, gall);
         }
     } else if constexpr (MODE == 2) {
         if constexpr (P::NST == 2) {
-            fast_dit_stage<P, 1, TX, NT, true, false>(buf, tw, gin, gout);
+            fast_dit_stage<T, P, 1, TX, NT, true, false>(buf, tw, gin, gout);
             __syncthreads();
-            fast_dit_stage<P, 0, TX, NT, false, true>(buf, tw, gin, gout);
+            fast_dit_stage<T, P, 0, TX, NT, false, true>(buf, tw, gin, gout);
         } else {
-            fast_dit_stage<P, 2, TX, NT, true, false>(buf, tw, gin, gout);
+            fast_dit_stage<T, P, 2, TX, NT, true, false>(buf, tw, gin, gout);
             __syncthreads();
-            fast_dit_stage<P, 1, TX, NT, false, false>(buf, tw, gin, gout);
+            fast_dit_stage<T, P, 1, TX, NT, false, false>(buf, tw, gin, gout);
             __syncthreads();
-            fast_dit_stage<P, 0, TX, NT, false, true>(buf, tw, gin, gout);
+            fast_dit_stage<T, P, 0, TX, NT, false, true>(buf, tw, gin, gout);
         }
     } else {
         // phi-hat = T(kappa) rho-hat between the forward and the inverse
@@ -307,37 +307,37 @@ __global__ void __launch_bounds__(NT) k_col_fast(const GridDev* __restrict__ gri
         // -i D_comp T(kappa) rho-hat
         const int ky = other;
         const int fy = ky <= M1 / 2 ? ky : M1 - ky;
-        TabCol<float> tabc;   // a dead line reads column 0 (its results are never stored)
+        TabCol<T> tabc;   // a dead line reads column 0 (its results are never stored)
         tabc.p = tab + (g.tab_off + (long long)fy * Hx + (live ? kx0 + line : 0));
         tabc.zst = g.Hy2 * Hx;
         tabc.L = L;
-        using Tab = typename std::conditional<MODE == 3, TabGrad<float>, TabCol<float>>::type;
+        using Tab = typename std::conditional<MODE == 3, TabGrad<T>, TabCol<T>>::type;
         Tab tabf;
         if constexpr (MODE == 3) {
             const int kx = kx0 + line;
             tabf.tab = tabc;
             tabf.comp = comp;
-            tabf.dz = (float)g.dk[2];
+            tabf.dz = (T)g.dk[2];
             const int M0 = g.M[0];
             const int kyc = ky <= M1 / 2 ? ky : ky - M1;
-            tabf.dline = comp == 1 ? (2 * kx == M0 ? 0.f : (float)(g.dk[0] * kx))
-                                   : (comp == 2 ? (2 * ky == M1 ? 0.f : (float)(g.dk[1] * kyc)) : 0.f);
+            tabf.dline = comp == 1 ? (2 * kx == M0 ? T(0) : (T)(g.dk[0] * kx))
+                                   : (comp == 2 ? (2 * ky == M1 ? T(0) : (T)(g.dk[1] * kyc)) : T(0));
         } else {
             tabf = tabc;
         }
-        fast_dif_stage<P, 0, TX, NT, true, false>(buf, tw, gin, gout);
+        fast_dif_stage<T, P, 0, TX, NT, true, false>(buf, tw, gin, gout);
         __syncthreads();
         if constexpr (P::NST == 3) {
-            fast_dif_stage<P, 1, TX, NT, false, false>(buf, tw, gin, gout);
+            fast_dif_stage<T, P, 1, TX, NT, false, false>(buf, tw, gin, gout);
             __syncthreads();
         }
-        fast_mid_stage<P, TX, NT>(buf, tabf);
+        fast_mid_stage<T, P, TX, NT>(buf, tabf);
         __syncthreads();
         if constexpr (P::NST == 3) {
-            fast_dit_stage<P, 1, TX, NT, false, false>(buf, tw, gin, gout);
+            fast_dit_stage<T, P, 1, TX, NT, false, false>(buf, tw, gin, gout);
             __syncthreads();
         }
-        fast_dit_stage<P, 0, TX, NT, false, true>(buf, tw, gin, gout);
+        fast_dit_stage<T, P, 0, TX, NT, false, true>(buf, tw, gin, gout);
     }
 }
 
@@ -345,9 +345,9 @@ __global__ void __launch_bounds__(NT) k_col_fast(const GridDev* __restrict__ gri
 // A CTA holds NP complex lines, each packing two real rows (2p, 2p+1) of the
 // grid (two-for-one real transforms); buffer element (position, line) at
 // pos (NP + 1) + line (the padding keeps the row-wise passes conflict-free).
-struct NoIO {
-    __device__ float2 ld(int) const { return make_float2(0.f, 0.f); }
-    __device__ void st(int, float2) const {}
+template <typename T> struct NoIO {
+    __device__ C<T> ld(int) const { return mk<T>(0, 0); }
+    __device__ void st(int, C<T>) const {}
 };
 
 // xf: GMF rows -> half spectra along x, A[z][y][kx] (the layout of k_xf).
@@ -357,15 +357,15 @@ struct NoIO {
 // positions past G0 and missing rows are zero.  Then the forward stages in place, and the separation of the
 // two real rows, A_k = (Z_k + conj Z_{L-k}) / 2, B_k = (Z_k - conj Z_{L-k}) / 2i,
 // written with consecutive threads on consecutive kx.
-template <class P, int NP, int NT>
+template <class P, int NP, int NT, typename T>
 __global__ void __launch_bounds__(NT) k_xf_fast(const GridDev* __restrict__ grids, const Chunk* __restrict__ chunks,
                                                 const int64_t* const* __restrict__ gmf,
-                                                const float2* __restrict__ tw_arena, float2* __restrict__ wsA,
+                                                const C<T>* __restrict__ tw_arena, C<T>* __restrict__ wsA,
                                                 int F) {
     constexpr int L = P::L, PITCH = NP + 1, H = L / 2 + 1;
     extern __shared__ __align__(16) unsigned char smem_fast[];
-    float2* buf = reinterpret_cast<float2*>(smem_fast);
-    float2* tw = buf + L * PITCH;
+    C<T>* buf = reinterpret_cast<C<T>*>(smem_fast);
+    C<T>* tw = buf + L * PITCH;
     const Chunk ch = chunks[blockIdx.x];
     const GridDev& g = grids[ch.grid];
     const int G0 = g.G[0];
@@ -373,7 +373,7 @@ __global__ void __launch_bounds__(NT) k_xf_fast(const GridDev* __restrict__ grid
     const int nr = (int)min(2LL * NP, (long long)g.G[1] * g.G[2] - r_first);
     const int64_t* __restrict__ in = gmf[ch.grid] + r_first * G0;
     for (int t = threadIdx.x; t < L; t += NT) tw[t] = tw_arena[g.fx.tw_off + t];
-    const float scale = pow2_neg<float>(F);
+    const T scale = pow2_neg<T>(F);
     // element (x, line p) = (row 2p, row 2p + 1) at x; one thread per pair of
     // positions of a line, with 16-byte loads of both rows when G0 is even
     {
@@ -407,31 +407,31 @@ __global__ void __launch_bounds__(NT) k_xf_fast(const GridDev* __restrict__ grid
                     if (x1) b1 = r0[G0 + 1];
                 }
             }
-            buf[x * PITCH + p] = make_float2(fixed_to_real<float>(a0, scale), fixed_to_real<float>(b0, scale));
+            buf[x * PITCH + p] = mk<T>(fixed_to_real<T>(a0, scale), fixed_to_real<T>(b0, scale));
             if (L % 2 == 0 || x + 1 < L)
                 buf[(x + 1) * PITCH + p] =
-                    make_float2(fixed_to_real<float>(a1, scale), fixed_to_real<float>(b1, scale));
+                    mk<T>(fixed_to_real<T>(a1, scale), fixed_to_real<T>(b1, scale));
         }
     }
     __syncthreads();
-    const NoIO none;
-    fast_dif_stage<P, 0, NP, NT, false, false, NoIO, NoIO, PITCH>(buf, tw, none, none);
+    const NoIO<T> none;
+    fast_dif_stage<T, P, 0, NP, NT, false, false, NoIO<T>, NoIO<T>, PITCH>(buf, tw, none, none);
     __syncthreads();
-    fast_dif_stage<P, 1, NP, NT, false, false, NoIO, NoIO, PITCH>(buf, tw, none, none);
+    fast_dif_stage<T, P, 1, NP, NT, false, false, NoIO<T>, NoIO<T>, PITCH>(buf, tw, none, none);
     __syncthreads();
     if constexpr (P::NST == 3) {
-        fast_dif_stage<P, 2, NP, NT, false, false, NoIO, NoIO, PITCH>(buf, tw, none, none);
+        fast_dif_stage<T, P, 2, NP, NT, false, false, NoIO<T>, NoIO<T>, PITCH>(buf, tw, none, none);
         __syncthreads();
     }
-    float2* __restrict__ out = wsA + (g.wsA + r_first * H);
+    C<T>* __restrict__ out = wsA + (g.wsA + r_first * H);
     for (int f = threadIdx.x; f < NP * H; f += NT) {
         const int p = f / H, k = f - p * H;
         const int q0 = 2 * p;
         if (q0 >= nr) continue;
-        const float2 z = buf[P::position(k) * PITCH + p];
-        const float2 zm = buf[P::position(k == 0 ? 0 : L - k) * PITCH + p];
-        out[q0 * H + k] = make_float2(0.5f * (z.x + zm.x), 0.5f * (z.y - zm.y));
-        if (q0 + 1 < nr) out[(q0 + 1) * H + k] = make_float2(0.5f * (z.y + zm.y), 0.5f * (zm.x - z.x));
+        const C<T> z = buf[P::position(k) * PITCH + p];
+        const C<T> zm = buf[P::position(k == 0 ? 0 : L - k) * PITCH + p];
+        out[q0 * H + k] = mk<T>(T(0.5) * (z.x + zm.x), T(0.5) * (z.y - zm.y));
+        if (q0 + 1 < nr) out[(q0 + 1) * H + k] = mk<T>(T(0.5) * (z.y + zm.y), T(0.5) * (zm.x - z.x));
     }
 }
 
@@ -449,8 +449,8 @@ template <class P, int PITCH>
 __device__ __forceinline__ int rows_index(int e) {
     return e * PITCH + e / P::radix(P::NST - 1);
 }
-template <class P, int S_, int NL, int NT, bool IN_G, bool OUT_G, int DIR, int PITCH, class GIN, class GOUT>
-__device__ __forceinline__ void fast_dif_stage_rows(float2* buf, const float2* __restrict__ tw, const GIN& gin,
+template <typename T, class P, int S_, int NL, int NT, bool IN_G, bool OUT_G, int DIR, int PITCH, class GIN, class GOUT>
+__device__ __forceinline__ void fast_dif_stage_rows(C<T>* buf, const C<T>* __restrict__ tw, const GIN& gin,
                                                     const GOUT& gout) {
     constexpr int R = P::radix(S_), S = P::inner(S_), L = P::L;
     constexpr int NB = L / R, ITEMS = NB * NL, TRIPS = (ITEMS + NT - 1) / NT;
@@ -462,16 +462,16 @@ __device__ __forceinline__ void fast_dif_stage_rows(float2* buf, const float2* _
         const int line = i / NB, b = i - line * NB;
         const int hi = b / S, lo = b - hi * S;
         const int base = hi * R * S + lo;
-        float2 v[R];
+        C<T> v[R];
 #pragma unroll
         for (int k = 0; k < R; ++k) {
             if constexpr (IN_G) v[k] = gin.ld(line, base + k * S);
             else v[k] = buf[rows_index<P, PITCH>(base + k * S) + line];
         }
-        FastDft<DIR, R>::run(v);
+        FastDft<T, DIR, R>::run(v);
         if constexpr (S > 1) {
 #pragma unroll
-            for (int k = 1; k < R; ++k) v[k] = mul<float>(v[k], twid<float, DIR>(tw, lo * k * TWS));
+            for (int k = 1; k < R; ++k) v[k] = mul<T>(v[k], twid<T, DIR>(tw, lo * k * TWS));
         }
         static_assert(!OUT_G || S == 1, "global output only from the last stage");
         const int nat0 = OUT_G ? P::natural(base) : 0;
@@ -491,29 +491,29 @@ __device__ __forceinline__ void fast_dif_stage_rows(float2* buf, const float2* _
 // real part to row 2p, imaginary part to row 2p+1, at window cell
 // w = (x - s0) mod L (and w + L when inside the window), times 1/(M0 M1 M2);
 // with a two-stage plan its neighbouring butterflies write neighbouring x.
-template <int L> struct XiRowsIn {
-    const float2* __restrict__ p;    // row 0 of this CTA
+template <typename T, int L> struct XiRowsIn {
+    const C<T>* __restrict__ p;    // row 0 of this CTA
     int nr;                          // rows of this CTA
-    __device__ __forceinline__ float2 ld(int line, int k) const {
+    __device__ __forceinline__ C<T> ld(int line, int k) const {
         constexpr int H = L / 2 + 1;
         const int kk = k < H ? k : L - k;
-        const float2* row = p + (2 * line) * H;
-        float2 a = make_float2(0.f, 0.f), b = make_float2(0.f, 0.f);
+        const C<T>* row = p + (2 * line) * H;
+        C<T> a = mk<T>(T(0), T(0)), b = mk<T>(T(0), T(0));
         if (2 * line < nr) a = row[kk];
         if (2 * line + 1 < nr) b = row[H + kk];
         if (k >= H) {
             a.y = -a.y;
             b.y = -b.y;
         }
-        return make_float2(a.x - b.y, a.y + b.x);
+        return mk<T>(a.x - b.y, a.y + b.x);
     }
 };
-template <int L> struct XiRowsOut {
-    float* __restrict__ p;           // row 0 of this CTA in the window
+template <typename T, int L> struct XiRowsOut {
+    T* __restrict__ p;           // row 0 of this CTA in the window
     int W0, s0, nr;
-    float norm;
-    __device__ __forceinline__ void st(int line, int x, float2 v) const {
-        float* row = p + (2 * line) * W0;
+    T norm;
+    __device__ __forceinline__ void st(int line, int x, C<T> v) const {
+        T* row = p + (2 * line) * W0;
         int w = x - s0;
         if (w < 0) w += L;
         for (; w < W0; w += L) {
@@ -523,42 +523,42 @@ template <int L> struct XiRowsOut {
     }
 };
 
-template <class P, int NP, int NT>
+template <class P, int NP, int NT, typename T>
 __global__ void __launch_bounds__(NT) k_xi_fast(const GridDev* __restrict__ grids, const Chunk* __restrict__ chunks,
-                                                const float2* __restrict__ tw_arena,
-                                                const float2* __restrict__ wsB, void* const* __restrict__ phis,
+                                                const C<T>* __restrict__ tw_arena,
+                                                const C<T>* __restrict__ wsB, void* const* __restrict__ phis,
                                                 int comp) {
     constexpr int L = P::L, H = L / 2 + 1, PITCH = NP + 1;
     extern __shared__ __align__(16) unsigned char smem_fast[];
-    float2* buf = reinterpret_cast<float2*>(smem_fast);
-    float2* tw = buf + rows_index<P, PITCH>(L);   // past the padded line buffer (<= L PITCH + L / 2)
+    C<T>* buf = reinterpret_cast<C<T>*>(smem_fast);
+    C<T>* tw = buf + rows_index<P, PITCH>(L);   // past the padded line buffer (<= L PITCH + L / 2)
     const Chunk ch = chunks[blockIdx.x];
     const GridDev& g = grids[ch.grid];
     const int W0 = g.W[0];
     const long long r_first = 2LL * ch.tile * NP;
     const int nr = (int)min(2LL * NP, (long long)g.W[1] * g.W[2] - r_first);
     for (int t = threadIdx.x; t < L; t += NT) tw[t] = tw_arena[g.fx.tw_off + t];
-    XiRowsIn<L> gin;
+    XiRowsIn<T, L> gin;
     gin.p = wsB + (g.wsB + r_first * H);
     gin.nr = nr;
-    XiRowsOut<L> gout;
+    XiRowsOut<T, L> gout;
     // component comp of a spectral-gradient solve: the comp-th window of W cells
-    gout.p = reinterpret_cast<float*>(phis[ch.grid]) + (long long)comp * g.W[0] * g.W[1] * g.W[2] + r_first * W0;
+    gout.p = reinterpret_cast<T*>(phis[ch.grid]) + (long long)comp * g.W[0] * g.W[1] * g.W[2] + r_first * W0;
     gout.W0 = W0;
     gout.s0 = g.s0[0];
     gout.nr = nr;
-    gout.norm = (float)g.inv_m3;
+    gout.norm = (T)g.inv_m3;
     __syncthreads();   // twiddles
-    using GI = XiRowsIn<L>;
-    using GO = XiRowsOut<L>;
-    fast_dif_stage_rows<P, 0, NP, NT, true, false, 1, PITCH, GI, GO>(buf, tw, gin, gout);
+    using GI = XiRowsIn<T, L>;
+    using GO = XiRowsOut<T, L>;
+    fast_dif_stage_rows<T, P, 0, NP, NT, true, false, 1, PITCH, GI, GO>(buf, tw, gin, gout);
     __syncthreads();
     if constexpr (P::NST == 3) {
-        fast_dif_stage_rows<P, 1, NP, NT, false, false, 1, PITCH, GI, GO>(buf, tw, gin, gout);
+        fast_dif_stage_rows<T, P, 1, NP, NT, false, false, 1, PITCH, GI, GO>(buf, tw, gin, gout);
         __syncthreads();
-        fast_dif_stage_rows<P, 2, NP, NT, false, true, 1, PITCH, GI, GO>(buf, tw, gin, gout);
+        fast_dif_stage_rows<T, P, 2, NP, NT, false, true, 1, PITCH, GI, GO>(buf, tw, gin, gout);
     } else {
-        fast_dif_stage_rows<P, 1, NP, NT, false, true, 1, PITCH, GI, GO>(buf, tw, gin, gout);
+        fast_dif_stage_rows<T, P, 1, NP, NT, false, true, 1, PITCH, GI, GO>(buf, tw, gin, gout);
     }
 }
 
@@ -651,7 +651,7 @@ __device__ __forceinline__ void xy_x_stage(float2* buf, const float2* __restrict
             if constexpr (IN_G) v[k] = gin.ld(line, base + k * S);
             else v[k] = lb[base + k * S];
         }
-        FastDft<-1, R>::run(v);
+        FastDft<float, -1, R>::run(v);
         if constexpr (S > 1) {
 #pragma unroll
             for (int k = 1; k < R; ++k) v[k] = mul<float>(v[k], tw[lo * k * TWS]);
@@ -678,7 +678,7 @@ __device__ __forceinline__ void xy_y_stage(float2* buf, const float2* __restrict
         float2 v[R];
 #pragma unroll
         for (int k = 0; k < R; ++k) v[k] = buf[(base + k * S) * H + col];
-        FastDft<-1, R>::run(v);
+        FastDft<float, -1, R>::run(v);
         if constexpr (S > 1) {
 #pragma unroll
             for (int k = 1; k < R; ++k) v[k] = mul<float>(v[k], tw[lo * k * TWS]);
@@ -712,7 +712,7 @@ __global__ void __launch_bounds__(NT, 2) k_xy_fast(const GridDev* __restrict__ g
     for (int t = threadIdx.x + 2 * nl * H; t < L * H; t += NT) buf[t] = make_float2(0.f, 0.f);
     xy_load_plane<L, NT, 2 * H>(buf, gmf[ch.grid] + (long long)z * G1 * G0, G0, G1, nl, pow2_neg<float>(F));
     __syncthreads();   // twiddles and the x lines
-    const NoIO none;
+    const NoIO<float> none;
     xy_x_stage<P, 0, NT, false, 2 * H>(buf, tw, none, nl);
     __syncthreads();
     xy_x_stage<P, 1, NT, false, 2 * H>(buf, tw, none, nl);
@@ -805,7 +805,7 @@ __device__ __forceinline__ void yx_y_stage(float2* buf, const float2* __restrict
             if constexpr (IN_G) v[k] = gin.ld(col, base + k * S);
             else v[k] = buf[(base + k * S) * H + col];
         }
-        FastDft<DIR, R>::run(v);
+        FastDft<float, DIR, R>::run(v);
         if constexpr (S > 1) {
 #pragma unroll
             for (int k = 1; k < R; ++k) v[k] = mul<float>(v[k], twid<float, DIR>(tw, lo * k * TWS));
@@ -849,7 +849,7 @@ __device__ __forceinline__ void yx_x_stage(float2* buf, const float2* __restrict
             const int e = base + k * S;
             v[k] = e < H ? buf[ra * H + e] : buf[rb * H + e - H];
         }
-        FastDft<1, R>::run(v);
+        FastDft<float, 1, R>::run(v);
         if constexpr (S > 1) {
 #pragma unroll
             for (int k = 1; k < R; ++k) v[k] = mul<float>(v[k], twid<float, 1>(tw, lo * k * TWS));

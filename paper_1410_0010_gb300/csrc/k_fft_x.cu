@@ -13,15 +13,39 @@ cudaError_t fft_configure_z_f64();
 cudaError_t fft_configure_yi_f64();
 cudaError_t fft_configure_zg_f32();
 cudaError_t fft_configure_zg_f64();
-// the FP32 passes with compile-time plans (k_fft_fast.cu)
-cudaError_t fft_configure_fast_yf();
-cudaError_t fft_configure_fast_z();
-cudaError_t fft_configure_fast_yi();
-cudaError_t fft_configure_fast_xf();
-cudaError_t fft_configure_fast_xi();
-cudaError_t fft_configure_fast_zg();
+// the passes with compile-time plans (k_fft_fast.cu, one unit per kernel,
+// precision and group of lengths)
+#define APM_FAST_DECL(m, p, g) \
+    cudaError_t fast_launch##m##_##p##_##g(int L, const FftArgs& a, const int64_t* const* gmf, void* const* phis, \
+                                           cudaStream_t s); \
+    cudaError_t fast_configure##m##_##p##_##g(int L);
+#define APM_FAST_F32(X, m) X(m, 0, 0) X(m, 0, 1) X(m, 0, 2) X(m, 0, 3)
+#define APM_FAST_F64(X, m) X(m, 1, 1) X(m, 1, 2) X(m, 1, 3)
+#define APM_FAST_UNITS(X) \
+    APM_FAST_F32(X, 0) APM_FAST_F32(X, 1) APM_FAST_F32(X, 2) APM_FAST_F32(X, 3) APM_FAST_F32(X, 4) \
+    APM_FAST_F32(X, 5) APM_FAST_F32(X, 6) APM_FAST_F32(X, 7) APM_FAST_F64(X, 0) APM_FAST_F64(X, 1) \
+    APM_FAST_F64(X, 2) APM_FAST_F64(X, 3) APM_FAST_F64(X, 4) APM_FAST_F64(X, 5)
+APM_FAST_UNITS(APM_FAST_DECL)
 
-// Allows every pass kernel up to kFftSmemLimit of dynamic shared memory
+cudaError_t launch_fft_fast(int kernel, bool f64, int L, const FftArgs& a, const int64_t* const* gmf,
+                            void* const* phis, cudaStream_t s) {
+    const int u = (kernel * 2 + (f64 ? 1 : 0)) * kFastGroups + fast_group(L, f64);
+#define APM_FAST_CASE(m, p, g) \
+    case (m * 2 + p) * kFastGroups + g: return fast_launch##m##_##p##_##g(L, a, gmf, phis, s);
+    if (fast_length(L, f64)) switch (u) { APM_FAST_UNITS(APM_FAST_CASE) }
+#undef APM_FAST_CASE
+    return cudaErrorInvalidValue;
+}
+cudaError_t configure_fft_fast(int kernel, bool f64, int L) {
+    const int u = (kernel * 2 + (f64 ? 1 : 0)) * kFastGroups + fast_group(L, f64);
+#define APM_FAST_CASE(m, p, g) \
+    case (m * 2 + p) * kFastGroups + g: return fast_configure##m##_##p##_##g(L);
+    if (fast_length(L, f64)) switch (u) { APM_FAST_UNITS(APM_FAST_CASE) }
+#undef APM_FAST_CASE
+    return cudaErrorInvalidValue;
+}
+
+// Allows every runtime-planned pass kernel up to kFftSmemLimit of dynamic shared memory
 // (above the 48 KB default).
 cudaError_t fft_configure() {
     const void* fns[] = {(const void*)k_xf<float, 128>, (const void*)k_xf<float, 256>,
@@ -34,9 +58,7 @@ cudaError_t fft_configure() {
     }
     cudaError_t (*cols[])() = {fft_configure_yf_f32, fft_configure_z_f32, fft_configure_yi_f32,
                                fft_configure_zg_f32, fft_configure_yf_f64, fft_configure_z_f64,
-                               fft_configure_yi_f64, fft_configure_zg_f64, fft_configure_fast_yf,
-                               fft_configure_fast_z, fft_configure_fast_yi, fft_configure_fast_xf,
-                               fft_configure_fast_xi, fft_configure_fast_zg};
+                               fft_configure_yi_f64, fft_configure_zg_f64};
     for (auto f : cols) {
         cudaError_t e = f();
         if (e != cudaSuccess) return e;
