@@ -387,15 +387,48 @@ __device__ __forceinline__ void load_twiddles(C<T>* dst, const C<T>* __restrict_
 }
 
 // Correctly rounded conversion of a fixed-point cell mass q * 2^-F to T:
-// q rounded to nearest-even in T (the hardware int64 conversion), then scaled
-// by scale = 2^-F, which is exact.  For T = float this equals the FP64
-// conversion (double)q * 2^-F rounded to float whenever |q| < 2^53.
+// q rounded to nearest-even in T, then scaled by scale = 2^-F, which is exact.
+// For T = float this equals the FP64 conversion (double)q * 2^-F rounded to
+// float whenever |q| < 2^53.
+// The 64-bit conversion instructions run at 2 lanes per clock and SM on this
+// chip (the FP64 rate, measured; the 32-bit ones at 32).  For
+// -2^47 <= q < 2^47 the FP32 path splits q = h 2^23 + l with h in
+// [-2^24, 2^24) and 0 <= l < 2^23, both exact in FP32, so h 2^23 + l is rounded
+// once, by the FMA: the same bits as __ll2float_rn.  Larger values (a cell of
+// 1/32 of the unit mass or more with the default 52 fraction bits) take the
+// instruction.
 template <typename T> __device__ __forceinline__ T fixed_to_real(long long q, T scale);
 template <> __device__ __forceinline__ double fixed_to_real<double>(long long q, double scale) {
     return __ll2double_rn(q) * scale;
 }
+// -2^47 <= q < 2^47
+__device__ __forceinline__ bool fits48(long long q) { return (unsigned)((int)(q >> 32) + 0x8000) < 0x10000u; }
+__device__ __forceinline__ float fixed48_to_float(long long q) {
+    const int h = (int)(q >> 23);
+    const float l = __uint_as_float(0x4b000000u | ((unsigned)q & 0x7fffffu)) - 8388608.0f;
+    return __fmaf_rn((float)h, 8388608.0f, l);
+}
 template <> __device__ __forceinline__ float fixed_to_real<float>(long long q, float scale) {
-    return __ll2float_rn(q) * scale;
+    return (fits48(q) ? fixed48_to_float(q) : __ll2float_rn(q)) * scale;
+}
+// two complex values (a + i b), (c + i d) at once, with one test for the four
+// (the load passes convert two cells of two rows per thread)
+template <typename T>
+__device__ __forceinline__ void fixed4_to_real(long long a, long long b, long long c, long long d, T scale, C<T>& u,
+                                               C<T>& v) {
+    u = mk<T>(fixed_to_real<T>(a, scale), fixed_to_real<T>(b, scale));
+    v = mk<T>(fixed_to_real<T>(c, scale), fixed_to_real<T>(d, scale));
+}
+template <>
+__device__ __forceinline__ void fixed4_to_real<float>(long long a, long long b, long long c, long long d, float scale,
+                                                      float2& u, float2& v) {
+    if (fits48(a) && fits48(b) && fits48(c) && fits48(d)) {
+        u = make_float2(fixed48_to_float(a) * scale, fixed48_to_float(b) * scale);
+        v = make_float2(fixed48_to_float(c) * scale, fixed48_to_float(d) * scale);
+    } else {
+        u = make_float2(__ll2float_rn(a) * scale, __ll2float_rn(b) * scale);
+        v = make_float2(__ll2float_rn(c) * scale, __ll2float_rn(d) * scale);
+    }
 }
 
 // 2^-F in T, 1 <= F <= 62

@@ -407,10 +407,10 @@ __global__ void __launch_bounds__(NT) k_xf_fast(const GridDev* __restrict__ grid
                     if (x1) b1 = r0[G0 + 1];
                 }
             }
-            buf[x * PITCH + p] = mk<T>(fixed_to_real<T>(a0, scale), fixed_to_real<T>(b0, scale));
-            if (L % 2 == 0 || x + 1 < L)
-                buf[(x + 1) * PITCH + p] =
-                    mk<T>(fixed_to_real<T>(a1, scale), fixed_to_real<T>(b1, scale));
+            C<T> u, v;
+            fixed4_to_real<T>(a0, b0, a1, b1, scale, u, v);
+            buf[x * PITCH + p] = u;
+            if (L % 2 == 0 || x + 1 < L) buf[(x + 1) * PITCH + p] = v;
         }
     }
     __syncthreads();
@@ -591,9 +591,12 @@ __device__ __forceinline__ void xy_load_plane(float2* buf, const int64_t* __rest
     const int half = (G0 + 1) / 2;   // position pairs per row
     const bool vec = !(G0 & 1) && !(reinterpret_cast<size_t>(in) & 15);
     const int items = nl * half;
+    // item i is pair i % half of line i / half, stepped without a division
+    int p = threadIdx.x / half, xp = threadIdx.x - p * half;
+    const int dp = NT / half, dx = NT - dp * half;
 #pragma unroll 4
     for (int i = threadIdx.x; i < items; i += NT) {
-        const int p = i / half, x = 2 * (i - p * half);
+        const int x = 2 * xp;
         const bool odd_row = 2 * p + 1 < G1;
         const int64_t* r0 = in + (long long)(2 * p) * G0 + x;
         long long a0, a1, b0 = 0, b1 = 0;
@@ -615,15 +618,18 @@ __device__ __forceinline__ void xy_load_plane(float2* buf, const int64_t* __rest
                 b1 = x1 ? r0[G0 + 1] : 0;
             }
         }
-        *reinterpret_cast<float4*>(buf + p * LS + x) =
-            make_float4(fixed_to_real<float>(a0, scale), fixed_to_real<float>(b0, scale),
-                        fixed_to_real<float>(a1, scale), fixed_to_real<float>(b1, scale));
+        float2 u, v;
+        fixed4_to_real<float>(a0, b0, a1, b1, scale, u, v);
+        *reinterpret_cast<float4*>(buf + p * LS + x) = make_float4(u.x, u.y, v.x, v.y);
+        xp += dx;
+        p += dp;
+        if (xp >= half) {
+            xp -= half;
+            ++p;
+        }
     }
-    const int pad = L - 2 * half;
-    for (int t = threadIdx.x; t < nl * pad; t += NT) {
-        const int p = t / pad;
-        buf[p * LS + 2 * half + (t - p * pad)] = make_float2(0.f, 0.f);
-    }
+    for (int q = threadIdx.x >> 5; q < nl; q += NT / 32)
+        for (int t = 2 * half + (threadIdx.x & 31); t < L; t += 32) buf[q * LS + t] = make_float2(0.f, 0.f);
 }
 template <int L> struct XyOut {
     float2* __restrict__ p;          // B row ky = 0 of this plane, column 0
