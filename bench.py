@@ -498,7 +498,7 @@ def run_apm(args):
                    mass_frac_bits=w.mass_frac_bits, device=local, gradient=gradient)
         if use_order if order is None else order:   # the particle processing order, recomputed every step
             s.reserve_order(w.n_particles)
-            s.set_deposit_tiles(use_tiles)          # ... and the deposit through shared-memory tiles
+            s.set_deposit_tiles(use_tiles)          # ... and the deposit visits them in bin order
         return s, s.alloc_all()
 
     host = {k: torch.from_numpy(np.ascontiguousarray(v)).pin_memory() for k, v in w.particles.items()}
@@ -872,7 +872,7 @@ def main():
     ap.add_argument("--order", choices=["auto", "on", "off", "tiles"], default="auto",
                     help="sort the particles by root-level bin every step before the particle kernels "
                          "(apm_order_particles; results are bit-identical either way); tiles: also deposit "
-                         "through shared-memory tiles (apm_set_deposit_tiles); auto: off when the workload "
+                         "in bin order (apm_set_deposit_tiles); auto: off when the workload "
                          "stores its particles in spatial order (the Zel'dovich lattice), otherwise the fastest "
                          "of five eager steps each way")
     ap.add_argument("--no-per-grid", action="store_true",

@@ -642,14 +642,10 @@ Particles to_dev(const apm_particles* p) {
 
 // the interpolation calls visit the particles in the current order when it
 // was computed for this many particles (any order gives the same results);
-// so do the deposits with apm_set_deposit_tiles(1), which then gather each
-// CTA's charges of its bin in shared memory (k_deposit<true>).  Without the
-// tiles the deposits keep the caller's order: in bin order neighbouring
-// threads reduce into the same cells and their L2 reductions serialise.
+// so do the deposits with apm_set_deposit_tiles(1), else they keep the caller's
 void use_order(const apm_ctx* c, Particles& P) {
     if (c->order.perm && c->order.n == P.n) {
         P.perm = c->order.perm;
-        P.order_shift = c->order.shift;
     }
 }
 
@@ -999,6 +995,9 @@ apm_status apm_set_hierarchy(apm_ctx* c, const apm_grid* grids, int32_t n) {
             const bool pow2 = std::frexp(D.delta0, &ex) == 0.5;
             D.pos_exp = kPosBits - (ex - 1);
             D.delta0_pow2 = (pow2 && D.pos_exp < 1000) ? 1 : 0;
+            unsigned long long bits;
+            std::memcpy(&bits, &D.delta0, sizeof(bits));
+            D.div_known = std::abs(ex) < 100 && (bits & 0xFFFFFFFFFFFFFULL) != 0xFFFFFFFFFFFFFULL ? 1 : 0;
         }
         D.frac_bits = kPosBits - L.level;
         D.span = (long long)N0 << kPosBits;

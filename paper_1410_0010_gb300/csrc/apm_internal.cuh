@@ -330,6 +330,7 @@ struct LevelDev {
     long long span;        // N0 2^31: the box in fixed-point units
     double box;
     int periodic;
+    int div_known;         // div_known() may divide by delta0 with inv_delta0
     int pos_exp;           // delta0 = 2^(31 - pos_exp) when delta0_pow2: X = rint(x 2^pos_exp)
     unsigned* status;      // the context's device status word (bounds-checked builds)
 };
@@ -342,25 +343,19 @@ constexpr int kPosBits = 31;
 constexpr unsigned long long kOne63 = 1ULL << 63;
 
 // rint(x 2^K), ties to even, of a finite double with |x 2^K| < 2^62, from its
-// exponent and significand with integer operations (no FP64 pipe); ok is
-// cleared for larger or non-finite values.
-__device__ __forceinline__ long long scaled_rint(double x, int K, bool& ok) {
+// exponent and significand with integer operations; kNoFixed for larger or
+// non-finite values.
+constexpr long long kNoFixed = (long long)(1ULL << 63);
+static __device__ __noinline__ long long scaled_rint_any(double x, int K) {
     const unsigned long long b = (unsigned long long)__double_as_longlong(x);
     const int e = (int)((b >> 52) & 0x7FF);
-    ok = true;
-    if (e == 0x7FF) {
-        ok = false;
-        return 0;
-    }
+    if (e == 0x7FF) return kNoFixed;
     if (e == 0) return 0;   // zero or subnormal: far below one unit here
     const unsigned long long m = (b & 0xFFFFFFFFFFFFFULL) | 0x10000000000000ULL;
     const int sh = e - 1075 + K;   // |x 2^K| = m 2^sh
     unsigned long long r;
     if (sh >= 0) {
-        if (sh >= 10) {            // m 2^sh >= 2^62
-            ok = false;
-            return 0;
-        }
+        if (sh >= 10) return kNoFixed;   // m 2^sh >= 2^62
         r = m << sh;
     } else if (sh < -54) {
         r = 0;
@@ -372,6 +367,40 @@ __device__ __forceinline__ long long scaled_rint(double x, int K, bool& ok) {
         if (rem > half || (rem == half && (r & 1))) ++r;
     }
     return (b >> 63) ? -(long long)r : (long long)r;
+}
+// The same, ok cleared in the place of kNoFixed (scaled_rint_small: and beyond
+// its range, |x 2^K| < 2^51).  For |x 2^K| < 2^51 (every coordinate and mass of an ordinary
+// problem) one FP64 addition rounds: x + 1.5 2^(52-K) lies where an FP64 unit in
+// the last place is 2^-K, so its significand holds rint(x 2^K), ties to even.
+// That is 16 clocks of the FP64 pipe for a warp, where the integer route takes
+// about 40 instructions.
+__device__ __forceinline__ long long scaled_rint_small(double x, int K, bool& ok) {
+    const int e = (__double2hiint(x) >> 20) & 0x7FF;   // |x| < 2^(e - 1022)
+    ok = e + K < 1073 && K > -900 && K < 1000;
+    const int chi = ((1023 + 52 - K) << 20) | 0x80000;
+    const double t = __dadd_rn(x, __hiloint2double(chi, 0));
+    return __double_as_longlong(t) - ((long long)chi << 32);
+}
+__device__ __forceinline__ long long scaled_rint(double x, int K, bool& ok) {
+    const long long v = scaled_rint_small(x, K, ok);
+    if (ok) return v;
+    const long long r = scaled_rint_any(x, K);
+    ok = r != kNoFixed;
+    return ok ? r : 0;
+}
+
+// RN(x / d) for a divisor known in advance: y = RN(1 / d), and two corrections
+// with exact FMA residuals.  The first makes the quotient faithful, the second
+// rounds it correctly (Markstein 1990; Cornea, Harrison and Tang 2002, for a
+// divisor whose significand is not all ones: checked on the host, as is the
+// range of d).  5 FP64 operations; x outside [2^-800, 2^800) takes the general
+// division, 0 included.
+__device__ __forceinline__ double div_known(double x, double d, double y, bool known) {
+    const unsigned e = (unsigned)((__double2hiint(x) >> 20) & 0x7FF);
+    if (!known || e - 223u >= 1600u) return __ddiv_rn(x, d);
+    double q = __dmul_rn(x, y);
+    q = __fma_rn(__fma_rn(-q, d, x), y, q);
+    return __fma_rn(__fma_rn(-q, d, x), y, q);
 }
 
 // x' = x + v half_dt in FP64 (two rounded operations)
@@ -390,9 +419,7 @@ __device__ __forceinline__ long long fixed_position(double xd, const LevelDev& L
     if (L.delta0_pow2) {
         X = scaled_rint(xd, L.pos_exp, ok);
     } else {
-        const double t = __dmul_rn(__ddiv_rn(xd, L.delta0), 2147483648.0);
-        ok = fabs(t) < 4611686018427387904.0;   // 2^62
-        X = ok ? __double2ll_rn(t) : 0;
+        X = scaled_rint(div_known(xd, L.delta0, L.inv_delta0, L.div_known != 0), 31, ok);
     }
     if (!ok) X = xd > 0.0 ? (1LL << 62) : -(1LL << 62);
     if (L.periodic) {
@@ -407,8 +434,8 @@ __device__ __forceinline__ long long fixed_position(double xd, const LevelDev& L
 }
 
 __device__ __forceinline__ long long tsc_fixed(long long X, int P, unsigned long long w[3]) {
-    long long i = X >> P;
-    unsigned f = (unsigned)(X - (i << P));
+    const long long i = X >> P;
+    const unsigned f = (unsigned)X & ((1u << P) - 1u);   // P <= 31
     unsigned S1 = (1u << P) - f;            // 2^P - f, at most 2^31
     const int up = 62 - 2 * P;
     w[2] = ((unsigned long long)f * f) << up;
@@ -478,12 +505,17 @@ __device__ __forceinline__ unsigned long long wmul63_small(unsigned long long a,
     const unsigned long long lo = (unsigned long long)a32 * (unsigned)b;
     return (hi + (lo >> 32) + (1ULL << 30)) >> 31;
 }
+// ... and its 32-bit result: a weight is at most 1, so the product is below 2^32
+__device__ __forceinline__ unsigned wmul63_32(unsigned a, unsigned long long b) {
+    const unsigned long long hi = (unsigned long long)a * (unsigned)(b >> 32) + (1ULL << 30);
+    return (unsigned)((hi + __umulhi(a, (unsigned)b)) >> 31);
+}
 
 struct Particles {
     long long n;
     const double *x, *y, *z, *vx, *vy, *vz, *m;
     const int* perm = nullptr;   // processing order (launch_order): slot i visits particle perm[i]
-    int order_shift = 0;         // ... sorted by bins of 2^order_shift root cells (x fastest)
+    unsigned stride = 0;         // the deposit's walk through its CTAs in that order (deposit_order)
     __device__ __forceinline__ long long at(long long i) const { return perm ? (long long)perm[i] : i; }
 };
 

@@ -228,8 +228,8 @@ class Solver:
 
     def set_deposit_tiles(self, on):
         """True: while a particle order is current, the deposits visit the
-        particles in it and gather each CTA's charges in shared-memory tiles
-        (bit-identical; pays where many particles share cells).  Default off."""
+        particles in it too (bit-identical; pays for particles in no spatial
+        order).  Default off."""
         check(lib().apm_set_deposit_tiles(self._ctx, 1 if on else 0), "apm_set_deposit_tiles")
 
     def fft_shapes(self, level):
