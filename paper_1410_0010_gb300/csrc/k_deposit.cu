@@ -32,16 +32,6 @@ __global__ void __launch_bounds__(256) k_gas_init(LevelDev L, const GridDev* __r
     const GridDev& g = L.g[c.grid];
     const int G0 = g.G[0], G1 = g.G[1];
     const int nrows = G1 * g.G[2];
-    const double scale = ldexp(1.0, F);
-    const double vol = __dmul_rn(__dmul_rn(g.delta, g.delta), g.delta);
-    // when delta is a power of two, 2^e, the two products are exact exponent
-    // shifts and rint((rho delta^3) 2^F) = rint(rho 2^(F + 3e)), which
-    // scaled_rint_small computes with one FP64 addition (the FP64 products remain
-    // for other cell sizes and for values beyond its range)
-    const unsigned long long db = (unsigned long long)__double_as_longlong(g.delta);
-    const int de = (int)((db >> 52) & 0x7FF);
-    const bool pow2 = (db & 0xFFFFFFFFFFFFFULL) == 0 && de > 0 && de < 0x7FF;
-    const int K = F + 3 * (de - 1023);
     const double* own = gas ? gas[c.grid] : nullptr;
     const double* par = (pgas && g.parent >= 0) ? pgas[g.parent] : nullptr;
     int64_t* __restrict__ out = gmf[c.grid];
@@ -53,6 +43,16 @@ __global__ void __launch_bounds__(256) k_gas_init(LevelDev L, const GridDev* __r
         zero_range(out + (long long)r0 * G0, (long long)(r1 - r0) * G0);
         return;
     }
+    const double scale = ldexp(1.0, F);
+    const double vol = __dmul_rn(__dmul_rn(g.delta, g.delta), g.delta);
+    // when delta is a power of two, 2^e, the two products are exact exponent
+    // shifts and rint((rho delta^3) 2^F) = rint(rho 2^(F + 3e)), which
+    // scaled_rint_small computes with one FP64 addition (the FP64 products remain
+    // for other cell sizes and for values beyond its range)
+    const unsigned long long db = (unsigned long long)__double_as_longlong(g.delta);
+    const int de = (int)((db >> 52) & 0x7FF);
+    const bool pow2 = (db & 0xFFFFFFFFFFFFFULL) == 0 && de > 0 && de < 0x7FF;
+    const int K = F + 3 * (de - 1023);
     int last = -1, cy = 0, cz = 0;
     bool yz_in = false;
     for (RowWalk it(r0, G0); it.r < r1; it.next()) {

@@ -372,6 +372,42 @@ __device__ __forceinline__ void interp_from(const LevelDev& L, const GridDev& g,
     for (int j = 0; j < 3; ++j)
         if (!APM_IN_BOUNDS(fold ? min(max(lc[j], 0), g.N[j] - 1) : lc[j], g.N[j], L.status)) return;
     T a0 = 0, a1 = 0, a2 = 0;
+    // the three cells of a row lie in two aligned pairs: 54 pair loads instead of
+    // 81 (the load/store unit is what bounds the kernel: 72% of its peak with
+    // single loads on the lattice).  Rows and components of even length from an
+    // aligned pointer start on a pair, so the pairs stay inside the row (its
+    // first cell has the parity of lc[0]); a cloud folded at an isolated root's
+    // faces is not contiguous.  The same bits; a Plummer sphere of 1 M 182 -> 155
+    // us in bin order and 236 -> 186 in its own, 16.8 M lattice particles 889 ->
+    // 875.  (The deposit's arrangement, 8 particles' rows a load, took 154 us
+    // for the sphere in its own order, but 1040 for the lattice, whose
+    // neighbouring lanes share sectors already.)
+    using V2 = typename Cplx<T>::type;
+    bool pairs = !(E0 & 1) && !(ncell & 1) && !(reinterpret_cast<size_t>(A) & (2 * sizeof(T) - 1));
+    for (int j = 0; j < 3; ++j) pairs = pairs && (!fold || (lc[j] > 0 && lc[j] < g.N[j] - 1));
+    if (pairs) {
+        const bool odd = lc[0] & 1;
+        const T* __restrict__ base = A + ((unsigned)(lc[0] & ~1) + (unsigned)E0 * ((unsigned)lc[1] + (unsigned)E1 * (unsigned)lc[2]));
+#pragma unroll
+        for (int c = 0; c < 3; ++c)
+#pragma unroll
+            for (int b = 0; b < 3; ++b) {
+                const unsigned row = (unsigned)E0 * ((unsigned)b + (unsigned)E1 * (unsigned)c);
+#pragma unroll
+                for (int j = 0; j < 3; ++j) {
+                    const V2* __restrict__ q = reinterpret_cast<const V2*>(base + (row + (unsigned)j * ncell));
+                    const V2 u = q[0], v = q[1];
+                    T& acc = j == 0 ? a0 : (j == 1 ? a1 : a2);
+                    acc += wq[c][b][0] * (odd ? u.y : u.x);
+                    acc += wq[c][b][1] * (odd ? v.x : u.y);
+                    acc += wq[c][b][2] * (odd ? v.y : v.x);
+                }
+            }
+        out[p] = a0;
+        out[n + p] = a1;
+        out[2 * n + p] = a2;
+        return;
+    }
 #pragma unroll
     for (int c = 0; c < 3; ++c) {
         int z = lc[2] + c - 1;
