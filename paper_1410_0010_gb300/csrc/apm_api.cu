@@ -86,6 +86,7 @@ struct Level {
     int packing = 0;                 // 0 hierarchy order, 1 largest transform first
     Chunk* d_gas = nullptr; int n_gas = 0;
     Chunk* d_acc = nullptr; int n_acc = 0;
+    int acc_zs = 1;                  // two-point acceleration: blocks a thread marches through
     std::vector<int> acc_first;      // per grid: its first acceleration chunk (ng + 1 entries)
     // pointer tables (device) + pinned mirrors + last uploaded values
     int cap = 0;
@@ -956,14 +957,27 @@ apm_status apm_set_hierarchy(apm_ctx* c, const apm_grid* grids, int32_t n) {
         if ((st = upload(c, &L.d_grids, L.hg)) != APM_OK) return st;
         std::vector<Chunk> gas, acc;
         L.acc_first.assign(ng + 1, 0);
+        // the acceleration's march: as long as it leaves kAccWaves CTAs per SM
+        {
+            constexpr int kSms = 152, kAccWaves = 8;
+            for (L.acc_zs = kAccMarch; L.acc_zs > 1; L.acc_zs /= 2) {
+                long long n_cta = 0;
+                for (const GridDev& g : L.hg)
+                    n_cta += ((long long)g.acc_nb[0] * g.acc_nb[1] + kAccThreads - 1) / kAccThreads *
+                             ((g.acc_nb[2] + L.acc_zs - 1) / L.acc_zs);
+                if (n_cta >= kSms * kAccWaves) break;
+            }
+        }
         for (int k = 0; k < ng; ++k) {
             L.acc_first[k] = (int)acc.size();
             const GridDev& g = L.hg[k];
             const long long grows = (long long)g.G[1] * g.G[2];
             for (long long t = 0; t < (grows + g.rows_gas - 1) / g.rows_gas; ++t) gas.push_back({k, (int)t});
             const long long nblocks = (long long)g.acc_nb[0] * g.acc_nb[1] * g.acc_nb[2];
-            for (long long t = 0; t < (nblocks + kAccBlocksPerCta - 1) / kAccBlocksPerCta; ++t)
-                acc.push_back({k, (int)t});
+            const long long ncc = ((long long)g.acc_nb[0] * g.acc_nb[1] + kAccThreads - 1) / kAccThreads;
+            const long long nch = cfg.gradient == APM_GRAD_FD2 ? ncc * ((g.acc_nb[2] + L.acc_zs - 1) / L.acc_zs)
+                                                               : (nblocks + kAccBlocksPerCta - 1) / kAccBlocksPerCta;
+            for (long long t = 0; t < nch; ++t) acc.push_back({k, (int)t});
         }
         L.acc_first[ng] = (int)acc.size();
         for (int q = 0; q < kFftPasses; ++q) {
@@ -1615,9 +1629,9 @@ apm_status apm_accel(apm_ctx* c, int32_t level, const void* const* phi_short,
         if (grad == APM_GRAD_FD2)
             e = c->cfg.precision == APM_FP64
                 ? launch_accel<double>(L.dev, pgrids, (const void* const*)d_phis, (const void* const*)d_pphi,
-                                       (const void* const*)d_pacc, d_phi, d_acc, ch, nch, s)
+                                       (const void* const*)d_pacc, d_phi, d_acc, ch, nch, L.acc_zs, s)
                 : launch_accel<float>(L.dev, pgrids, (const void* const*)d_phis, (const void* const*)d_pphi,
-                                      (const void* const*)d_pacc, d_phi, d_acc, ch, nch, s);
+                                      (const void* const*)d_pacc, d_phi, d_acc, ch, nch, L.acc_zs, s);
         else
             e = c->cfg.precision == APM_FP64
                 ? launch_accel_var<double>(L.dev, pgrids, (const void* const*)d_phis, (const void* const*)d_pphi,

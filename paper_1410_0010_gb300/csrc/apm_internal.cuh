@@ -270,9 +270,22 @@ struct RowWalk {
     }
 };
 
-// 2x2x2 output blocks per CTA of the acceleration kernel (flat ranges of the
-// grid's blocks, x fastest, so every thread gets the same count)
+// 2x2x2 output blocks per CTA of the four-point and spectral acceleration
+// kernel (flat ranges of the grid's blocks, x fastest, so every thread gets the
+// same count)
 constexpr int kAccBlocksPerCta = 512;
+// threads of an acceleration CTA; the two-point kernel gives each one (x, y)
+// column of blocks and marches through up to kAccMarch blocks of it (4 to 16
+// measure alike on large levels; the host halves it while a level would leave
+// SMs idle)
+#ifndef APM_ACC_THREADS
+#define APM_ACC_THREADS 128
+#endif
+constexpr int kAccThreads = APM_ACC_THREADS;
+#ifndef APM_ACC_MARCH
+#define APM_ACC_MARCH 8
+#endif
+constexpr int kAccMarch = APM_ACC_MARCH;
 
 // Threads of a CTA walking the flat range [f0, f0 + count) of elements of rows
 // of length n: thread t starts at f0 + t and strides by the block size, with
@@ -610,18 +623,19 @@ cudaError_t launch_fft_fast(int kernel, bool f64, int L, const FftArgs& a, const
 cudaError_t configure_fft_fast(int kernel, bool f64, int L);
 
 // accelerations + parent carry for the four-point and spectral gradients (the
-// two-point one runs launch_accel), on launch_accel's block work list
+// two-point one runs launch_accel), on flat ranges of blocks
 template <typename T>
 cudaError_t launch_accel_var(const LevelDev& L, const GridDev* parent_grids, const void* const* phis,
                                const void* const* pphi, const void* const* pacc, void* const* phi,
                                void* const* acc, const Chunk* chunks, int n_chunks, int grad,
                                cudaStream_t s);
 
-// FD accelerations + parent carry; TSC interpolation
+// FD accelerations + parent carry (two-point; a chunk is kAccThreads columns of
+// blocks of one segment of zs blocks along z); TSC interpolation
 template <typename T>
 cudaError_t launch_accel(const LevelDev& L, const GridDev* parent_grids, const void* const* phis,
                          const void* const* pphi, const void* const* pacc, void* const* phi,
-                         void* const* acc, const Chunk* chunks, int n_chunks,
+                         void* const* acc, const Chunk* chunks, int n_chunks, int zs,
                          cudaStream_t s);
 template <typename T>
 cudaError_t launch_interp(const LevelDev& L, const LevelDev* finer, const Particles& P,

@@ -10,10 +10,9 @@ namespace {
 // I is the trilinear interpolation from the parent cell centres (Sec. 2.2), for
 // R = 2: level cells 2k+1 and 2k+2 lie 1/4 and 3/4 of a parent cell above the
 // centre of parent cell k, so they weigh parent cells (k, k+1) with (3/4, 1/4)
-// and (1/4, 3/4).  Each thread computes one 2x2x2 block of such cells: the 8
-// parent values of a field serve all 8 cells, interpolated separably (x, then
-// y, then z), and the 32 values of phis around the block serve the 8 centred
-// differences.  Everything is evaluated in T; the weights are exact.
+// and (1/4, 3/4).  The work unit is a 2x2x2 block of such cells: the 8 parent
+// values of a field serve all 8 cells, interpolated separably (x, then y, then
+// z).  Everything is evaluated in T; the weights are exact.
 // A block may straddle the edge of [-1, N]: its outside cells are not written
 // and the loads they would need are clamped into the window.
 template <typename T>
@@ -57,227 +56,192 @@ __device__ __forceinline__ void load_parent(const T* __restrict__ f, unsigned ba
             for (int dx = 0; dx < 2; ++dx) q[dz][dy][dx] = f[base + dx + dy * P0 + dz * P01];
 }
 
-// CTA size and minimum resident CTAs per SM of the FP32 acceleration kernel
-#ifndef APM_ACC_THREADS
-#define APM_ACC_THREADS 128
-#endif
+// minimum resident CTAs per SM of the FP32 acceleration kernels: the two-point
+// march wants its 128 registers (32 grids of 128^3: 324 us at 4 CTAs, 402 at 5,
+// 490 at 6, 376 at 3), the others one block per thread
 #ifndef APM_ACC_MIN_CTAS
-#define APM_ACC_MIN_CTAS 6
+#define APM_ACC_MIN_CTAS 4
 #endif
-constexpr int kAccThreads = APM_ACC_THREADS;
-template <typename T> struct AccMinCtas { static constexpr int value = APM_ACC_MIN_CTAS; };
-template <> struct AccMinCtas<double> { static constexpr int value = 1; };
+template <typename T> struct AccMinCtas { static constexpr int march = APM_ACC_MIN_CTAS, value = 6; };
+template <> struct AccMinCtas<double> { static constexpr int march = 1, value = 1; };
 
+// The two-point difference.  What bounds it is the latency of its loads (and
+// HBM: 0.60 of the measured copy rate with one block per thread).  A thread
+// marches up z through zs blocks of one (x, y) column, so a block takes from the
+// one below it the parent plane between them, interpolated in x and y, and the
+// potential planes: 16 parent values and 16 loads of the potential a block
+// instead of 32 and 24.  The next block's first plane is loaded with the current
+// one (its centres are this block's upper z neighbours).
+// 32 refined grids of 128^3: 391 -> 324 us (1566 MB: 4.0 -> 4.8 TB/s).
+
+// the potential around one plane of a block: rows 0, 1 at x = -1 .. 2 (relative
+// to the block's cells), rows -1 and 2 at x = 0, 1
+template <typename T> struct AccPlane {
+    T x[2][4], y[2][2];
+};
 template <typename T>
-__global__ void __launch_bounds__(kAccThreads, AccMinCtas<T>::value) k_accel(LevelDev L, const GridDev* __restrict__ pgrids,
-                                               const void* const* __restrict__ phis_p,
-                                               const void* const* __restrict__ pphi_p,
-                                               const void* const* __restrict__ pacc_p,
-                                               void* const* __restrict__ phi_p,
-                                               void* const* __restrict__ acc_p,
-                                               const Chunk* __restrict__ chunks) {
+__device__ __forceinline__ AccPlane<T> load_acc_plane(const T* __restrict__ f, const unsigned yrow[4], int ex0,
+                                                      const int xi[4], bool vload) {
+    using V2 = typename Cplx<T>::type;
+    AccPlane<T> r;
+#pragma unroll
+    for (int b = 0; b < 2; ++b) {
+        const T* __restrict__ row = f + yrow[1 + b];
+        if (vload) {
+            const V2 u = *reinterpret_cast<const V2*>(row + ex0), v = *reinterpret_cast<const V2*>(row + ex0 + 2);
+            r.x[b][0] = u.x; r.x[b][1] = u.y; r.x[b][2] = v.x; r.x[b][3] = v.y;
+        } else {
+#pragma unroll
+            for (int k = 0; k < 4; ++k) r.x[b][k] = row[xi[k]];
+        }
+#pragma unroll
+        for (int a = 0; a < 2; ++a) r.y[b][a] = f[yrow[3 * b] + xi[1 + a]];
+    }
+    return r;
+}
+// a parent plane's 2x2 values of a field at the block's four (x, y) positions
+template <typename T>
+__device__ __forceinline__ void lerp_plane(const T* __restrict__ f, unsigned base, int P0, T out[2][2]) {
+    const T a = (T)0.75, b = (T)0.25;
+    const T q00 = f[base], q01 = f[base + 1], q10 = f[base + P0], q11 = f[base + P0 + 1];
+    const T x00 = a * q00 + b * q01, x01 = b * q00 + a * q01, x10 = a * q10 + b * q11, x11 = b * q10 + a * q11;
+    out[0][0] = a * x00 + b * x10;
+    out[0][1] = a * x01 + b * x11;
+    out[1][0] = b * x00 + a * x10;
+    out[1][1] = b * x01 + a * x11;
+}
+
+template <typename T, bool CARRY>
+__global__ void __launch_bounds__(kAccThreads, AccMinCtas<T>::march) k_accel(
+    LevelDev L, const GridDev* __restrict__ pgrids, const void* const* __restrict__ phis_p,
+    const void* const* __restrict__ pphi_p, const void* const* __restrict__ pacc_p, void* const* __restrict__ phi_p,
+    void* const* __restrict__ acc_p, const Chunk* __restrict__ chunks, int zs) {
     const Chunk ch = chunks[blockIdx.x];
     const GridDev& g = L.g[ch.grid];
+    const int nbx = g.acc_nb[0], ncol = nbx * g.acc_nb[1], nbz = g.acc_nb[2];
+    const int ncc = (ncol + kAccThreads - 1) / kAccThreads;   // CTAs across the columns
+    const int seg = ch.tile / ncc;
+    const int col = (ch.tile - seg * ncc) * kAccThreads + (int)threadIdx.x;
+    if (col >= ncol) return;
+    const int by = col / nbx;
+    const int ex0 = 2 * (col - by * nbx) - g.acc_sh[0], ey0 = 2 * by - g.acc_sh[1];
+    const int bz0 = seg * zs, bz1 = min(nbz, bz0 + zs);
     const int E0 = g.N[0] + 2, E1 = g.N[1] + 2, E2 = g.N[2] + 2;
     const unsigned ncell = (unsigned)E0 * E1 * E2;
     const int W0 = g.W[0], W1 = g.W[1], W2 = g.W[2];
-    const int nbx = g.acc_nb[0], nby = g.acc_nb[1];
-    const int nbrows = nby * g.acc_nb[2];
     const T* __restrict__ phis = reinterpret_cast<const T*>(phis_p[ch.grid]);
     T* __restrict__ phi = reinterpret_cast<T*>(phi_p[ch.grid]);
     T* __restrict__ acc = reinterpret_cast<T*>(acc_p[ch.grid]);
-    const bool carry = pphi_p != nullptr && g.parent >= 0;
-    const T* __restrict__ pphi = carry ? reinterpret_cast<const T*>(pphi_p[g.parent]) : nullptr;
-    const T* __restrict__ pacc = carry ? reinterpret_cast<const T*>(pacc_p[g.parent]) : nullptr;
+    const T inv2d = (T)g.inv2d;
+    // output cell e has phis index e + 1 on each axis; clamped into [0, W)
+    const unsigned sz = (unsigned)W0 * W1;
+    unsigned yrow[4];
+    int xi[4];
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+        yrow[k] = (unsigned)W0 * (unsigned)min(max(ey0 + k, 0), W1 - 1);
+        xi[k] = min(max(ex0 + k, 0), W0 - 1);
+    }
+    // pair loads and stores need even row lengths and pointers aligned to two elements
+    using V2 = typename Cplx<T>::type;
+    const size_t amask = 2 * sizeof(T) - 1;
+    const bool vpair = !((W0 | E0 | ex0) & 1) && !(reinterpret_cast<size_t>(phis) & amask) &&
+                       !(reinterpret_cast<size_t>(phi) & amask) && !(reinterpret_cast<size_t>(acc) & amask) &&
+                       !((size_t)ncell & 1);
+    const bool vload = vpair && ex0 >= 0 && ex0 + 3 <= W0 - 1;
+    // cells written: x = ex0 + a, y = ey0 + b
+    const bool wx0 = ex0 >= 0 && ex0 < E0, wx1 = ex0 + 1 < E0;
+    const bool wy0 = ey0 >= 0 && ey0 < E1, wy1 = ey0 + 1 < E1;
+    // parent: cell k of the odd level cell (2k+1) of each pair
+    const T *pf[4] = {nullptr, nullptr, nullptr, nullptr};
     int P0 = 0;
-    unsigned P01 = 0, pn = 0;
-    long long ps[3] = {0, 0, 0};
-    if (carry) {
+    unsigned P01 = 0, pn = 0, pbase = 0;
+    T yp[4][2][2];   // phi and the accelerations on the parent plane below the block
+    if (CARRY) {
         const GridDev& p = pgrids[g.parent];
         P0 = p.N[0] + 2;
         P01 = (unsigned)P0 * (p.N[1] + 2);
         pn = P01 * (p.N[2] + 2);
-        ps[0] = p.start[0]; ps[1] = p.start[1]; ps[2] = p.start[2];
+        pf[0] = reinterpret_cast<const T*>(pphi_p[g.parent]);
+#pragma unroll
+        for (int j = 0; j < 3; ++j) pf[1 + j] = reinterpret_cast<const T*>(pacc_p[g.parent]) + (size_t)j * pn;
+        const long long kx = ((g.start[0] + ex0 - 1) - 1) >> 1, ky = ((g.start[1] + ey0 - 1) - 1) >> 1;
+        const long long kz = ((g.start[2] + 2 * bz0 - g.acc_sh[2] - 1) - 1) >> 1;
+        pbase = (unsigned)(kx - p.start[0] + 1) + (unsigned)(ky - p.start[1] + 1) * (unsigned)P0 +
+                (unsigned)(kz - p.start[2] + 1) * P01;
+        // the blocks' parent cells: pbase .. pbase + 1 + P0 + (bz1 - bz0) P01
+        if (!APM_IN_BOUNDS((long long)pbase + 1 + P0 + (long long)(bz1 - bz0) * P01, pn, L.status)) return;
+#pragma unroll
+        for (int j = 0; j < 4; ++j) lerp_plane(pf[j], pbase, P0, yp[j]);
     }
-    const T inv2d = (T)g.inv2d;
-    const unsigned sy = W0, sz = (unsigned)W0 * W1;
-    const long long nblocks = (long long)nbx * nbrows;
-    const long long f0 = (long long)ch.tile * kAccBlocksPerCta;
-    const int count = (int)min((long long)kAccBlocksPerCta, nblocks - f0);
-    // pair loads and stores need even row lengths and pointers aligned to two elements
-    using V2 = typename Cplx<T>::type;
-    const size_t amask = 2 * sizeof(T) - 1;
-    const bool valign = !(W0 & 1) && !(E0 & 1) && !(reinterpret_cast<size_t>(phis) & amask) &&
-                        !(reinterpret_cast<size_t>(phi) & amask) && !(reinterpret_cast<size_t>(acc) & amask) &&
-                        !((size_t)ncell & 1);
-    int last = -1;
-    int ey0 = 0, ez0 = 0;
-    unsigned ybase[4] = {0, 0, 0, 0}, zbase[4] = {0, 0, 0, 0};   // phis offsets of rows -1, 0, 1, 2 of the block
-    unsigned prow = 0;
-    for (FlatWalk it(f0, count, nbx); it.ok(); it.next()) {
-        if (it.r != last) {
-            last = it.r;
-            const int by = it.r % nby, bz = it.r / nby;
-            ey0 = 2 * by - g.acc_sh[1];
-            ez0 = 2 * bz - g.acc_sh[2];
-            // output cell e has phis index e + 1 on each axis; clamp into [0, W)
+    auto plane = [&](int k) { return phis + sz * (unsigned)min(max(k, 0), W2 - 1); };
+    int ez0 = 2 * bz0 - g.acc_sh[2];
+    T z0[2][2];   // centres of the plane below the block
+    {
+        const T* __restrict__ f = plane(ez0);
 #pragma unroll
-            for (int k = 0; k < 4; ++k) {
-                ybase[k] = sy * (unsigned)min(max(ey0 + k, 0), W1 - 1);
-                zbase[k] = sz * (unsigned)min(max(ez0 + k, 0), W2 - 1);
-            }
-            if (carry) {
-                // the odd level cell of the block's pair (2k+1) gives parent cell k
-                const long long ky = ((g.start[1] + ey0 - 1) - 1) >> 1;
-                const long long kz = ((g.start[2] + ez0 - 1) - 1) >> 1;
-                prow = (unsigned)(ky - ps[1] + 1) * (unsigned)P0 + (unsigned)(kz - ps[2] + 1) * P01;
-            }
+        for (int b = 0; b < 2; ++b)
+#pragma unroll
+            for (int a = 0; a < 2; ++a) z0[b][a] = f[yrow[1 + b] + xi[1 + a]];
+    }
+    AccPlane<T> p1 = load_acc_plane(plane(ez0 + 1), yrow, ex0, xi, vload);
+#pragma unroll 1
+    for (int bz = bz0; bz < bz1; ++bz, ez0 += 2) {
+        const AccPlane<T> p2 = load_acc_plane(plane(ez0 + 2), yrow, ex0, xi, vload);
+        const AccPlane<T> p3 = load_acc_plane(plane(ez0 + 3), yrow, ex0, xi, vload);
+        T yn[4][2][2];   // the parent plane above
+        if (CARRY) {
+            pbase += P01;
+#pragma unroll
+            for (int j = 0; j < 4; ++j) lerp_plane(pf[j], pbase, P0, yn[j]);
         }
-        const int ex0 = 2 * it.x - g.acc_sh[0];
-        int xi[4];
-#pragma unroll
-        for (int k = 0; k < 4; ++k) xi[k] = min(max(ex0 + k, 0), W0 - 1);
-        // phis of the four centre rows at x indices ex0 .. ex0+3 (the x
-        // neighbours and the centres e + 1 = ex0 + 1 + a): two pair loads when
-        // the row is even-aligned and unclamped
-        const bool vload = valign && ex0 >= 0 && ex0 + 3 <= W0 - 1 && !(ex0 & 1);
-        T xr[2][2][4];
-#pragma unroll
-        for (int c = 0; c < 2; ++c)
-#pragma unroll
-            for (int b = 0; b < 2; ++b) {
-                const unsigned row = zbase[1 + c] + ybase[1 + b];
-                if (vload) {
-                    const V2 u = *reinterpret_cast<const V2*>(phis + row + ex0);
-                    const V2 v = *reinterpret_cast<const V2*>(phis + row + ex0 + 2);
-                    xr[c][b][0] = u.x; xr[c][b][1] = u.y; xr[c][b][2] = v.x; xr[c][b][3] = v.y;
-                } else {
-#pragma unroll
-                    for (int k = 0; k < 4; ++k) xr[c][b][k] = phis[row + xi[k]];
-                }
+        const bool wz[2] = {ez0 >= 0 && ez0 < E2, ez0 + 1 < E2};
+        // field j (0 phi, 1-3 acc) of cells (.., b, c): values v0, v1 plus the carry
+        auto put = [&](T* __restrict__ f, int j, int c, int b, T v0, T v1) {
+            if (CARRY) {
+                const T a = c == 0 ? (T)0.75 : (T)0.25, d = c == 0 ? (T)0.25 : (T)0.75;
+                v0 += a * yp[j][b][0] + d * yn[j][b][0];
+                v1 += a * yp[j][b][1] + d * yn[j][b][1];
             }
-        T out[2][2][2], q[2][2][2];
-        unsigned pbase = 0;
-        if (carry) {
-            const long long kx = ((g.start[0] + ex0 - 1) - 1) >> 1;
-            pbase = prow + (unsigned)(kx - ps[0] + 1);
-            // the block's 8 parent cells: pbase .. pbase + 1 + P0 + P01
-            if (!APM_IN_BOUNDS((long long)pbase + 1 + P0 + P01, pn, L.status)) continue;
-        }
-        // output cells: (ex0 + a, ey0 + b, ez0 + c); the pair a = 0, 1 is one
-        // aligned pair store when both are inside and ex0 is even
-        bool wr[2][2][2];
-        unsigned o[2][2];
-#pragma unroll
-        for (int c = 0; c < 2; ++c)
-#pragma unroll
-            for (int b = 0; b < 2; ++b) {
-                const int ey = ey0 + b, ez = ez0 + c;
-                const bool yz = ey >= 0 && ey < E1 && ez >= 0 && ez < E2;
-                wr[c][b][0] = yz && ex0 >= 0 && ex0 < E0;
-                wr[c][b][1] = yz && ex0 + 1 < E0;
-                o[c][b] = (unsigned)ex0 + (unsigned)E0 * ((unsigned)ey + (unsigned)E1 * (unsigned)ez);
-            }
-        const bool vpair = valign && !(ex0 & 1);
-        auto put = [&](T* __restrict__ f, int c, int b, T v0, T v1) {
-            if (vpair && wr[c][b][0] && wr[c][b][1]) {
-                *reinterpret_cast<V2*>(f + o[c][b]) = mk2(v0, v1);
+            if (!((b == 0 ? wy0 : wy1) && wz[c])) return;
+            // signed: with ex0 = -1 the row's first written cell is o[1] (fields hold fewer than 2^31 cells)
+            T* __restrict__ o = f + (ex0 + E0 * ((ey0 + b) + E1 * (ez0 + c)));
+            if (vpair && wx0 && wx1) {
+                *reinterpret_cast<V2*>(o) = mk2(v0, v1);
             } else {
-                if (wr[c][b][0]) f[o[c][b]] = v0;
-                if (wr[c][b][1]) f[o[c][b] + 1] = v1;
+                if (wx0) o[0] = v0;
+                if (wx1) o[1] = v1;
             }
         };
-        // phi
-        if (carry) {
-            load_parent<T>(pphi, pbase, P0, P01, q);
-            lerp_block<T>(q, out);
-        }
 #pragma unroll
-        for (int c = 0; c < 2; ++c)
+        for (int c = 0; c < 2; ++c) {
+            const AccPlane<T>& p = c == 0 ? p1 : p2;
 #pragma unroll
             for (int b = 0; b < 2; ++b) {
-                T v0 = xr[c][b][1], v1 = xr[c][b][2];
-                if (carry) {
-                    v0 += out[c][b][0];
-                    v1 += out[c][b][1];
-                }
-                put(phi, c, b, v0, v1);
-            }
-        // acc_x: neighbours xr[.][.][0] and xr[.][.][3]
-        {
-            if (carry) {
-                load_parent<T>(pacc, pbase, P0, P01, q);
-                lerp_block<T>(q, out);
-            }
-#pragma unroll
-            for (int c = 0; c < 2; ++c)
-#pragma unroll
-                for (int b = 0; b < 2; ++b) {
-                    T g0 = -(xr[c][b][2] - xr[c][b][0]) * inv2d;
-                    T g1 = -(xr[c][b][3] - xr[c][b][1]) * inv2d;
-                    if (carry) {
-                        g0 += out[c][b][0];
-                        g1 += out[c][b][1];
-                    }
-                    put(acc, c, b, g0, g1);
-                }
-        }
-        // acc_y: rows ybase[0] and ybase[3]
-        {
-            if (carry) {
-                load_parent<T>(pacc + pn, pbase, P0, P01, q);
-                lerp_block<T>(q, out);
-            }
-            T gy[2][2][2];
-#pragma unroll
-            for (int c = 0; c < 2; ++c)
+                put(phi, 0, c, b, p.x[b][1], p.x[b][2]);
+                put(acc, 1, c, b, -(p.x[b][2] - p.x[b][0]) * inv2d, -(p.x[b][3] - p.x[b][1]) * inv2d);
+                T gy[2], gz[2];
 #pragma unroll
                 for (int a = 0; a < 2; ++a) {
-                    const T lo = phis[zbase[1 + c] + ybase[0] + xi[1 + a]];
-                    const T hi = phis[zbase[1 + c] + ybase[3] + xi[1 + a]];
-                    gy[c][0][a] = -(xr[c][1][1 + a] - lo) * inv2d;
-                    gy[c][1][a] = -(hi - xr[c][0][1 + a]) * inv2d;
+                    const T ylo = b == 0 ? p.y[0][a] : p.x[0][1 + a], yhi = b == 0 ? p.x[1][1 + a] : p.y[1][a];
+                    const T zlo = c == 0 ? z0[b][a] : p1.x[b][1 + a], zhi = c == 0 ? p2.x[b][1 + a] : p3.x[b][1 + a];
+                    gy[a] = -(yhi - ylo) * inv2d;
+                    gz[a] = -(zhi - zlo) * inv2d;
                 }
-#pragma unroll
-            for (int c = 0; c < 2; ++c)
-#pragma unroll
-                for (int b = 0; b < 2; ++b) {
-                    T v0 = gy[c][b][0], v1 = gy[c][b][1];
-                    if (carry) {
-                        v0 += out[c][b][0];
-                        v1 += out[c][b][1];
-                    }
-                    put(acc + ncell, c, b, v0, v1);
-                }
-        }
-        // acc_z: planes zbase[0] and zbase[3]
-        {
-            if (carry) {
-                load_parent<T>(pacc + 2 * pn, pbase, P0, P01, q);
-                lerp_block<T>(q, out);
+                put(acc + ncell, 2, c, b, gy[0], gy[1]);
+                put(acc + 2 * ncell, 3, c, b, gz[0], gz[1]);
             }
-            T gz[2][2][2];
-#pragma unroll
-            for (int b = 0; b < 2; ++b)
-#pragma unroll
-                for (int a = 0; a < 2; ++a) {
-                    const T lo = phis[zbase[0] + ybase[1 + b] + xi[1 + a]];
-                    const T hi = phis[zbase[3] + ybase[1 + b] + xi[1 + a]];
-                    gz[0][b][a] = -(xr[1][b][1 + a] - lo) * inv2d;
-                    gz[1][b][a] = -(hi - xr[0][b][1 + a]) * inv2d;
-                }
-#pragma unroll
-            for (int c = 0; c < 2; ++c)
-#pragma unroll
-                for (int b = 0; b < 2; ++b) {
-                    T v0 = gz[c][b][0], v1 = gz[c][b][1];
-                    if (carry) {
-                        v0 += out[c][b][0];
-                        v1 += out[c][b][1];
-                    }
-                    put(acc + 2 * ncell, c, b, v0, v1);
-                }
         }
+#pragma unroll
+        for (int b = 0; b < 2; ++b)
+#pragma unroll
+            for (int a = 0; a < 2; ++a) {
+                z0[b][a] = p2.x[b][1 + a];
+                if (CARRY)
+#pragma unroll
+                    for (int j = 0; j < 4; ++j) yp[j][b][a] = yn[j][b][a];
+            }
+        p1 = p3;
     }
 }
 
@@ -691,10 +655,13 @@ __global__ void __launch_bounds__(kAccThreads, AccMinCtas<T>::value) k_accel_var
 template <typename T>
 cudaError_t launch_accel(const LevelDev& L, const GridDev* parent_grids, const void* const* phis,
                          const void* const* pphi, const void* const* pacc, void* const* phi,
-                         void* const* acc, const Chunk* chunks, int n_chunks,
+                         void* const* acc, const Chunk* chunks, int n_chunks, int zs,
                          cudaStream_t s) {
     if (n_chunks <= 0) return cudaSuccess;
-    k_accel<T><<<n_chunks, kAccThreads, 0, s>>>(L, parent_grids, phis, pphi, pacc, phi, acc, chunks);
+    if (pphi)   // every grid of a level that gets parent fields has a parent
+        k_accel<T, true><<<n_chunks, kAccThreads, 0, s>>>(L, parent_grids, phis, pphi, pacc, phi, acc, chunks, zs);
+    else
+        k_accel<T, false><<<n_chunks, kAccThreads, 0, s>>>(L, parent_grids, phis, pphi, pacc, phi, acc, chunks, zs);
     return cudaGetLastError();
 }
 
@@ -734,10 +701,10 @@ cudaError_t launch_interp_levels(const LevelDev* levels, int nl, const Particles
 
 template cudaError_t launch_accel<float>(const LevelDev&, const GridDev*, const void* const*,
                                          const void* const*, const void* const*, void* const*,
-                                         void* const*, const Chunk*, int, cudaStream_t);
+                                         void* const*, const Chunk*, int, int, cudaStream_t);
 template cudaError_t launch_accel<double>(const LevelDev&, const GridDev*, const void* const*,
                                           const void* const*, const void* const*, void* const*,
-                                          void* const*, const Chunk*, int, cudaStream_t);
+                                          void* const*, const Chunk*, int, int, cudaStream_t);
 template cudaError_t launch_accel_var<float>(const LevelDev&, const GridDev*, const void* const*,
                                                const void* const*, const void* const*, void* const*,
                                                void* const*, const Chunk*, int, int, cudaStream_t);
