@@ -388,10 +388,11 @@ apm_status build_pass(apm_ctx* c, const Level& L, int q, int budget, int threads
     };
     // ... and the fused y + x inverse (k_yx_fast) as its x-inverse segment when
     // the window's row pairs are distinct rows of the transform (2 ceil(W1/2)
-    // <= M1: a periodic root, whose window is taller than M1, is excluded)
+    // <= M1: a periodic root, whose window is taller than M1, is excluded) and
+    // its rows no longer than the transform's
     auto fused_yx = [&](const GridDev& g) {
         return !f64 && fuses(kPassXi, g.M[0]) && fft_fast_enabled() && g.M[0] == g.M[1] && fast_xy_length(g.M[0]) &&
-               2 * ((g.W[1] + 1) / 2) <= g.M[1];
+               2 * ((g.W[1] + 1) / 2) <= g.M[1] && g.W[0] <= g.M[0];
     };
     for (int k = 0; k < ng; ++k) {
         const GridDev& g = L.hg[k];

@@ -533,6 +533,45 @@ struct Particles {
 };
 
 // ---------------------------------------------------------------------------
+// launches
+// ---------------------------------------------------------------------------
+// Every kernel of a solve is launched as a programmatic dependent of the one
+// before it on its stream, so the launch itself overlaps that one's end; each
+// begins with begin_kernel(), which waits until everything before it is complete
+// and visible (nothing is read or written early, whatever comes before: a kernel
+// of the caller's, a copy, another stream joined by an event).  The 9 launches of
+// an isolated 96^3 root's solve 59.7 -> 52.7 us, a 1 M Plummer step of three
+// nested levels 826 -> 765, 32 grids of 128^3 886 -> 871, a two-level 64^3 step
+// replayed as a graph 97.6 -> 95.9.  Letting the next kernel's CTAs in early
+// (griddepcontrol.launch_dependents) costs more than it gives: the cosmological
+// step 10.2 -> 11.6 ms, that graph 99.5 -> 123 us.
+// The block index comes out of the same instruction sequence, so that every
+// address a kernel forms from it, and with it every load, depends on the wait
+// (loads through const __restrict__ pointers may otherwise be moved across it).
+__device__ __forceinline__ unsigned begin_kernel() {
+    unsigned block;
+    asm volatile("griddepcontrol.wait;\n\tmov.u32 %0, %%ctaid.x;" : "=r"(block) : : "memory");
+    return block;
+}
+template <typename... KA, typename... A>
+cudaError_t launch_kernel(void (*kernel)(KA...), unsigned blocks, unsigned threads, size_t smem, cudaStream_t s,
+                          A... args) {
+    cudaLaunchAttribute attr{};
+    attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr.val.programmaticStreamSerializationAllowed = 1;
+    cudaLaunchConfig_t cfg{};
+    cfg.gridDim = dim3(blocks);
+    cfg.blockDim = dim3(threads);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = s;
+    cfg.attrs = &attr;
+    cfg.numAttrs = 1;
+    const cudaError_t e = cudaLaunchKernelEx(&cfg, kernel, static_cast<KA>(args)...);
+    if (e != cudaSuccess) cudaGetLastError();
+    return e;
+}
+
+// ---------------------------------------------------------------------------
 // launchers (each returns the launch error)
 // ---------------------------------------------------------------------------
 // twiddles exp(-2 pi i t / L) for t < L, FP64 and FP32

@@ -676,7 +676,8 @@ __global__ void __launch_bounds__(NT, MinCtas<T>::value * (kFftThreads / NT)) k_
                                                      const T* __restrict__ tab,
                                                      C<T>* __restrict__ wsA, C<T>* __restrict__ wsB,
                                                      int comp) {
-    const Chunk ch = chunks[blockIdx.x];
+    const unsigned block = begin_kernel();
+    const Chunk ch = chunks[block];
     const GridDev& g = grids[ch.grid];
     const int Hx = g.Hx;
     const int tx = g.lines[AX == 2 ? kPassZ : (MODE == 0 ? kPassYf : kPassYi)];
@@ -808,8 +809,9 @@ __global__ void __launch_bounds__(NT, MinCtas<T>::value * (kFftThreads / NT)) k_
                                                     const C<T>* __restrict__ tw_arena,
                                                     C<T>* __restrict__ wsA, int F,
                                                     unsigned* __restrict__ status, int inject_wait) {
+    const unsigned block = begin_kernel();
     extern __shared__ __align__(128) unsigned char smem_xf[];
-    const Chunk ch = chunks[blockIdx.x];
+    const Chunk ch = chunks[block];
     const GridDev& g = grids[ch.grid];
     const int M0 = g.M[0], G0 = g.G[0], Hx = g.Hx, np = g.lines[kPassXf], lg = ilog2(np), es = np + 1;
     const size_t stage = fft_xf_stage_bytes(np, G0);
@@ -895,7 +897,8 @@ __global__ void __launch_bounds__(NT, MinCtas<T>::value * (kFftThreads / NT)) k_
                                                     const C<T>* __restrict__ tw_arena,
                                                     const C<T>* __restrict__ wsB,
                                                     void* const* __restrict__ phis, int comp) {
-    const Chunk ch = chunks[blockIdx.x];
+    const unsigned block = begin_kernel();
+    const Chunk ch = chunks[block];
     const GridDev& g = grids[ch.grid];
     const int M0 = g.M[0], Hx = g.Hx, np = g.lines[kPassXi], W0 = g.W[0], lg = ilog2(np), es = np + 1;
     C<T>* cur = smem_c<T>();

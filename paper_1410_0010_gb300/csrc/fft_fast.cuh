@@ -103,10 +103,11 @@ __device__ __forceinline__ void fast_dif_stage(C<T>* buf, const C<T>* __restrict
         const int hi = b / S, lo = b - hi * S;
         const int base = hi * R * S + lo;
         C<T> v[R];
+        if constexpr (IN_G) {
+            gin.template ld<R, S>(base, v);
+        } else {
 #pragma unroll
-        for (int k = 0; k < R; ++k) {
-            if constexpr (IN_G) v[k] = gin.ld(base + k * S);
-            else v[k] = buf[(base + k * S) * PITCH + line];
+            for (int k = 0; k < R; ++k) v[k] = buf[(base + k * S) * PITCH + line];
         }
         FastDft<T, DIR, R>::run(v);
         if constexpr (S > 1) {
@@ -114,11 +115,11 @@ __device__ __forceinline__ void fast_dif_stage(C<T>* buf, const C<T>* __restrict
             for (int k = 1; k < R; ++k) v[k] = mul<T>(v[k], twid<T, DIR>(tw, lo * k * TWS));
         }
         static_assert(!OUT_G || S == 1, "global output only from the last stage");
-        const int nat0 = OUT_G ? P::natural(base) : 0;
+        if constexpr (OUT_G) {
+            gout.template st<R, P::last_weight()>(P::natural(base), v);
+        } else {
 #pragma unroll
-        for (int k = 0; k < R; ++k) {
-            if constexpr (OUT_G) gout.st(nat0 + k * P::last_weight(), v[k]);
-            else buf[(base + k * S) * PITCH + line] = v[k];
+            for (int k = 0; k < R; ++k) buf[(base + k * S) * PITCH + line] = v[k];
         }
     }
 }
@@ -145,21 +146,22 @@ __device__ __forceinline__ void fast_dit_stage(C<T>* buf, const C<T>* __restrict
         const int base = hi * R * S + lo;
         C<T> v[R];
         static_assert(!IN_G || S == 1, "global input only to the first inverse stage");
-        const int nat0 = IN_G ? P::natural(base) : 0;
+        if constexpr (IN_G) {
+            gin.template ld<R, P::last_weight()>(P::natural(base), v);
+        } else {
 #pragma unroll
-        for (int k = 0; k < R; ++k) {
-            if constexpr (IN_G) v[k] = gin.ld(nat0 + k * P::last_weight());
-            else v[k] = buf[(base + k * S) * PITCH + line];
+            for (int k = 0; k < R; ++k) v[k] = buf[(base + k * S) * PITCH + line];
         }
         if constexpr (S > 1) {
 #pragma unroll
             for (int k = 1; k < R; ++k) v[k] = mul<T>(v[k], twid<T, 1>(tw, lo * k * TWS));
         }
         FastDft<T, 1, R>::run(v);
+        if constexpr (OUT_G) {
+            gout.template st<R, S>(base, v);
+        } else {
 #pragma unroll
-        for (int k = 0; k < R; ++k) {
-            if constexpr (OUT_G) gout.st(base + k * S, v[k]);
-            else buf[(base + k * S) * PITCH + line] = v[k];
+            for (int k = 0; k < R; ++k) buf[(base + k * S) * PITCH + line] = v[k];
         }
     }
 }
@@ -182,49 +184,110 @@ __device__ __forceinline__ void fast_mid_stage(C<T>* buf, const TAB& tabf) {
         for (int k = 0; k < R; ++k) v[k] = buf[(base + k) * TX + line];
         FastDft<T, -1, R>::run(v);
         // natural index of output k: the digits of hi, then k as the last digit
-        const int k0 = P::natural(base);
-#pragma unroll
-        for (int k = 0; k < R; ++k) v[k] = tabf.apply(k0 + k * (L / R), v[k]);
+        tabf.template apply<R, L>(P::natural(base), v);
         FastDft<T, 1, R>::run(v);
 #pragma unroll
         for (int k = 0; k < R; ++k) buf[(base + k) * TX + line] = v[k];
     }
 }
 
-// Global element n of this thread's line: p[n stride] for n < n_in (zero
-// beyond: the padding); nothing for a dead line (kx >= Hx).  Offsets stay
+// A butterfly's R elements i0 + k W (k < R, W compile-time) of this thread's
+// global line, element i at p[i stride]: one address per butterfly, and per
+// element only a multiple of W stride, the same for every thread.  Offsets stay
 // 32-bit (lines of at most 1024 elements, strides below 1024 x 513).
-template <typename T> struct FastIn {
+// Inputs: zero for i >= n (the padding).  FULL: the line has no padding.
+template <typename T, bool FULL> struct FastIn {
     const C<T>* __restrict__ p;
     int stride, n;
-    bool live;
-    __device__ __forceinline__ C<T> ld(int i) const {
-        return (live && i < n) ? p[i * stride] : mk<T>(T(0), T(0));
+    template <int R, int W> __device__ __forceinline__ void ld(int i0, C<T>* v) const {
+        const C<T>* __restrict__ q = p + i0 * stride;
+        const int step = W * stride;
+#pragma unroll
+        for (int k = 0; k < R; ++k) v[k] = FULL || i0 + k * W < n ? q[k * step] : mk<T>(0, 0);
     }
 };
-// Output element i at window index w = (i - s0) mod L, written when w < n, and
+// Outputs: element i at window index w = (i - s0) mod L, written when w < n, and
 // again at w + L when that is inside the window too (a periodic root's window
-// N + 4 exceeds M = N).
+// N + 4 exceeds M = N).  wrap: the window passes the end of the line (the
+// roots); a line that is not there has n = 0 and no wrap.
 template <typename T, int L> struct FastOut {
     C<T>* __restrict__ p;
     int stride, n, s0;
-    bool live;
-    __device__ __forceinline__ void st(int i, C<T> v) const {
-        if (!live) return;
-        int w = i - s0;
-        if (w < 0) w += L;
-        if (w < n) p[w * stride] = v;
-        if (w + L < n) p[(w + L) * stride] = v;
+    bool wrap;
+    template <int R, int W> __device__ __forceinline__ void st(int i0, const C<T>* v) const {
+        const int w0 = i0 - s0;
+        if (!wrap) {
+            C<T>* __restrict__ q = p + w0 * stride;
+            const int step = W * stride;
+#pragma unroll
+            for (int k = 0; k < R; ++k)
+                if ((unsigned)(w0 + k * W) < (unsigned)n) q[k * step] = v[k];
+        } else {
+#pragma unroll
+            for (int k = 0; k < R; ++k) {
+                int w = w0 + k * W;
+                if (w < 0) w += L;
+                if (w < n) p[w * stride] = v[k];
+                if (w + L < n) p[(w + L) * stride] = v[k];
+            }
+        }
     }
 };
-
-// Output element i of a pass with no window (the y forward: all L outputs)
+// Outputs of a pass with no window (the y forward: all L of them)
 template <typename T> struct FastOutAll {
     C<T>* __restrict__ p;
     int stride;
     bool live;
-    __device__ __forceinline__ void st(int i, C<T> v) const {
-        if (live) p[i * stride] = v;
+    template <int R, int W> __device__ __forceinline__ void st(int i0, const C<T>* v) const {
+        if (!live) return;
+        C<T>* __restrict__ q = p + i0 * stride;
+        const int step = W * stride;
+#pragma unroll
+        for (int k = 0; k < R; ++k) q[k * step] = v[k];
+    }
+};
+
+// The z pass's table at the R elements kz = k0 + k L/R (k0 < L/R) of a column:
+// which side of L/2 an element lies on, and so how it folds onto the octant, is
+// known at compile time for all but the middle one or two.
+template <typename T> struct FastTab {
+    const T* __restrict__ p;   // at (|ky|, kx), kz = 0
+    int zst;
+    template <int R, int L> __device__ __forceinline__ void value(int k0, T* t) const {
+        constexpr int W = L / R;
+        const T* __restrict__ up = p + k0 * zst;
+        const T* __restrict__ down = p - k0 * zst;
+#pragma unroll
+        for (int k = 0; k < R; ++k) {
+            if (k * W + W - 1 <= L / 2) t[k] = up[k * W * zst];
+            else if (k * W > L / 2) t[k] = down[(L - k * W) * zst];
+            else t[k] = k0 + k * W <= L / 2 ? up[k * W * zst] : down[(L - k * W) * zst];
+        }
+    }
+    template <int R, int L> __device__ __forceinline__ void apply(int k0, C<T>* v) const {
+        T t[R];
+        value<R, L>(k0, t);
+#pragma unroll
+        for (int k = 0; k < R; ++k) v[k] = mk<T>(v[k].x * t[k], v[k].y * t[k]);
+    }
+};
+// ... times -i D_comp of a spectral-gradient component (see TabGrad)
+template <typename T> struct FastTabGrad {
+    FastTab<T> tab;
+    int comp;
+    T dline, dz;
+    template <int R, int L> __device__ __forceinline__ void apply(int k0, C<T>* v) const {
+        constexpr int W = L / R;
+        T t[R];
+        tab.template value<R, L>(k0, t);
+#pragma unroll
+        for (int k = 0; k < R; ++k) {
+            const int kz = k0 + k * W;
+            T d = dline;
+            if (comp == 3) d = 2 * kz == L ? T(0) : dz * (T)(kz <= L / 2 ? kz : kz - L);
+            const T f = t[k] * d;
+            v[k] = mk<T>(v[k].y * f, -v[k].x * f);
+        }
     }
 };
 
@@ -236,11 +299,12 @@ template <class P, int AX, int MODE, int TX, int NT, typename T>
 __global__ void __launch_bounds__(NT) k_col_fast(const GridDev* __restrict__ grids, const Chunk* __restrict__ chunks,
                                                  const C<T>* __restrict__ tw_arena, const T* __restrict__ tab,
                                                  C<T>* __restrict__ wsA, C<T>* __restrict__ wsB, int comp) {
+    const unsigned block = begin_kernel();
     constexpr int L = P::L;
     extern __shared__ __align__(16) unsigned char smem_fast[];
     C<T>* buf = reinterpret_cast<C<T>*>(smem_fast);
     C<T>* tw = buf + L * TX;
-    const Chunk ch = chunks[blockIdx.x];
+    const Chunk ch = chunks[block];
     const GridDev& g = grids[ch.grid];
     const int Hx = g.Hx;
     const int other = ch.tile & ((1 << kColOtherBits) - 1);
@@ -254,25 +318,28 @@ __global__ void __launch_bounds__(NT) k_col_fast(const GridDev* __restrict__ gri
     static_assert(NT % TX == 0, "NT must be a multiple of TX");
     const int line = threadIdx.x % TX;
     const bool live = kx0 + line < Hx;
-    FastIn<T> gin;
+    // a dead line reads its CTA's first column (its results are never stored)
+    const int in_line = live ? line : 0;
+    FastIn<T, MODE == 2> gin;
     FastOut<T, L> gout;
-    gin.live = gout.live = live;
     if (AX == 1 && MODE == 0) {
-        gin.p = wsA + (g.wsA + (long long)other * g.G[1] * Hx + kx0 + line);
+        gin.p = wsA + (g.wsA + (long long)other * g.G[1] * Hx + kx0 + in_line);
         gin.stride = Hx; gin.n = g.G[1];
         gout.p = wsB + (g.wsB + (long long)other * M1 * Hx + kx0 + line);
         gout.stride = Hx; gout.n = M1; gout.s0 = 0;
     } else if (AX == 2) {
-        gin.p = wsB + (g.wsB + (long long)other * Hx + kx0 + line);
+        gin.p = wsB + (g.wsB + (long long)other * Hx + kx0 + in_line);
         gin.stride = M1 * Hx; gin.n = g.G[2];
         gout.p = wsA + (g.wsA + (long long)other * Hx + kx0 + line);
         gout.stride = M1 * Hx; gout.n = g.W[2]; gout.s0 = g.s0[2];
     } else {
-        gin.p = wsA + (g.wsA + (long long)other * M1 * Hx + kx0 + line);
+        gin.p = wsA + (g.wsA + (long long)other * M1 * Hx + kx0 + in_line);
         gin.stride = Hx; gin.n = M1;
         gout.p = wsB + (g.wsB + (long long)other * g.W[1] * Hx + kx0 + line);
         gout.stride = Hx; gout.n = g.W[1]; gout.s0 = g.s0[1];
     }
+    gout.wrap = live && gout.s0 + gout.n > L;
+    if (!live) gout.n = 0;
     __syncthreads();   // twiddles
 
     if constexpr (MODE == 0) {
@@ -307,11 +374,10 @@ __global__ void __launch_bounds__(NT) k_col_fast(const GridDev* __restrict__ gri
         // -i D_comp T(kappa) rho-hat
         const int ky = other;
         const int fy = ky <= M1 / 2 ? ky : M1 - ky;
-        TabCol<T> tabc;   // a dead line reads column 0 (its results are never stored)
-        tabc.p = tab + (g.tab_off + (long long)fy * Hx + (live ? kx0 + line : 0));
+        FastTab<T> tabc;
+        tabc.p = tab + (g.tab_off + (long long)fy * Hx + kx0 + in_line);
         tabc.zst = g.Hy2 * Hx;
-        tabc.L = L;
-        using Tab = typename std::conditional<MODE == 3, TabGrad<T>, TabCol<T>>::type;
+        using Tab = typename std::conditional<MODE == 3, FastTabGrad<T>, FastTab<T>>::type;
         Tab tabf;
         if constexpr (MODE == 3) {
             const int kx = kx0 + line;
@@ -345,10 +411,7 @@ __global__ void __launch_bounds__(NT) k_col_fast(const GridDev* __restrict__ gri
 // A CTA holds NP complex lines, each packing two real rows (2p, 2p+1) of the
 // grid (two-for-one real transforms); buffer element (position, line) at
 // pos (NP + 1) + line (the padding keeps the row-wise passes conflict-free).
-template <typename T> struct NoIO {
-    __device__ C<T> ld(int) const { return mk<T>(0, 0); }
-    __device__ void st(int, C<T>) const {}
-};
+struct NoIO {};
 
 // xf: GMF rows -> half spectra along x, A[z][y][kx] (the layout of k_xf).
 // Load pass: the CTA's rows are one contiguous int64 range, read with
@@ -362,11 +425,12 @@ __global__ void __launch_bounds__(NT) k_xf_fast(const GridDev* __restrict__ grid
                                                 const int64_t* const* __restrict__ gmf,
                                                 const C<T>* __restrict__ tw_arena, C<T>* __restrict__ wsA,
                                                 int F) {
+    const unsigned block = begin_kernel();
     constexpr int L = P::L, PITCH = NP + 1, H = L / 2 + 1;
     extern __shared__ __align__(16) unsigned char smem_fast[];
     C<T>* buf = reinterpret_cast<C<T>*>(smem_fast);
     C<T>* tw = buf + L * PITCH;
-    const Chunk ch = chunks[blockIdx.x];
+    const Chunk ch = chunks[block];
     const GridDev& g = grids[ch.grid];
     const int G0 = g.G[0];
     const long long r_first = 2LL * ch.tile * NP;
@@ -414,13 +478,13 @@ __global__ void __launch_bounds__(NT) k_xf_fast(const GridDev* __restrict__ grid
         }
     }
     __syncthreads();
-    const NoIO<T> none;
-    fast_dif_stage<T, P, 0, NP, NT, false, false, NoIO<T>, NoIO<T>, PITCH>(buf, tw, none, none);
+    const NoIO none;
+    fast_dif_stage<T, P, 0, NP, NT, false, false, NoIO, NoIO, PITCH>(buf, tw, none, none);
     __syncthreads();
-    fast_dif_stage<T, P, 1, NP, NT, false, false, NoIO<T>, NoIO<T>, PITCH>(buf, tw, none, none);
+    fast_dif_stage<T, P, 1, NP, NT, false, false, NoIO, NoIO, PITCH>(buf, tw, none, none);
     __syncthreads();
     if constexpr (P::NST == 3) {
-        fast_dif_stage<T, P, 2, NP, NT, false, false, NoIO<T>, NoIO<T>, PITCH>(buf, tw, none, none);
+        fast_dif_stage<T, P, 2, NP, NT, false, false, NoIO, NoIO, PITCH>(buf, tw, none, none);
         __syncthreads();
     }
     C<T>* __restrict__ out = wsA + (g.wsA + r_first * H);
@@ -528,11 +592,12 @@ __global__ void __launch_bounds__(NT) k_xi_fast(const GridDev* __restrict__ grid
                                                 const C<T>* __restrict__ tw_arena,
                                                 const C<T>* __restrict__ wsB, void* const* __restrict__ phis,
                                                 int comp) {
+    const unsigned block = begin_kernel();
     constexpr int L = P::L, H = L / 2 + 1, PITCH = NP + 1;
     extern __shared__ __align__(16) unsigned char smem_fast[];
     C<T>* buf = reinterpret_cast<C<T>*>(smem_fast);
     C<T>* tw = buf + rows_index<P, PITCH>(L);   // past the padded line buffer (<= L PITCH + L / 2)
-    const Chunk ch = chunks[blockIdx.x];
+    const Chunk ch = chunks[block];
     const GridDev& g = grids[ch.grid];
     const int W0 = g.W[0];
     const long long r_first = 2LL * ch.tile * NP;
@@ -631,16 +696,22 @@ __device__ __forceinline__ void xy_load_plane(float2* buf, const int64_t* __rest
     for (int q = threadIdx.x >> 5; q < nl; q += NT / 32)
         for (int t = 2 * half + (threadIdx.x & 31); t < L; t += 32) buf[q * LS + t] = make_float2(0.f, 0.f);
 }
+// the plane's spectrum rows are H = L / 2 + 1 long: every offset is a constant
+// from the butterfly's first
 template <int L> struct XyOut {
     float2* __restrict__ p;          // B row ky = 0 of this plane, column 0
-    int Hx;
-    __device__ __forceinline__ void st(int col, int ky, float2 v) const { p[ky * Hx + col] = v; }
+    template <int R, int W> __device__ __forceinline__ void st(int col, int ky0, const float2* v) const {
+        constexpr int H = L / 2 + 1;
+        float2* __restrict__ q = p + (ky0 * H + col);
+#pragma unroll
+        for (int k = 0; k < R; ++k) q[k * W * H] = v[k];
+    }
 };
 
 // one DIF stage of the x lines (line-major, line storage LS complex apart,
 // butterflies on consecutive threads); nl lines (runtime)
-template <class P, int S_, int NT, bool IN_G, int LS, class GIN>
-__device__ __forceinline__ void xy_x_stage(float2* buf, const float2* __restrict__ tw, const GIN& gin, int nl) {
+template <class P, int S_, int NT, int LS>
+__device__ __forceinline__ void xy_x_stage(float2* buf, const float2* __restrict__ tw, int nl) {
     constexpr int R = P::radix(S_), S = P::inner(S_), L = P::L;
     constexpr int NB = L / R;
     constexpr int TWS = L / (R * S);
@@ -653,10 +724,7 @@ __device__ __forceinline__ void xy_x_stage(float2* buf, const float2* __restrict
         float2* lb = buf + line * LS;
         float2 v[R];
 #pragma unroll
-        for (int k = 0; k < R; ++k) {
-            if constexpr (IN_G) v[k] = gin.ld(line, base + k * S);
-            else v[k] = lb[base + k * S];
-        }
+        for (int k = 0; k < R; ++k) v[k] = lb[base + k * S];
         FastDft<float, -1, R>::run(v);
         if constexpr (S > 1) {
 #pragma unroll
@@ -690,11 +758,11 @@ __device__ __forceinline__ void xy_y_stage(float2* buf, const float2* __restrict
             for (int k = 1; k < R; ++k) v[k] = mul<float>(v[k], tw[lo * k * TWS]);
         }
         static_assert(!OUT_G || S == 1, "global output only from the last stage");
-        const int nat0 = OUT_G ? P::natural(base) : 0;
+        if constexpr (OUT_G) {
+            gout.template st<R, P::last_weight()>(col, P::natural(base), v);
+        } else {
 #pragma unroll
-        for (int k = 0; k < R; ++k) {
-            if constexpr (OUT_G) gout.st(col, nat0 + k * P::last_weight(), v[k]);
-            else buf[(base + k * S) * H + col] = v[k];
+            for (int k = 0; k < R; ++k) buf[(base + k * S) * H + col] = v[k];
         }
     }
 }
@@ -704,11 +772,12 @@ __global__ void __launch_bounds__(NT, 2) k_xy_fast(const GridDev* __restrict__ g
                                                    const int64_t* const* __restrict__ gmf,
                                                    const float2* __restrict__ tw_arena, float2* __restrict__ wsB,
                                                    int F) {
+    const unsigned block = begin_kernel();
     constexpr int L = P::L, H = L / 2 + 1;
     extern __shared__ __align__(16) unsigned char smem_fast[];
     float2* buf = reinterpret_cast<float2*>(smem_fast);   // L x H
     float2* tw = buf + L * H;
-    const Chunk ch = chunks[blockIdx.x];
+    const Chunk ch = chunks[block];
     const GridDev& g = grids[ch.grid];
     const int z = ch.tile;
     const int G0 = g.G[0], G1 = g.G[1];
@@ -718,13 +787,13 @@ __global__ void __launch_bounds__(NT, 2) k_xy_fast(const GridDev* __restrict__ g
     for (int t = threadIdx.x + 2 * nl * H; t < L * H; t += NT) buf[t] = make_float2(0.f, 0.f);
     xy_load_plane<L, NT, 2 * H>(buf, gmf[ch.grid] + (long long)z * G1 * G0, G0, G1, nl, pow2_neg<float>(F));
     __syncthreads();   // twiddles and the x lines
-    const NoIO<float> none;
-    xy_x_stage<P, 0, NT, false, 2 * H>(buf, tw, none, nl);
+    const NoIO none;
+    xy_x_stage<P, 0, NT, 2 * H>(buf, tw, nl);
     __syncthreads();
-    xy_x_stage<P, 1, NT, false, 2 * H>(buf, tw, none, nl);
+    xy_x_stage<P, 1, NT, 2 * H>(buf, tw, nl);
     if constexpr (P::NST == 3) {
         __syncthreads();
-        xy_x_stage<P, 2, NT, false, 2 * H>(buf, tw, none, nl);
+        xy_x_stage<P, 2, NT, 2 * H>(buf, tw, nl);
     }
     __syncthreads();
     // separation, one warp per line (its storage is touched by no other warp)
@@ -758,8 +827,7 @@ __global__ void __launch_bounds__(NT, 2) k_xy_fast(const GridDev* __restrict__ g
     }
     __syncthreads();
     XyOut<L> gout;
-    gout.p = wsB + (g.wsB + (long long)z * L * g.Hx);
-    gout.Hx = g.Hx;
+    gout.p = wsB + (g.wsB + (long long)z * L * H);
     xy_y_stage<P, 0, NT, false>(buf, tw, none);
     __syncthreads();
     if constexpr (P::NST == 3) {
@@ -788,8 +856,12 @@ __global__ void __launch_bounds__(NT, 2) k_xy_fast(const GridDev* __restrict__ g
 //    2p + 1 times 1/(M0 M1 M2).
 template <int L> struct YxIn {
     const float2* __restrict__ p;    // A row ky = 0 of this plane, column 0
-    int Hx;
-    __device__ __forceinline__ float2 ld(int col, int ky) const { return p[ky * Hx + col]; }
+    template <int R, int W> __device__ __forceinline__ void ld(int col, int ky0, float2* v) const {
+        constexpr int H = L / 2 + 1;
+        const float2* __restrict__ q = p + (ky0 * H + col);
+#pragma unroll
+        for (int k = 0; k < R; ++k) v[k] = q[k * W * H];
+    }
 };
 
 // one DIF stage of the y columns with DIR and an optional HBM input
@@ -806,10 +878,11 @@ __device__ __forceinline__ void yx_y_stage(float2* buf, const float2* __restrict
         const int hi = b / S, lo = b - hi * S;
         const int base = hi * R * S + lo;
         float2 v[R];
+        if constexpr (IN_G) {
+            gin.template ld<R, S>(col, base, v);
+        } else {
 #pragma unroll
-        for (int k = 0; k < R; ++k) {
-            if constexpr (IN_G) v[k] = gin.ld(col, base + k * S);
-            else v[k] = buf[(base + k * S) * H + col];
+            for (int k = 0; k < R; ++k) v[k] = buf[(base + k * S) * H + col];
         }
         FastDft<float, DIR, R>::run(v);
         if constexpr (S > 1) {
@@ -850,11 +923,17 @@ __device__ __forceinline__ void yx_x_stage(float2* buf, const float2* __restrict
         int ra, rb;
         yx_rows<P>(line, s0y, ra, rb);
         float2 v[R];
+        // element e lives at row ra's e or, from H on, at row rb's e - H: for the
+        // first stage (e = lo + k S, lo < S) mostly known at compile time
+        float2* const ea = buf + (ra * H + base);
+        float2* const eb = buf + (rb * H + base - H);
+        auto at = [&](int k) -> float2* {
+            if (S_ == 0 && k * S + S - 1 < H) return ea + k * S;
+            if (S_ == 0 && k * S >= H) return eb + k * S;
+            return (base + k * S < H ? ea : eb) + k * S;
+        };
 #pragma unroll
-        for (int k = 0; k < R; ++k) {
-            const int e = base + k * S;
-            v[k] = e < H ? buf[ra * H + e] : buf[rb * H + e - H];
-        }
+        for (int k = 0; k < R; ++k) v[k] = *at(k);
         FastDft<float, 1, R>::run(v);
         if constexpr (S > 1) {
 #pragma unroll
@@ -868,18 +947,14 @@ __device__ __forceinline__ void yx_x_stage(float2* buf, const float2* __restrict
             for (int k = 0; k < R; ++k) {
                 int w = P::natural(base) + k * P::last_weight() - s0x;
                 if (w < 0) w += L;
-                for (; w < W0; w += L) {
+                if (w < W0) {   // W0 <= L: these grids' windows are shorter than their transforms
                     r0[w] = v[k].x * norm;
                     if (has1) r0[W0 + w] = v[k].y * norm;
                 }
             }
         } else {
 #pragma unroll
-            for (int k = 0; k < R; ++k) {
-                const int e = base + k * S;
-                if (e < H) buf[ra * H + e] = v[k];
-                else buf[rb * H + e - H] = v[k];
-            }
+            for (int k = 0; k < R; ++k) *at(k) = v[k];
         }
     }
 }
@@ -889,19 +964,19 @@ __global__ void __launch_bounds__(NT, 2) k_yx_fast(const GridDev* __restrict__ g
                                                    const float2* __restrict__ tw_arena,
                                                    const float2* __restrict__ wsA, void* const* __restrict__ phis,
                                                    int comp) {
+    const unsigned block = begin_kernel();
     constexpr int L = P::L, H = L / 2 + 1;
     extern __shared__ __align__(16) unsigned char smem_fast[];
     float2* buf = reinterpret_cast<float2*>(smem_fast);   // L x H
     float2* tw = buf + L * H;
-    const Chunk ch = chunks[blockIdx.x];
+    const Chunk ch = chunks[block];
     const GridDev& g = grids[ch.grid];
     const int zw = ch.tile;
     const int W0 = g.W[0], W1 = g.W[1];
     const int nl = (W1 + 1) / 2;
     for (int t = threadIdx.x; t < L; t += NT) tw[t] = tw_arena[g.fx.tw_off + t];
     YxIn<L> gin;
-    gin.p = wsA + (g.wsA + (long long)zw * L * g.Hx);
-    gin.Hx = g.Hx;
+    gin.p = wsA + (g.wsA + (long long)zw * L * H);
     __syncthreads();   // twiddles
     yx_y_stage<P, 0, NT, true, 1>(buf, tw, gin);
     __syncthreads();

@@ -28,7 +28,8 @@ __global__ void __launch_bounds__(256) k_gas_init(LevelDev L, const GridDev* __r
                            const double* const* __restrict__ gas,
                            const double* const* __restrict__ pgas, int64_t* const* __restrict__ gmf,
                            const Chunk* __restrict__ chunks, int F) {
-    const Chunk c = chunks[blockIdx.x];
+    const unsigned block = begin_kernel();
+    const Chunk c = chunks[block];
     const GridDev& g = L.g[c.grid];
     const int G0 = g.G[0], G1 = g.G[1];
     const int nrows = G1 * g.G[2];
@@ -349,8 +350,7 @@ __device__ __forceinline__ bool particle_of_level(const LevelDev& L, const Parti
 
 // the first slot of this CTA: in the caller's order CTA after CTA; in bin order
 // spread over the bins (deposit_stride, coprime to the number of CTAs)
-__device__ __forceinline__ long long first_slot(const Particles& P) {
-    unsigned b = blockIdx.x;
+__device__ __forceinline__ long long first_slot(const Particles& P, unsigned b) {
     if (P.stride) b = (unsigned)((unsigned long long)b * P.stride % gridDim.x);
     return (long long)b * kDepThreads;
 }
@@ -360,8 +360,9 @@ __global__ void __launch_bounds__(kDepThreads, APM_DEP_MIN_CTAS) k_deposit(Level
                                                  double box, int F,
                                                  int64_t* const* __restrict__ gmf,
                                                  unsigned* __restrict__ status) {
+    const unsigned block = begin_kernel();
     __shared__ WarpCharges charges[kDepThreads / 32];
-    const long long i = first_slot(P) + threadIdx.x;
+    const long long i = first_slot(P, block) + threadIdx.x;
     long long X[3] = {0, 0, 0}, M = 0;
     bool outside = false;
     const bool ok = i < P.n && particle_of_level(L, P, i, half_dt, box, F, X, &M, &outside, status);
@@ -375,8 +376,9 @@ __global__ void __launch_bounds__(kDepThreads, APM_DEP_MIN_CTAS) k_deposit(Level
 __global__ void __launch_bounds__(kDepThreads, APM_DEP_MIN_CTAS) k_deposit_levels(
     const LevelDev* __restrict__ levels, int nl, Particles P, double half_dt, double box, int F,
     int64_t* const* const* __restrict__ gmfs, unsigned* __restrict__ status) {
+    const unsigned block = begin_kernel();
     __shared__ WarpCharges charges[kDepThreads / 32];
-    const long long i = first_slot(P) + threadIdx.x;
+    const long long i = first_slot(P, block) + threadIdx.x;
     long long X[3] = {0, 0, 0}, M = 0;
     bool outside = false, ok = false;
     if (i < P.n) ok = particle_fixed(levels[0], P, P.at(i), half_dt, box, F, X, &M, &outside, status);
@@ -393,8 +395,7 @@ cudaError_t launch_gas_init(const LevelDev& L, const GridDev* parent_grids,
                             int64_t* const* gmf, const Chunk* chunks, int n_chunks,
                             int F, cudaStream_t s) {
     if (n_chunks <= 0) return cudaSuccess;
-    k_gas_init<<<n_chunks, 256, 0, s>>>(L, parent_grids, gas, pgas, gmf, chunks, F);
-    return cudaGetLastError();
+    return launch_kernel(k_gas_init, n_chunks, 256, 0, s, L, parent_grids, gas, pgas, gmf, chunks, F);
 }
 
 // In bin order the CTAs that run together would add into the same few cells
@@ -423,8 +424,7 @@ cudaError_t launch_deposit(const LevelDev& L, const Particles& P, double half_dt
                            int F, int64_t* const* gmf, unsigned* status, cudaStream_t s) {
     if (P.n <= 0) return cudaSuccess;
     unsigned blocks = (unsigned)((P.n + kDepThreads - 1) / kDepThreads);
-    k_deposit<<<blocks, kDepThreads, 0, s>>>(L, deposit_order(P, blocks), half_dt, box, F, gmf, status);
-    return cudaGetLastError();
+    return launch_kernel(k_deposit, blocks, kDepThreads, 0, s, L, deposit_order(P, blocks), half_dt, box, F, gmf, status);
 }
 
 cudaError_t launch_deposit_levels(const LevelDev* levels, int nl, const Particles& P, double half_dt,
@@ -432,8 +432,7 @@ cudaError_t launch_deposit_levels(const LevelDev* levels, int nl, const Particle
                                   cudaStream_t s) {
     if (P.n <= 0 || nl <= 0) return cudaSuccess;
     unsigned blocks = (unsigned)((P.n + kDepThreads - 1) / kDepThreads);
-    k_deposit_levels<<<blocks, kDepThreads, 0, s>>>(levels, nl, deposit_order(P, blocks), half_dt, box, F, gmfs, status);
-    return cudaGetLastError();
+    return launch_kernel(k_deposit_levels, blocks, kDepThreads, 0, s, levels, nl, deposit_order(P, blocks), half_dt, box, F, gmfs, status);
 }
 
 }  // namespace apm

@@ -30,7 +30,8 @@ __global__ void __launch_bounds__(256) k_kick_drift(long long n, double* __restr
                                                     double* __restrict__ z, double* __restrict__ vx,
                                                     double* __restrict__ vy, double* __restrict__ vz,
                                                     const T* __restrict__ acc, double dt) {
-    const long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x;
+    const unsigned block = begin_kernel();
+    const long long i = (long long)block * blockDim.x + threadIdx.x;
     const bool live = i < n;
     const long long p = live ? i : n - 1;   // a thread past the end redoes the last particle, unstored
     // all nine loads first (the arrays are distinct), then the updates
@@ -78,8 +79,7 @@ cudaError_t launch_kick_drift(long long n, double* x, double* y, double* z, doub
                               const void* acc, double dt, cudaStream_t s) {
     if (n <= 0) return cudaSuccess;
     const unsigned blocks = (unsigned)((n + 255) / 256);
-    k_kick_drift<T><<<blocks, 256, 0, s>>>(n, x, y, z, vx, vy, vz, reinterpret_cast<const T*>(acc), dt);
-    return cudaGetLastError();
+    return launch_kernel(k_kick_drift<T>, blocks, 256, 0, s, n, x, y, z, vx, vy, vz, reinterpret_cast<const T*>(acc), dt);
 }
 
 template cudaError_t launch_kick_drift<float>(long long, double*, double*, double*, double*, double*, double*,

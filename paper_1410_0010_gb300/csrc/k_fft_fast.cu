@@ -54,17 +54,15 @@ cudaError_t launch_one(const FftArgs& a, const int64_t* const* gmf, void* const*
         constexpr auto kern = K::get();
         const auto* tw = (const C<FT>*)a.tw;
         if constexpr (kMode == kFastXf)
-            kern<<<a.n_chunks, K::NT, K::smem, s>>>(a.g, a.chunks, gmf, tw, (C<FT>*)a.wsA, a.F);
+            return launch_kernel(kern, a.n_chunks, K::NT, K::smem, s, a.g, a.chunks, gmf, tw, (C<FT>*)a.wsA, a.F);
         else if constexpr (kMode == kFastXy)
-            kern<<<a.n_chunks, K::NT, K::smem, s>>>(a.g, a.chunks, gmf, tw, (C<FT>*)a.wsB, a.F);
+            return launch_kernel(kern, a.n_chunks, K::NT, K::smem, s, a.g, a.chunks, gmf, tw, (C<FT>*)a.wsB, a.F);
         else if constexpr (kMode == kFastXi)
-            kern<<<a.n_chunks, K::NT, K::smem, s>>>(a.g, a.chunks, tw, (const C<FT>*)a.wsB, phis, a.comp);
+            return launch_kernel(kern, a.n_chunks, K::NT, K::smem, s, a.g, a.chunks, tw, (const C<FT>*)a.wsB, phis, a.comp);
         else if constexpr (kMode == kFastYx)
-            kern<<<a.n_chunks, K::NT, K::smem, s>>>(a.g, a.chunks, tw, (const C<FT>*)a.wsA, phis, a.comp);
+            return launch_kernel(kern, a.n_chunks, K::NT, K::smem, s, a.g, a.chunks, tw, (const C<FT>*)a.wsA, phis, a.comp);
         else
-            kern<<<a.n_chunks, K::NT, K::smem, s>>>(a.g, a.chunks, tw, (const FT*)a.tab, (C<FT>*)a.wsA,
-                                                    (C<FT>*)a.wsB, a.comp);
-        return cudaGetLastError();
+            return launch_kernel(kern, a.n_chunks, K::NT, K::smem, s, a.g, a.chunks, tw, (const FT*)a.tab, (C<FT>*)a.wsA, (C<FT>*)a.wsB, a.comp);
     }
     return cudaErrorInvalidValue;
 }

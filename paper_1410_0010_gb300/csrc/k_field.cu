@@ -116,7 +116,8 @@ __global__ void __launch_bounds__(kAccThreads, AccMinCtas<T>::march) k_accel(
     LevelDev L, const GridDev* __restrict__ pgrids, const void* const* __restrict__ phis_p,
     const void* const* __restrict__ pphi_p, const void* const* __restrict__ pacc_p, void* const* __restrict__ phi_p,
     void* const* __restrict__ acc_p, const Chunk* __restrict__ chunks, int zs) {
-    const Chunk ch = chunks[blockIdx.x];
+    const unsigned block = begin_kernel();
+    const Chunk ch = chunks[block];
     const GridDev& g = L.g[ch.grid];
     const int nbx = g.acc_nb[0], ncol = nbx * g.acc_nb[1], nbz = g.acc_nb[2];
     const int ncc = (ncol + kAccThreads - 1) / kAccThreads;   // CTAs across the columns
@@ -410,7 +411,8 @@ template <typename T>
 __global__ void __launch_bounds__(256) k_interp(LevelDev L, LevelDev F, int has_finer, Particles P,
                                                 double half_dt, const void* const* __restrict__ acc_p,
                                                 T* __restrict__ out) {
-    const long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x;
+    const unsigned block = begin_kernel();
+    const long long i = (long long)block * blockDim.x + threadIdx.x;
     if (i >= P.n) return;
     const long long p = P.at(i);
     long long X[3];
@@ -444,7 +446,8 @@ template <typename T>
 __global__ void __launch_bounds__(kIntThreads, APM_INT_MIN_CTAS) k_interp_levels(const LevelDev* __restrict__ levels, int nl, Particles P,
                                                        double half_dt, const void* const* const* __restrict__ accs,
                                                        T* __restrict__ out) {
-    const long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x;
+    const unsigned block = begin_kernel();
+    const long long i = (long long)block * blockDim.x + threadIdx.x;
     if (i >= P.n) return;
     const long long p = P.at(i);
     long long X[3];
@@ -476,7 +479,8 @@ __global__ void __launch_bounds__(kAccThreads, AccMinCtas<T>::value) k_accel_var
     LevelDev L, const GridDev* __restrict__ pgrids, const void* const* __restrict__ phis_p,
     const void* const* __restrict__ pphi_p, const void* const* __restrict__ pacc_p,
     void* const* __restrict__ phi_p, void* const* __restrict__ acc_p, const Chunk* __restrict__ chunks) {
-    const Chunk ch = chunks[blockIdx.x];
+    const unsigned block = begin_kernel();
+    const Chunk ch = chunks[block];
     const GridDev& g = L.g[ch.grid];
     const int E0 = g.N[0] + 2, E1 = g.N[1] + 2, E2 = g.N[2] + 2;
     const unsigned ncell = (unsigned)E0 * E1 * E2;
@@ -659,10 +663,9 @@ cudaError_t launch_accel(const LevelDev& L, const GridDev* parent_grids, const v
                          cudaStream_t s) {
     if (n_chunks <= 0) return cudaSuccess;
     if (pphi)   // every grid of a level that gets parent fields has a parent
-        k_accel<T, true><<<n_chunks, kAccThreads, 0, s>>>(L, parent_grids, phis, pphi, pacc, phi, acc, chunks, zs);
+        return launch_kernel(k_accel<T, true>, n_chunks, kAccThreads, 0, s, L, parent_grids, phis, pphi, pacc, phi, acc, chunks, zs);
     else
-        k_accel<T, false><<<n_chunks, kAccThreads, 0, s>>>(L, parent_grids, phis, pphi, pacc, phi, acc, chunks, zs);
-    return cudaGetLastError();
+        return launch_kernel(k_accel<T, false>, n_chunks, kAccThreads, 0, s, L, parent_grids, phis, pphi, pacc, phi, acc, chunks, zs);
 }
 
 template <typename T>
@@ -672,12 +675,9 @@ cudaError_t launch_accel_var(const LevelDev& L, const GridDev* parent_grids, con
                                cudaStream_t s) {
     if (n_chunks <= 0) return cudaSuccess;
     if (grad == APM_GRAD_FD4)
-        k_accel_var<T, APM_GRAD_FD4><<<n_chunks, kAccThreads, 0, s>>>(L, parent_grids, phis, pphi, pacc, phi, acc,
-                                                                      chunks);
+        return launch_kernel(k_accel_var<T, APM_GRAD_FD4>, n_chunks, kAccThreads, 0, s, L, parent_grids, phis, pphi, pacc, phi, acc, chunks);
     else
-        k_accel_var<T, APM_GRAD_SPECTRAL><<<n_chunks, kAccThreads, 0, s>>>(L, parent_grids, phis, pphi, pacc, phi,
-                                                                           acc, chunks);
-    return cudaGetLastError();
+        return launch_kernel(k_accel_var<T, APM_GRAD_SPECTRAL>, n_chunks, kAccThreads, 0, s, L, parent_grids, phis, pphi, pacc, phi, acc, chunks);
 }
 
 template <typename T>
@@ -686,8 +686,7 @@ cudaError_t launch_interp(const LevelDev& L, const LevelDev* finer, const Partic
     if (P.n <= 0) return cudaSuccess;
     unsigned blocks = (unsigned)((P.n + 255) / 256);
     LevelDev F = finer ? *finer : L;
-    k_interp<T><<<blocks, 256, 0, s>>>(L, F, finer ? 1 : 0, P, half_dt, acc, reinterpret_cast<T*>(out));
-    return cudaGetLastError();
+    return launch_kernel(k_interp<T>, blocks, 256, 0, s, L, F, finer ? 1 : 0, P, half_dt, acc, reinterpret_cast<T*>(out));
 }
 
 template <typename T>
@@ -695,8 +694,7 @@ cudaError_t launch_interp_levels(const LevelDev* levels, int nl, const Particles
                                  const void* const* const* accs, void* out, cudaStream_t s) {
     if (P.n <= 0 || nl <= 0) return cudaSuccess;
     unsigned blocks = (unsigned)((P.n + kIntThreads - 1) / kIntThreads);
-    k_interp_levels<T><<<blocks, kIntThreads, 0, s>>>(levels, nl, P, half_dt, accs, reinterpret_cast<T*>(out));
-    return cudaGetLastError();
+    return launch_kernel(k_interp_levels<T>, blocks, kIntThreads, 0, s, levels, nl, P, half_dt, accs, reinterpret_cast<T*>(out));
 }
 
 template cudaError_t launch_accel<float>(const LevelDev&, const GridDev*, const void* const*,

@@ -43,7 +43,8 @@ __device__ __forceinline__ int bin_of(double x, double v, const BinScale& s) {
 // of 1 M, whose core bins hold up to 1e5 particles, 141 -> 94)
 __global__ void __launch_bounds__(256) k_order_bins(Particles P, BinScale s, unsigned* __restrict__ count,
                                                     unsigned* __restrict__ key, unsigned* __restrict__ rank) {
-    const long long p = blockIdx.x * (long long)blockDim.x + threadIdx.x;
+    const unsigned block = begin_kernel();
+    const long long p = (long long)block * blockDim.x + threadIdx.x;
     const bool live = p < P.n;
     unsigned k = 0xffffffffu;
     if (live) {
@@ -65,8 +66,9 @@ __global__ void __launch_bounds__(256) k_order_bins(Particles P, BinScale s, uns
 // to sums[chunk]
 __global__ void __launch_bounds__(1024) k_order_scan_local(unsigned* __restrict__ count, int nbins,
                                                            unsigned* __restrict__ sums) {
+    const unsigned block = begin_kernel();
     __shared__ unsigned warp_tot[32];
-    const int base = blockIdx.x * kScanChunk + 2 * threadIdx.x;
+    const int base = block * kScanChunk + 2 * threadIdx.x;
     const unsigned a = base < nbins ? count[base] : 0u;
     const unsigned b = base + 1 < nbins ? count[base + 1] : 0u;
     const unsigned t = a + b;
@@ -93,11 +95,12 @@ __global__ void __launch_bounds__(1024) k_order_scan_local(unsigned* __restrict_
     const unsigned before = v - t + (warp > 0 ? warp_tot[warp - 1] : 0u);   // exclusive prefix of a
     if (base < nbins) count[base] = before;
     if (base + 1 < nbins) count[base + 1] = before + a;
-    if (threadIdx.x == blockDim.x - 1) sums[blockIdx.x] = before + t;
+    if (threadIdx.x == blockDim.x - 1) sums[block] = before + t;
 }
 
 // exclusive scan of the chunk totals (at most 1024 chunks) in place, one CTA
 __global__ void __launch_bounds__(1024) k_order_scan_sums(unsigned* __restrict__ sums, int n) {
+    begin_kernel();
     __shared__ unsigned warp_tot[32];
     const unsigned t = threadIdx.x < (unsigned)n ? sums[threadIdx.x] : 0u;
     unsigned v = t;
@@ -127,7 +130,8 @@ __global__ void __launch_bounds__(256) k_order_scatter(long long n, const unsign
                                                        const unsigned* __restrict__ rank,
                                                        const unsigned* __restrict__ count,
                                                        const unsigned* __restrict__ sums, int* __restrict__ perm) {
-    const long long p = blockIdx.x * (long long)blockDim.x + threadIdx.x;
+    const unsigned block = begin_kernel();
+    const long long p = (long long)block * blockDim.x + threadIdx.x;
     if (p >= n) return;
     const unsigned k = key[p];
     const unsigned slot = sums[k / kScanChunk] + count[k] + rank[p];
@@ -168,11 +172,12 @@ cudaError_t launch_order(const LevelDev& root, const Particles& P, double half_d
     cudaError_t e = cudaMemsetAsync(count, 0, (size_t)nbins * sizeof(unsigned), s);
     if (e != cudaSuccess) return e;
     const unsigned blocks = (unsigned)((P.n + 255) / 256);
-    k_order_bins<<<blocks, 256, 0, s>>>(P, bin_scale(root, half_dt, shift, nb), count, key, rank);
-    k_order_scan_local<<<nchunks, 1024, 0, s>>>(count, nbins, sums);
-    k_order_scan_sums<<<1, 1024, 0, s>>>(sums, nchunks);
-    k_order_scatter<<<blocks, 256, 0, s>>>(P.n, key, rank, count, sums, perm);
-    return cudaGetLastError();
+    if ((e = launch_kernel(k_order_bins, blocks, 256, 0, s, P, bin_scale(root, half_dt, shift, nb), count, key,
+                           rank)) != cudaSuccess ||
+        (e = launch_kernel(k_order_scan_local, nchunks, 1024, 0, s, count, nbins, sums)) != cudaSuccess ||
+        (e = launch_kernel(k_order_scan_sums, 1, 1024, 0, s, sums, nchunks)) != cudaSuccess)
+        return e;
+    return launch_kernel(k_order_scatter, blocks, 256, 0, s, P.n, key, rank, count, sums, perm);
 }
 
 }  // namespace apm
