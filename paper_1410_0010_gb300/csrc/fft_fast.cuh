@@ -95,7 +95,7 @@ __device__ __forceinline__ void fast_dif_stage(C<T>* buf, const C<T>* __restrict
     constexpr int R = P::radix(S_), S = P::inner(S_), L = P::L;
     constexpr int NB = L / R, ITEMS = NB * TX, TRIPS = (ITEMS + NT - 1) / NT;
     constexpr int TWS = L / (R * S);
-#pragma unroll
+#pragma unroll 1
     for (int it = 0; it < TRIPS; ++it) {
         const int i = threadIdx.x + it * NT;
         if (ITEMS % NT != 0 && i >= ITEMS) break;
@@ -137,7 +137,7 @@ __device__ __forceinline__ void fast_dit_stage(C<T>* buf, const C<T>* __restrict
     constexpr int R = P::radix(S_), S = P::inner(S_), L = P::L;
     constexpr int NB = L / R, ITEMS = NB * TX, TRIPS = (ITEMS + NT - 1) / NT;
     constexpr int TWS = L / (R * S);
-#pragma unroll
+#pragma unroll 1
     for (int it = 0; it < TRIPS; ++it) {
         const int i = threadIdx.x + it * NT;
         if (ITEMS % NT != 0 && i >= ITEMS) break;
@@ -173,7 +173,7 @@ __device__ __forceinline__ void fast_mid_stage(C<T>* buf, const TAB& tabf) {
     constexpr int SL = P::NST - 1;
     constexpr int R = P::radix(SL), L = P::L;
     constexpr int NB = L / R, ITEMS = NB * TX, TRIPS = (ITEMS + NT - 1) / NT;
-#pragma unroll
+#pragma unroll 1
     for (int it = 0; it < TRIPS; ++it) {
         const int i = threadIdx.x + it * NT;
         if (ITEMS % NT != 0 && i >= ITEMS) break;
