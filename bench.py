@@ -277,7 +277,7 @@ def ncu_label(name):
     return {"gas_init": "gas_init", "deposit_levels": "tsc_deposit", "deposit": "tsc_deposit",
             "xf": "fft_x_fwd", "xf_fast": "fft_x_fwd", "xy_fast": "fft_x_fwd",
             "xi": "fft_x_inv", "xi_fast": "fft_x_inv", "yx_fast": "fft_x_inv",
-            "accel": "accel_carry", "accel_var": "accel_carry", "interp_levels": "tsc_interp",
+            "accel": "accel_carry", "accel_var": "accel_carry", "accel_spectral": "accel_carry", "interp_levels": "tsc_interp",
             "interp": "tsc_interp"}.get(base)
 
 

@@ -976,7 +976,7 @@ apm_status apm_set_hierarchy(apm_ctx* c, const apm_grid* grids, int32_t n) {
             for (long long t = 0; t < (grows + g.rows_gas - 1) / g.rows_gas; ++t) gas.push_back({k, (int)t});
             const long long nblocks = (long long)g.acc_nb[0] * g.acc_nb[1] * g.acc_nb[2];
             const long long ncc = ((long long)g.acc_nb[0] * g.acc_nb[1] + kAccThreads - 1) / kAccThreads;
-            const long long nch = cfg.gradient == APM_GRAD_FD2 ? ncc * ((g.acc_nb[2] + L.acc_zs - 1) / L.acc_zs)
+            const long long nch = cfg.gradient != APM_GRAD_FD4 ? ncc * ((g.acc_nb[2] + L.acc_zs - 1) / L.acc_zs)
                                                                : (nblocks + kAccBlocksPerCta - 1) / kAccBlocksPerCta;
             for (long long t = 0; t < nch; ++t) acc.push_back({k, (int)t});
         }
@@ -1636,9 +1636,9 @@ apm_status apm_accel(apm_ctx* c, int32_t level, const void* const* phi_short,
         else
             e = c->cfg.precision == APM_FP64
                 ? launch_accel_var<double>(L.dev, pgrids, (const void* const*)d_phis, (const void* const*)d_pphi,
-                                             (const void* const*)d_pacc, d_phi, d_acc, ch, nch, grad, s)
+                                             (const void* const*)d_pacc, d_phi, d_acc, ch, nch, grad, L.acc_zs, s)
                 : launch_accel_var<float>(L.dev, pgrids, (const void* const*)d_phis, (const void* const*)d_pphi,
-                                            (const void* const*)d_pacc, d_phi, d_acc, ch, nch, grad, s);
+                                            (const void* const*)d_pacc, d_phi, d_acc, ch, nch, grad, L.acc_zs, s);
         if (e != cudaSuccess) return APM_E_CUDA;
     }
     return APM_OK;

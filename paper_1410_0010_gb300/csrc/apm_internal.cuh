@@ -274,12 +274,11 @@ struct RowWalk {
     }
 };
 
-// 2x2x2 output blocks per CTA of the four-point and spectral acceleration
-// kernel (flat ranges of the grid's blocks, x fastest, so every thread gets the
+// 2x2x2 output blocks per CTA of the four-point acceleration kernel (flat ranges of the grid's blocks, x fastest, so every thread gets the
 // same count)
 constexpr int kAccBlocksPerCta = 512;
-// threads of an acceleration CTA; the two-point kernel gives each one (x, y)
-// column of blocks and marches through up to kAccMarch blocks of it (4 to 16
+// threads of an acceleration CTA; the two-point and spectral kernels give each one (x, y)
+// column of blocks and march through up to kAccMarch blocks of it (4 to 16
 // measure alike on large levels; the host halves it while a level would leave
 // SMs idle)
 #ifndef APM_ACC_THREADS
@@ -666,11 +665,12 @@ cudaError_t launch_fft_fast(int kernel, bool f64, int L, const FftArgs& a, const
 cudaError_t configure_fft_fast(int kernel, bool f64, int L);
 
 // accelerations + parent carry for the four-point and spectral gradients (the
-// two-point one runs launch_accel), on flat ranges of blocks
+// two-point one runs launch_accel): the four-point one on flat ranges of blocks,
+// the spectral one on launch_accel's columns
 template <typename T>
 cudaError_t launch_accel_var(const LevelDev& L, const GridDev* parent_grids, const void* const* phis,
                                const void* const* pphi, const void* const* pacc, void* const* phi,
-                               void* const* acc, const Chunk* chunks, int n_chunks, int grad,
+                               void* const* acc, const Chunk* chunks, int n_chunks, int grad, int zs,
                                cudaStream_t s);
 
 // FD accelerations + parent carry (two-point; a chunk is kAccThreads columns of

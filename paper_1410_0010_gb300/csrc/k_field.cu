@@ -111,6 +111,77 @@ __device__ __forceinline__ void lerp_plane(const T* __restrict__ f, unsigned bas
     out[1][1] = b * x01 + a * x11;
 }
 
+// this thread's column of blocks of a marching kernel: blocks [bz0, bz1) at
+// output cells ex0, ey0; false: none
+struct AccColumn {
+    int ex0, ey0, bz0, bz1;
+    __device__ __forceinline__ bool start(const GridDev& g, int tile, int zs) {
+        const int nbx = g.acc_nb[0], ncol = nbx * g.acc_nb[1];
+        const int ncc = (ncol + kAccThreads - 1) / kAccThreads;   // CTAs across the columns
+        const int seg = tile / ncc;
+        const int col = (tile - seg * ncc) * kAccThreads + (int)threadIdx.x;
+        if (col >= ncol) return false;
+        const int by = col / nbx;
+        ex0 = 2 * (col - by * nbx) - g.acc_sh[0];
+        ey0 = 2 * by - g.acc_sh[1];
+        bz0 = seg * zs;
+        bz1 = min(g.acc_nb[2], bz0 + zs);
+        return true;
+    }
+};
+// the parent's phi (0) and accelerations (1-3) along that column: the planes
+// below (yp) and above (yn) a block, interpolated in x and y
+template <typename T, bool CARRY> struct AccCarry {
+    const T* pf[4];
+    int P0;
+    unsigned P01, pbase;
+    T yp[4][2][2], yn[4][2][2];
+    __device__ __forceinline__ bool start(const LevelDev& L, const GridDev& g, const GridDev* __restrict__ pgrids,
+                                          const void* const* __restrict__ pphi_p,
+                                          const void* const* __restrict__ pacc_p, const AccColumn& c) {
+        if (!CARRY) return true;
+        const GridDev& p = pgrids[g.parent];
+        P0 = p.N[0] + 2;
+        P01 = (unsigned)P0 * (p.N[1] + 2);
+        const unsigned pn = P01 * (p.N[2] + 2);
+        pf[0] = reinterpret_cast<const T*>(pphi_p[g.parent]);
+#pragma unroll
+        for (int j = 0; j < 3; ++j) pf[1 + j] = reinterpret_cast<const T*>(pacc_p[g.parent]) + (size_t)j * pn;
+        // parent cell k of the odd level cell (2k+1) of each pair
+        const long long kx = ((g.start[0] + c.ex0 - 1) - 1) >> 1, ky = ((g.start[1] + c.ey0 - 1) - 1) >> 1;
+        const long long kz = ((g.start[2] + 2 * c.bz0 - g.acc_sh[2] - 1) - 1) >> 1;
+        pbase = (unsigned)(kx - p.start[0] + 1) + (unsigned)(ky - p.start[1] + 1) * (unsigned)P0 +
+                (unsigned)(kz - p.start[2] + 1) * P01;
+        // the blocks' parent cells: pbase .. pbase + 1 + P0 + (bz1 - bz0) P01
+        if (!APM_IN_BOUNDS((long long)pbase + 1 + P0 + (long long)(c.bz1 - c.bz0) * P01, pn, L.status)) return false;
+#pragma unroll
+        for (int j = 0; j < 4; ++j) lerp_plane(pf[j], pbase, P0, yp[j]);
+        return true;
+    }
+    __device__ __forceinline__ void next() {   // the plane above the block
+        if (!CARRY) return;
+        pbase += P01;
+#pragma unroll
+        for (int j = 0; j < 4; ++j) lerp_plane(pf[j], pbase, P0, yn[j]);
+    }
+    // field j of the block's cells (0, b, z), (1, b, z)
+    __device__ __forceinline__ void add(int j, int z, int b, T& v0, T& v1) const {
+        if (!CARRY) return;
+        const T a = z == 0 ? (T)0.75 : (T)0.25, d = z == 0 ? (T)0.25 : (T)0.75;
+        v0 += a * yp[j][b][0] + d * yn[j][b][0];
+        v1 += a * yp[j][b][1] + d * yn[j][b][1];
+    }
+    __device__ __forceinline__ void up() {
+        if (!CARRY) return;
+#pragma unroll
+        for (int j = 0; j < 4; ++j)
+#pragma unroll
+            for (int b = 0; b < 2; ++b)
+#pragma unroll
+                for (int a = 0; a < 2; ++a) yp[j][b][a] = yn[j][b][a];
+    }
+};
+
 template <typename T, bool CARRY>
 __global__ void __launch_bounds__(kAccThreads, AccMinCtas<T>::march) k_accel(
     LevelDev L, const GridDev* __restrict__ pgrids, const void* const* __restrict__ phis_p,
@@ -119,14 +190,9 @@ __global__ void __launch_bounds__(kAccThreads, AccMinCtas<T>::march) k_accel(
     const unsigned block = begin_kernel();
     const Chunk ch = chunks[block];
     const GridDev& g = L.g[ch.grid];
-    const int nbx = g.acc_nb[0], ncol = nbx * g.acc_nb[1], nbz = g.acc_nb[2];
-    const int ncc = (ncol + kAccThreads - 1) / kAccThreads;   // CTAs across the columns
-    const int seg = ch.tile / ncc;
-    const int col = (ch.tile - seg * ncc) * kAccThreads + (int)threadIdx.x;
-    if (col >= ncol) return;
-    const int by = col / nbx;
-    const int ex0 = 2 * (col - by * nbx) - g.acc_sh[0], ey0 = 2 * by - g.acc_sh[1];
-    const int bz0 = seg * zs, bz1 = min(nbz, bz0 + zs);
+    AccColumn col;
+    if (!col.start(g, ch.tile, zs)) return;
+    const int ex0 = col.ex0, ey0 = col.ey0;
     const int E0 = g.N[0] + 2, E1 = g.N[1] + 2, E2 = g.N[2] + 2;
     const unsigned ncell = (unsigned)E0 * E1 * E2;
     const int W0 = g.W[0], W1 = g.W[1], W2 = g.W[2];
@@ -153,30 +219,10 @@ __global__ void __launch_bounds__(kAccThreads, AccMinCtas<T>::march) k_accel(
     // cells written: x = ex0 + a, y = ey0 + b
     const bool wx0 = ex0 >= 0 && ex0 < E0, wx1 = ex0 + 1 < E0;
     const bool wy0 = ey0 >= 0 && ey0 < E1, wy1 = ey0 + 1 < E1;
-    // parent: cell k of the odd level cell (2k+1) of each pair
-    const T *pf[4] = {nullptr, nullptr, nullptr, nullptr};
-    int P0 = 0;
-    unsigned P01 = 0, pn = 0, pbase = 0;
-    T yp[4][2][2];   // phi and the accelerations on the parent plane below the block
-    if (CARRY) {
-        const GridDev& p = pgrids[g.parent];
-        P0 = p.N[0] + 2;
-        P01 = (unsigned)P0 * (p.N[1] + 2);
-        pn = P01 * (p.N[2] + 2);
-        pf[0] = reinterpret_cast<const T*>(pphi_p[g.parent]);
-#pragma unroll
-        for (int j = 0; j < 3; ++j) pf[1 + j] = reinterpret_cast<const T*>(pacc_p[g.parent]) + (size_t)j * pn;
-        const long long kx = ((g.start[0] + ex0 - 1) - 1) >> 1, ky = ((g.start[1] + ey0 - 1) - 1) >> 1;
-        const long long kz = ((g.start[2] + 2 * bz0 - g.acc_sh[2] - 1) - 1) >> 1;
-        pbase = (unsigned)(kx - p.start[0] + 1) + (unsigned)(ky - p.start[1] + 1) * (unsigned)P0 +
-                (unsigned)(kz - p.start[2] + 1) * P01;
-        // the blocks' parent cells: pbase .. pbase + 1 + P0 + (bz1 - bz0) P01
-        if (!APM_IN_BOUNDS((long long)pbase + 1 + P0 + (long long)(bz1 - bz0) * P01, pn, L.status)) return;
-#pragma unroll
-        for (int j = 0; j < 4; ++j) lerp_plane(pf[j], pbase, P0, yp[j]);
-    }
+    AccCarry<T, CARRY> carry;
+    if (!carry.start(L, g, pgrids, pphi_p, pacc_p, col)) return;
     auto plane = [&](int k) { return phis + sz * (unsigned)min(max(k, 0), W2 - 1); };
-    int ez0 = 2 * bz0 - g.acc_sh[2];
+    int ez0 = 2 * col.bz0 - g.acc_sh[2];
     T z0[2][2];   // centres of the plane below the block
     {
         const T* __restrict__ f = plane(ez0);
@@ -187,23 +233,14 @@ __global__ void __launch_bounds__(kAccThreads, AccMinCtas<T>::march) k_accel(
     }
     AccPlane<T> p1 = load_acc_plane(plane(ez0 + 1), yrow, ex0, xi, vload);
 #pragma unroll 1
-    for (int bz = bz0; bz < bz1; ++bz, ez0 += 2) {
+    for (int bz = col.bz0; bz < col.bz1; ++bz, ez0 += 2) {
         const AccPlane<T> p2 = load_acc_plane(plane(ez0 + 2), yrow, ex0, xi, vload);
         const AccPlane<T> p3 = load_acc_plane(plane(ez0 + 3), yrow, ex0, xi, vload);
-        T yn[4][2][2];   // the parent plane above
-        if (CARRY) {
-            pbase += P01;
-#pragma unroll
-            for (int j = 0; j < 4; ++j) lerp_plane(pf[j], pbase, P0, yn[j]);
-        }
+        carry.next();
         const bool wz[2] = {ez0 >= 0 && ez0 < E2, ez0 + 1 < E2};
         // field j (0 phi, 1-3 acc) of cells (.., b, c): values v0, v1 plus the carry
         auto put = [&](T* __restrict__ f, int j, int c, int b, T v0, T v1) {
-            if (CARRY) {
-                const T a = c == 0 ? (T)0.75 : (T)0.25, d = c == 0 ? (T)0.25 : (T)0.75;
-                v0 += a * yp[j][b][0] + d * yn[j][b][0];
-                v1 += a * yp[j][b][1] + d * yn[j][b][1];
-            }
+            carry.add(j, c, b, v0, v1);
             if (!((b == 0 ? wy0 : wy1) && wz[c])) return;
             // signed: with ex0 = -1 the row's first written cell is o[1] (fields hold fewer than 2^31 cells)
             T* __restrict__ o = f + (ex0 + E0 * ((ey0 + b) + E1 * (ez0 + c)));
@@ -236,12 +273,8 @@ __global__ void __launch_bounds__(kAccThreads, AccMinCtas<T>::march) k_accel(
 #pragma unroll
         for (int b = 0; b < 2; ++b)
 #pragma unroll
-            for (int a = 0; a < 2; ++a) {
-                z0[b][a] = p2.x[b][1 + a];
-                if (CARRY)
-#pragma unroll
-                    for (int j = 0; j < 4; ++j) yp[j][b][a] = yn[j][b][a];
-            }
+            for (int a = 0; a < 2; ++a) z0[b][a] = p2.x[b][1 + a];
+        carry.up();
         p1 = p3;
     }
 }
@@ -466,15 +499,89 @@ __global__ void __launch_bounds__(kIntThreads, APM_INT_MIN_CTAS) k_interp_levels
     interp_from<T>(L, L.g[own_g], reinterpret_cast<const T*>(accs[own_l][own_g]), X, p, P.n, out);
 }
 
-// Four-point and spectral gradients (Sec. 2.2; apm_gradient), on the 2x2x2
-// blocks of k_accel (same work list, same parent interpolation):
+// The spectral gradient's accelerations: phi and acc_j are the solve's four
+// windows of [-2, N+2) plus the parent's, on k_accel's columns of blocks; each
+// thread marches up z and keeps the parent plane between two blocks, so a block
+// loads 16 parent values instead of 32.  8 grids of 100^3: 113 -> 68 us.
+template <typename T, bool CARRY>
+__global__ void __launch_bounds__(kAccThreads, AccMinCtas<T>::march) k_accel_spectral(
+    LevelDev L, const GridDev* __restrict__ pgrids, const void* const* __restrict__ phis_p,
+    const void* const* __restrict__ pphi_p, const void* const* __restrict__ pacc_p, void* const* __restrict__ phi_p,
+    void* const* __restrict__ acc_p, const Chunk* __restrict__ chunks, int zs) {
+    const unsigned block = begin_kernel();
+    const Chunk ch = chunks[block];
+    const GridDev& g = L.g[ch.grid];
+    AccColumn c;
+    if (!c.start(g, ch.tile, zs)) return;
+    const int E0 = g.N[0] + 2, E1 = g.N[1] + 2, E2 = g.N[2] + 2;
+    const unsigned ncell = (unsigned)E0 * E1 * E2;
+    const int W0 = g.W[0], W1 = g.W[1];
+    const unsigned sz = (unsigned)W0 * W1, nw = sz * (unsigned)g.W[2];
+    const T* __restrict__ phis = reinterpret_cast<const T*>(phis_p[ch.grid]);
+    T* __restrict__ phi = reinterpret_cast<T*>(phi_p[ch.grid]);
+    T* __restrict__ acc = reinterpret_cast<T*>(acc_p[ch.grid]);
+    using V2 = typename Cplx<T>::type;
+    const size_t amask = 2 * sizeof(T) - 1;
+    const bool vst = !((E0 | c.ex0) & 1) && !(reinterpret_cast<size_t>(phi) & amask) &&
+                     !(reinterpret_cast<size_t>(acc) & amask) && !(ncell & 1);
+    // output cell e is window cell e + 1 on each axis
+    const bool wx0 = c.ex0 >= 0 && c.ex0 < E0, wx1 = c.ex0 + 1 < E0;
+    const bool vld = !((W0 | nw) & 1) && (c.ex0 & 1) && wx0 && wx1 && !(reinterpret_cast<size_t>(phis) & amask);
+    AccCarry<T, CARRY> carry;
+    if (!carry.start(L, g, pgrids, pphi_p, pacc_p, c)) return;
+    int ez0 = 2 * c.bz0 - g.acc_sh[2];
+#pragma unroll 1
+    for (int bz = c.bz0; bz < c.bz1; ++bz, ez0 += 2) {
+        T v[4][2][2][2];
+#pragma unroll
+        for (int j = 0; j < 4; ++j)
+#pragma unroll
+            for (int z = 0; z < 2; ++z)
+#pragma unroll
+                for (int b = 0; b < 2; ++b) {
+                    const int ey = c.ey0 + b, ez = ez0 + z;
+                    const bool ok = ey >= 0 && ey < E1 && ez >= 0 && ez < E2;
+                    const T* __restrict__ q = phis + ((size_t)j * nw + (unsigned)(W0 * (ey + 1)) + sz * (unsigned)(ez + 1));
+                    if (vld) {
+                        const V2 u = ok ? *reinterpret_cast<const V2*>(q + c.ex0 + 1) : mk2((T)0, (T)0);
+                        v[j][z][b][0] = u.x;
+                        v[j][z][b][1] = u.y;
+                    } else {
+                        v[j][z][b][0] = ok && wx0 ? q[c.ex0 + 1] : (T)0;
+                        v[j][z][b][1] = ok && wx1 ? q[c.ex0 + 2] : (T)0;
+                    }
+                }
+        carry.next();
+#pragma unroll
+        for (int j = 0; j < 4; ++j)
+#pragma unroll
+            for (int z = 0; z < 2; ++z)
+#pragma unroll
+                for (int b = 0; b < 2; ++b) {
+                    const int ey = c.ey0 + b, ez = ez0 + z;
+                    if (!(ey >= 0 && ey < E1 && ez >= 0 && ez < E2)) continue;
+                    T v0 = v[j][z][b][0], v1 = v[j][z][b][1];
+                    carry.add(j, z, b, v0, v1);
+                    T* __restrict__ o = (j == 0 ? phi : acc + (size_t)(j - 1) * ncell) + (c.ex0 + E0 * (ey + E1 * ez));
+                    if (vst && wx0 && wx1) {
+                        *reinterpret_cast<V2*>(o) = mk2(v0, v1);
+                    } else {
+                        if (wx0) o[0] = v0;
+                        if (wx1) o[1] = v1;
+                    }
+                }
+        carry.up();
+    }
+}
+
+// The four-point gradient (Sec. 2.2; apm_gradient), one 2x2x2 block of k_accel's
+// per thread (flat ranges of blocks, the same parent interpolation):
 //   phi(c)   = phis(c) + I(parent phi)(c)
 //   acc_j(c) = A_j(c) + I(parent acc_j)(c),        c in [-1, N]^3, with
 //   A_j = -(8 (phis(c+e_j) - phis(c-e_j)) - (phis(c+2e_j) - phis(c-2e_j))) / (12 delta)
-//         (four-point; phis spans [-3, N+3)), or the solve's spectral component
-//         j + 1 (phis: four windows of [-2, N+2)).
+//         (phis spans [-3, N+3)).
 // Output cell e (index 0..E-1) is level cell e - 1 and phis cell e - 1 + h.
-template <typename T, int GRAD>
+template <typename T>
 __global__ void __launch_bounds__(kAccThreads, AccMinCtas<T>::value) k_accel_var(
     LevelDev L, const GridDev* __restrict__ pgrids, const void* const* __restrict__ phis_p,
     const void* const* __restrict__ pphi_p, const void* const* __restrict__ pacc_p,
@@ -609,39 +716,31 @@ __global__ void __launch_bounds__(kAccThreads, AccMinCtas<T>::value) k_accel_var
                     const unsigned ci = c0[c][b][0];
                     T v[2] = {0, 0};
                     if (wr[c][b][0] && wr[c][b][1]) {
-                        if constexpr (GRAD == APM_GRAD_FD4) {
-                            if (j == 0) {   // x: cells ci-2 .. ci+3
-                                T m2, m1, p0, p1, p2, p3;
-                                ld2(phis, ci - 2, m2, m1);
-                                ld2(phis, ci, p0, p1);
-                                ld2(phis, ci + 2, p2, p3);
-                                v[0] = -((T)8 * (p1 - m1) - (p2 - m2)) * inv12d;
-                                v[1] = -((T)8 * (p2 - p0) - (p3 - m1)) * inv12d;
-                            } else {
-                                T a1[2], b1[2], a2[2], b2[2];
-                                ld2(phis, ci + st[j], a1[0], a1[1]);
-                                ld2(phis, ci - st[j], b1[0], b1[1]);
-                                ld2(phis, ci + 2 * st[j], a2[0], a2[1]);
-                                ld2(phis, ci - 2 * st[j], b2[0], b2[1]);
-#pragma unroll
-                                for (int a = 0; a < 2; ++a)
-                                    v[a] = -((T)8 * (a1[a] - b1[a]) - (a2[a] - b2[a])) * inv12d;
-                            }
+                        if (j == 0) {   // x: cells ci-2 .. ci+3
+                            T m2, m1, p0, p1, p2, p3;
+                            ld2(phis, ci - 2, m2, m1);
+                            ld2(phis, ci, p0, p1);
+                            ld2(phis, ci + 2, p2, p3);
+                            v[0] = -((T)8 * (p1 - m1) - (p2 - m2)) * inv12d;
+                            v[1] = -((T)8 * (p2 - p0) - (p3 - m1)) * inv12d;
                         } else {
-                            ld2(phis, (j + 1) * nw + ci, v[0], v[1]);
+                            T a1[2], b1[2], a2[2], b2[2];
+                            ld2(phis, ci + st[j], a1[0], a1[1]);
+                            ld2(phis, ci - st[j], b1[0], b1[1]);
+                            ld2(phis, ci + 2 * st[j], a2[0], a2[1]);
+                            ld2(phis, ci - 2 * st[j], b2[0], b2[1]);
+#pragma unroll
+                            for (int a = 0; a < 2; ++a)
+                                v[a] = -((T)8 * (a1[a] - b1[a]) - (a2[a] - b2[a])) * inv12d;
                         }
                     } else {
 #pragma unroll
                         for (int a = 0; a < 2; ++a) {
                             if (!wr[c][b][a]) continue;
                             const unsigned cc = ci + a;
-                            if constexpr (GRAD == APM_GRAD_FD4) {
-                                const T d1 = phis[cc + st[j]] - phis[cc - st[j]];
-                                const T d2 = phis[cc + 2 * st[j]] - phis[cc - 2 * st[j]];
-                                v[a] = -((T)8 * d1 - d2) * inv12d;
-                            } else {
-                                v[a] = phis[(j + 1) * nw + cc];
-                            }
+                            const T d1 = phis[cc + st[j]] - phis[cc - st[j]];
+                            const T d2 = phis[cc + 2 * st[j]] - phis[cc - 2 * st[j]];
+                            v[a] = -((T)8 * d1 - d2) * inv12d;
                         }
                     }
                     if (carry) {
@@ -671,13 +770,16 @@ cudaError_t launch_accel(const LevelDev& L, const GridDev* parent_grids, const v
 template <typename T>
 cudaError_t launch_accel_var(const LevelDev& L, const GridDev* parent_grids, const void* const* phis,
                                const void* const* pphi, const void* const* pacc, void* const* phi,
-                               void* const* acc, const Chunk* chunks, int n_chunks, int grad,
+                               void* const* acc, const Chunk* chunks, int n_chunks, int grad, int zs,
                                cudaStream_t s) {
     if (n_chunks <= 0) return cudaSuccess;
     if (grad == APM_GRAD_FD4)
-        return launch_kernel(k_accel_var<T, APM_GRAD_FD4>, n_chunks, kAccThreads, 0, s, L, parent_grids, phis, pphi, pacc, phi, acc, chunks);
-    else
-        return launch_kernel(k_accel_var<T, APM_GRAD_SPECTRAL>, n_chunks, kAccThreads, 0, s, L, parent_grids, phis, pphi, pacc, phi, acc, chunks);
+        return launch_kernel(k_accel_var<T>, n_chunks, kAccThreads, 0, s, L, parent_grids, phis, pphi, pacc, phi, acc,
+                             chunks);
+    return pphi ? launch_kernel(k_accel_spectral<T, true>, n_chunks, kAccThreads, 0, s, L, parent_grids, phis, pphi,
+                                pacc, phi, acc, chunks, zs)
+                : launch_kernel(k_accel_spectral<T, false>, n_chunks, kAccThreads, 0, s, L, parent_grids, phis, pphi,
+                                pacc, phi, acc, chunks, zs);
 }
 
 template <typename T>
@@ -705,10 +807,10 @@ template cudaError_t launch_accel<double>(const LevelDev&, const GridDev*, const
                                           void* const*, const Chunk*, int, int, cudaStream_t);
 template cudaError_t launch_accel_var<float>(const LevelDev&, const GridDev*, const void* const*,
                                                const void* const*, const void* const*, void* const*,
-                                               void* const*, const Chunk*, int, int, cudaStream_t);
+                                               void* const*, const Chunk*, int, int, int, cudaStream_t);
 template cudaError_t launch_accel_var<double>(const LevelDev&, const GridDev*, const void* const*,
                                                 const void* const*, const void* const*, void* const*,
-                                                void* const*, const Chunk*, int, int, cudaStream_t);
+                                                void* const*, const Chunk*, int, int, int, cudaStream_t);
 template cudaError_t launch_interp<float>(const LevelDev&, const LevelDev*, const Particles&, double,
                                           const void* const*, void*, cudaStream_t);
 template cudaError_t launch_interp<double>(const LevelDev&, const LevelDev*, const Particles&, double,

@@ -1,8 +1,8 @@
-"""The two-point acceleration kernel marches each thread through a column of
-blocks where a level is large enough: every cell of levels that march 1, 2
-and 8 blocks, with ragged last segments and odd sizes and starts, against the
-difference and trilinear carry in plain FP64 torch (FP64 1e-12, FP32 2e-5 / 1e-4,
-the suite's tolerances)."""
+"""The two-point and spectral acceleration kernels march each thread through a
+column of blocks where a level is large enough: every cell of levels that march
+1, 2 and 8 blocks, with ragged last segments and odd sizes and starts, against
+the difference (the window's components) and the trilinear carry in plain FP64
+torch (FP64 1e-12, FP32 2e-5 / 1e-4, the suite's tolerances)."""
 import itertools
 
 import pytest
@@ -25,9 +25,10 @@ def _carry(f, start, dims, pstart):
     return f
 
 
+@pytest.mark.parametrize("gradient", ["fd2", "spectral"])
 @pytest.mark.parametrize("precision", ["fp64", "fp32"])
 @pytest.mark.parametrize("per_axis,dims", [(1, (40, 33, 47)), (2, (52, 53, 50)), (3, (50, 45, 59)), (4, (52, 57, 60))])
-def test_march_matches_plain_formula(per_axis, dims, precision):
+def test_march_matches_plain_formula(per_axis, dims, precision, gradient):
     import torch
 
     from paper_1410_0010_gb300.solver import Solver
@@ -38,7 +39,7 @@ def test_march_matches_plain_formula(per_axis, dims, precision):
     grids = [GridDesc(0, -1, (0, 0, 0), (root,) * 3)]
     for i, o in enumerate(itertools.product(range(per_axis), repeat=3)):
         grids.append(GridDesc(1, 0, tuple(2 * (4 + step * v) + i % 2 for v in o), dims))
-    s = Solver(grids, periodic=True, precision=precision, device=0)
+    s = Solver(grids, periodic=True, precision=precision, device=0, gradient=gradient)
     gen = torch.Generator(device="cuda").manual_seed(3)
 
     def field(shape):
@@ -55,12 +56,17 @@ def test_march_matches_plain_formula(per_axis, dims, precision):
     e = [n + 2 for n in dims]
     for g, phis, phi, acc in zip(grids[1:], b["phis"], b["phi"], b["acc"]):
         p = phis.double()
+        comps = p[1:] if gradient == "spectral" else None
+        p = p[0] if gradient == "spectral" else p
 
         def at(j, o):
             c = [1, 1, 1]
             c[j] += o
             return p[c[2]:c[2] + e[2], c[1]:c[1] + e[1], c[0]:c[0] + e[0]]
-        want = torch.stack([-(at(j, 1) - at(j, -1)) / (2 * d) for j in range(3)])
+        if gradient == "spectral":
+            want = comps[:, 1:1 + e[2], 1:1 + e[1], 1:1 + e[0]]
+        else:
+            want = torch.stack([-(at(j, 1) - at(j, -1)) / (2 * d) for j in range(3)])
         want = want + _carry(pacc.double(), g.start, dims, (0, 0, 0))
         wphi = at(0, 0) + _carry(pphi.double(), g.start, dims, (0, 0, 0))
         assert ((acc.double() - want).norm() / want.norm()).item() <= TOL[precision]["acc"]
