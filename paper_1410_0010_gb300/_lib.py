@@ -132,7 +132,4 @@ def check(code, where):
 
 def ptr_array(ptrs):
     """HOST array of device pointers (None -> NULL entry)."""
-    arr = (c_void_p * len(ptrs))()
-    for i, p in enumerate(ptrs):
-        arr[i] = p
-    return arr
+    return (c_void_p * len(ptrs))(*ptrs)

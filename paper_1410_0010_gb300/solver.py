@@ -15,6 +15,9 @@ PARTICLE_KEYS = ("x", "y", "z", "vx", "vy", "vz", "m")
 
 
 def _stream_handle(stream=None):
+    """The C handle of a torch stream (None: the current one); a handle is returned as it is."""
+    if isinstance(stream, ctypes.c_void_p):
+        return stream
     s = stream if stream is not None else torch.cuda.current_stream()
     return ctypes.c_void_p(s.cuda_stream)
 
@@ -387,6 +390,7 @@ class Solver:
             for gi, g in enumerate(gas):
                 if g is not None:
                     check_field(g, tuple(self.grids[gi][3])[::-1], torch.float64, self.device, f"gas of grid {gi}")
+        stream = _stream_handle(stream)   # once for the calls below
         levs = range(self.n_levels) if levels is None else levels
         whole = batched and (levels is None or list(levels) == list(range(self.n_levels)))
         if 0 < P.n <= getattr(self, "order_capacity", 0):
