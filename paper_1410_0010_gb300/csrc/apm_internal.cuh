@@ -166,18 +166,26 @@ constexpr int kFastGroups = 4;
 // x pass; 128 bytes of each HBM row in both precisions
 constexpr int fast_lines(bool f64) { return f64 ? 8 : 16; }
 
-// threads of a fast pass CTA for `lines` lines: whole warps, at least 3 (4 for
-// L > 96: fewer leave the SM short of warps, 5 or 6 help no further), and among
-// up to 6 warps the count whose stages leave the fewest threads without a
-// butterfly in their last trip.  The z pass of 32 grids of L = 150: 264 us with
-// 2 warps, 171 with 3 to 5; 8 spectral ones of 120: 155 with 3, 131 with 4; 343
-// grids of 36 to 84: all passes 531 with 2, 495 with 3, 512 with 4.
+// threads of a fast pass CTA for `lines` lines: whole warps.  Up to L = 96, of 3
+// to 6 warps the count whose stages leave the fewest threads without a butterfly
+// in their last trip; above, 4 or, where that fits the first stage's butterflies,
+// 5; and as many as give 24 warps per SM with as many CTAs as the shared memory
+// of their lines lets in (128 bytes of each of L elements and a pad; 8 warps for
+// L = 512).  The z pass of 32 grids of L = 150: 264 us with 2 warps, 178 with 3,
+// 181 with 4, 171 with 5; 8 spectral ones of 120: 155 with 3, 131 with 4; 343
+// grids of 36 to 84: all passes 531 with 2 or more, 498 with 3 or more, 515 with
+// 3 always; the x forward of a 512^3 root: 671 with 4, 449 with 8.
 constexpr int fast_threads(int r1, int r2, int r3, int lines) {
     const int L = r1 * r2 * r3;
     const int items[3] = {L / r1 * lines, L / r2 * lines, r3 > 1 ? L / r3 * lines : 0};
-    const int least = L > 96 ? 128 : 96;
-    int best = least, best_cost = 1 << 30;
-    for (int nt = least; nt <= 192; nt += 32) {
+    if (L > 96) {
+        const int ctas = 220 * 1024 / (L * 17 * 8);
+        int nt = items[0] > 128 && items[0] <= 160 ? 160 : 128;
+        while (nt < 256 && nt * ctas < 768) nt += 32;
+        return nt;
+    }
+    int best = 96, best_cost = 1 << 30;
+    for (int nt = 96; nt <= 192; nt += 32) {
         int cost = 0;
         for (int k = 0; k < 3; ++k) cost += (items[k] + nt - 1) / nt * nt;
         if (cost < best_cost || (cost == best_cost && nt <= 160)) {

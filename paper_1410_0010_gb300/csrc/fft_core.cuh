@@ -411,23 +411,23 @@ __device__ __forceinline__ float fixed48_to_float(long long q) {
 template <> __device__ __forceinline__ float fixed_to_real<float>(long long q, float scale) {
     return (fits48(q) ? fixed48_to_float(q) : __ll2float_rn(q)) * scale;
 }
-// two complex values (a + i b), (c + i d) at once, with one test for the four
-// (the load passes convert two cells of two rows per thread)
-template <typename T>
+// two complex values (a + i b), (c + i d) at once (the load passes convert two
+// cells of two rows per thread).  WIDE false: without the test, *wide set where
+// one of the four needed the instruction (the pass is then done again); a branch
+// per value would keep the compiler from issuing a thread's loads together.
+template <typename T, bool WIDE>
 __device__ __forceinline__ void fixed4_to_real(long long a, long long b, long long c, long long d, T scale, C<T>& u,
-                                               C<T>& v) {
-    u = mk<T>(fixed_to_real<T>(a, scale), fixed_to_real<T>(b, scale));
-    v = mk<T>(fixed_to_real<T>(c, scale), fixed_to_real<T>(d, scale));
-}
-template <>
-__device__ __forceinline__ void fixed4_to_real<float>(long long a, long long b, long long c, long long d, float scale,
-                                                      float2& u, float2& v) {
-    if (fits48(a) && fits48(b) && fits48(c) && fits48(d)) {
-        u = make_float2(fixed48_to_float(a) * scale, fixed48_to_float(b) * scale);
-        v = make_float2(fixed48_to_float(c) * scale, fixed48_to_float(d) * scale);
+                                               C<T>& v, bool& wide) {
+    if constexpr (sizeof(T) == 8) {
+        u = mk<T>(__ll2double_rn(a) * scale, __ll2double_rn(b) * scale);
+        v = mk<T>(__ll2double_rn(c) * scale, __ll2double_rn(d) * scale);
+    } else if constexpr (WIDE) {
+        u = mk<T>(__ll2float_rn(a) * scale, __ll2float_rn(b) * scale);
+        v = mk<T>(__ll2float_rn(c) * scale, __ll2float_rn(d) * scale);
     } else {
-        u = make_float2(__ll2float_rn(a) * scale, __ll2float_rn(b) * scale);
-        v = make_float2(__ll2float_rn(c) * scale, __ll2float_rn(d) * scale);
+        wide = wide || !(fits48(a) && fits48(b) && fits48(c) && fits48(d));
+        u = mk<T>(fixed48_to_float(a) * scale, fixed48_to_float(b) * scale);
+        v = mk<T>(fixed48_to_float(c) * scale, fixed48_to_float(d) * scale);
     }
 }
 
