@@ -28,7 +28,7 @@
  *    asynchronous on it; calls on one context must be ordered (one stream, or
  *    synchronised by the caller).  A context is not thread-safe.  Within a
  *    call, an FFT pass whose grids run different kernels spreads them over the
- *    context's three auxiliary streams, forked from `stream` and joined back
+ *    context's five auxiliary streams, forked from `stream` and joined back
  *    to it with events: the work stays ordered on `stream`, and a capture of
  *    `stream` takes the branches in.
  *  - Errors detectable on the host are returned immediately and nothing is
