@@ -172,13 +172,14 @@ template <typename T, bool CARRY> struct AccCarry {
         v1 += a * yp[j][b][1] + d * yn[j][b][1];
     }
     __device__ __forceinline__ void up() {
-        if (!CARRY) return;
+        if constexpr (CARRY) {
 #pragma unroll
-        for (int j = 0; j < 4; ++j)
+            for (int j = 0; j < 4; ++j)
 #pragma unroll
-            for (int b = 0; b < 2; ++b)
+                for (int b = 0; b < 2; ++b)
 #pragma unroll
-                for (int a = 0; a < 2; ++a) yp[j][b][a] = yn[j][b][a];
+                    for (int a = 0; a < 2; ++a) yp[j][b][a] = yn[j][b][a];
+        }
     }
 };
 
