@@ -235,8 +235,9 @@ long long floor_div(long long a, long long b) {
     return q;
 }
 
-// the passes use the compile-time plans of fft_fast.cuh where a length has one (APM_FFT_FAST=0 keeps every pass on the runtime-planned
-// kernels, for comparison)
+// the passes use the compile-time plans of fft_fast.cuh where a length has one
+// (APM_FFT_FAST=0 keeps every pass on the runtime-planned kernels, for
+// comparison)
 bool fft_fast_enabled() {
     const char* v = std::getenv("APM_FFT_FAST");
     return !(v && std::atoi(v) == 0);
@@ -375,8 +376,9 @@ apm_status build_pass(apm_ctx* c, const Level& L, int q, int budget, int threads
     std::vector<int> fast(ng, 0), lens(ng, 0);
     const bool row = q == kPassXf || q == kPassXi;
     // with plan 2 on the x-forward pass (or plan 0 and a length of
-    // fast_xy_default), a grid with M0 = M1 whose plane fits runs the fused x + y forward (k_xy_fast) as its x-forward segment (kind
-    // -L) and has no y-forward work (kind kSkip); other grids run plan 0
+    // fast_xy_default), a grid with M0 = M1 whose plane fits runs the fused x + y
+    // forward (k_xy_fast) as its x-forward segment (kind -L) and has no y-forward
+    // work (kind kSkip); other grids run plan 0
     constexpr int kSkip = INT_MIN;
     auto fuses = [&](int x_pass, int len) {
         return L.plan[x_pass] == 2 || (L.plan[x_pass] == 0 && fast_xy_default(len));

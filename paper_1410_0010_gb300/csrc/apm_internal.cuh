@@ -282,13 +282,13 @@ struct RowWalk {
     }
 };
 
-// 2x2x2 output blocks per CTA of the four-point acceleration kernel (flat ranges of the grid's blocks, x fastest, so every thread gets the
-// same count)
+// 2x2x2 output blocks per CTA of the four-point acceleration kernel (flat ranges
+// of the grid's blocks, x fastest, so every thread gets the same count)
 constexpr int kAccBlocksPerCta = 512;
-// threads of an acceleration CTA; the two-point and spectral kernels give each one (x, y)
-// column of blocks and march through up to kAccMarch blocks of it (4 to 16
-// measure alike on large levels; the host halves it while a level would leave
-// SMs idle)
+// threads of an acceleration CTA; the two-point and spectral kernels give each
+// one (x, y) column of blocks and march through up to kAccMarch blocks of it (4
+// to 16 measure alike on large levels; the host halves it while a level would
+// leave SMs idle)
 #ifndef APM_ACC_THREADS
 #define APM_ACC_THREADS 128
 #endif

@@ -424,7 +424,8 @@ cudaError_t launch_deposit(const LevelDev& L, const Particles& P, double half_dt
                            int F, int64_t* const* gmf, unsigned* status, cudaStream_t s) {
     if (P.n <= 0) return cudaSuccess;
     unsigned blocks = (unsigned)((P.n + kDepThreads - 1) / kDepThreads);
-    return launch_kernel(k_deposit, blocks, kDepThreads, 0, s, L, deposit_order(P, blocks), half_dt, box, F, gmf, status);
+    return launch_kernel(k_deposit, blocks, kDepThreads, 0, s, L, deposit_order(P, blocks), half_dt, box, F, gmf,
+                         status);
 }
 
 cudaError_t launch_deposit_levels(const LevelDev* levels, int nl, const Particles& P, double half_dt,
@@ -432,7 +433,8 @@ cudaError_t launch_deposit_levels(const LevelDev* levels, int nl, const Particle
                                   cudaStream_t s) {
     if (P.n <= 0 || nl <= 0) return cudaSuccess;
     unsigned blocks = (unsigned)((P.n + kDepThreads - 1) / kDepThreads);
-    return launch_kernel(k_deposit_levels, blocks, kDepThreads, 0, s, levels, nl, deposit_order(P, blocks), half_dt, box, F, gmfs, status);
+    return launch_kernel(k_deposit_levels, blocks, kDepThreads, 0, s, levels, nl, deposit_order(P, blocks),
+                         half_dt, box, F, gmfs, status);
 }
 
 }  // namespace apm

@@ -79,7 +79,8 @@ cudaError_t launch_kick_drift(long long n, double* x, double* y, double* z, doub
                               const void* acc, double dt, cudaStream_t s) {
     if (n <= 0) return cudaSuccess;
     const unsigned blocks = (unsigned)((n + 255) / 256);
-    return launch_kernel(k_kick_drift<T>, blocks, 256, 0, s, n, x, y, z, vx, vy, vz, reinterpret_cast<const T*>(acc), dt);
+    return launch_kernel(k_kick_drift<T>, blocks, 256, 0, s, n, x, y, z, vx, vy, vz,
+                         reinterpret_cast<const T*>(acc), dt);
 }
 
 template cudaError_t launch_kick_drift<float>(long long, double*, double*, double*, double*, double*, double*,

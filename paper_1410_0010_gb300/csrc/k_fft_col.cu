@@ -37,9 +37,11 @@ cudaError_t launch_col(const FftArgs& a, cudaStream_t s) {
     using T = ColT;
     if (a.n_chunks <= 0) return cudaSuccess;
     if (a.threads == 128)
-        return launch_kernel(k_col<T, kColAx, kColMode, 128>, a.n_chunks, 128, a.smem, s, a.g, a.chunks, (const C<T>*)a.tw, (const T*)a.tab, (C<T>*)a.wsA, (C<T>*)a.wsB, a.comp);
+        return launch_kernel(k_col<T, kColAx, kColMode, 128>, a.n_chunks, 128, a.smem, s, a.g, a.chunks,
+                             (const C<T>*)a.tw, (const T*)a.tab, (C<T>*)a.wsA, (C<T>*)a.wsB, a.comp);
     else
-        return launch_kernel(k_col<T, kColAx, kColMode, 256>, a.n_chunks, 256, a.smem, s, a.g, a.chunks, (const C<T>*)a.tw, (const T*)a.tab, (C<T>*)a.wsA, (C<T>*)a.wsB, a.comp);
+        return launch_kernel(k_col<T, kColAx, kColMode, 256>, a.n_chunks, 256, a.smem, s, a.g, a.chunks,
+                             (const C<T>*)a.tw, (const T*)a.tab, (C<T>*)a.wsA, (C<T>*)a.wsB, a.comp);
 }
 }  // namespace
 

@@ -58,11 +58,14 @@ cudaError_t launch_one(const FftArgs& a, const int64_t* const* gmf, void* const*
         else if constexpr (kMode == kFastXy)
             return launch_kernel(kern, a.n_chunks, K::NT, K::smem, s, a.g, a.chunks, gmf, tw, (C<FT>*)a.wsB, a.F);
         else if constexpr (kMode == kFastXi)
-            return launch_kernel(kern, a.n_chunks, K::NT, K::smem, s, a.g, a.chunks, tw, (const C<FT>*)a.wsB, phis, a.comp);
+            return launch_kernel(kern, a.n_chunks, K::NT, K::smem, s, a.g, a.chunks, tw, (const C<FT>*)a.wsB, phis,
+                                 a.comp);
         else if constexpr (kMode == kFastYx)
-            return launch_kernel(kern, a.n_chunks, K::NT, K::smem, s, a.g, a.chunks, tw, (const C<FT>*)a.wsA, phis, a.comp);
+            return launch_kernel(kern, a.n_chunks, K::NT, K::smem, s, a.g, a.chunks, tw, (const C<FT>*)a.wsA, phis,
+                                 a.comp);
         else
-            return launch_kernel(kern, a.n_chunks, K::NT, K::smem, s, a.g, a.chunks, tw, (const FT*)a.tab, (C<FT>*)a.wsA, (C<FT>*)a.wsB, a.comp);
+            return launch_kernel(kern, a.n_chunks, K::NT, K::smem, s, a.g, a.chunks, tw, (const FT*)a.tab,
+                                 (C<FT>*)a.wsA, (C<FT>*)a.wsB, a.comp);
     }
     return cudaErrorInvalidValue;
 }

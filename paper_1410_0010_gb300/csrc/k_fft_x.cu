@@ -71,18 +71,22 @@ template <typename T>
 cudaError_t launch_fft_xf(const FftArgs& a, const int64_t* const* gmf, cudaStream_t s) {
     if (a.n_chunks <= 0) return cudaSuccess;
     if (a.threads == 128)
-        return launch_kernel(k_xf<T, 128>, a.n_chunks, 128, a.smem, s, a.g, a.chunks, gmf, (const C<T>*)a.tw, (C<T>*)a.wsA, a.F, a.status, a.inject_wait);
+        return launch_kernel(k_xf<T, 128>, a.n_chunks, 128, a.smem, s, a.g, a.chunks, gmf, (const C<T>*)a.tw,
+                             (C<T>*)a.wsA, a.F, a.status, a.inject_wait);
     else
-        return launch_kernel(k_xf<T, 256>, a.n_chunks, 256, a.smem, s, a.g, a.chunks, gmf, (const C<T>*)a.tw, (C<T>*)a.wsA, a.F, a.status, a.inject_wait);
+        return launch_kernel(k_xf<T, 256>, a.n_chunks, 256, a.smem, s, a.g, a.chunks, gmf, (const C<T>*)a.tw,
+                             (C<T>*)a.wsA, a.F, a.status, a.inject_wait);
 }
 
 template <typename T>
 cudaError_t launch_fft_xi(const FftArgs& a, void* const* phis, cudaStream_t s) {
     if (a.n_chunks <= 0) return cudaSuccess;
     if (a.threads == 128)
-        return launch_kernel(k_xi<T, 128>, a.n_chunks, 128, a.smem, s, a.g, a.chunks, (const C<T>*)a.tw, (const C<T>*)a.wsB, phis, a.comp);
+        return launch_kernel(k_xi<T, 128>, a.n_chunks, 128, a.smem, s, a.g, a.chunks, (const C<T>*)a.tw,
+                             (const C<T>*)a.wsB, phis, a.comp);
     else
-        return launch_kernel(k_xi<T, 256>, a.n_chunks, 256, a.smem, s, a.g, a.chunks, (const C<T>*)a.tw, (const C<T>*)a.wsB, phis, a.comp);
+        return launch_kernel(k_xi<T, 256>, a.n_chunks, 256, a.smem, s, a.g, a.chunks, (const C<T>*)a.tw,
+                             (const C<T>*)a.wsB, phis, a.comp);
 }
 
 template cudaError_t launch_fft_xf<float>(const FftArgs&, const int64_t* const*, cudaStream_t);

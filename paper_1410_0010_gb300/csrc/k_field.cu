@@ -386,7 +386,8 @@ __device__ __forceinline__ void interp_from(const LevelDev& L, const GridDev& g,
     for (int j = 0; j < 3; ++j) pairs = pairs && (!fold || (lc[j] > 0 && lc[j] < g.N[j] - 1));
     if (pairs) {
         const bool odd = lc[0] & 1;
-        const T* __restrict__ base = A + ((unsigned)(lc[0] & ~1) + (unsigned)E0 * ((unsigned)lc[1] + (unsigned)E1 * (unsigned)lc[2]));
+        const T* __restrict__ base =
+            A + ((unsigned)(lc[0] & ~1) + (unsigned)E0 * ((unsigned)lc[1] + (unsigned)E1 * (unsigned)lc[2]));
 #pragma unroll
         for (int c = 0; c < 3; ++c)
 #pragma unroll
@@ -763,9 +764,11 @@ cudaError_t launch_accel(const LevelDev& L, const GridDev* parent_grids, const v
                          cudaStream_t s) {
     if (n_chunks <= 0) return cudaSuccess;
     if (pphi)   // every grid of a level that gets parent fields has a parent
-        return launch_kernel(k_accel<T, true>, n_chunks, kAccThreads, 0, s, L, parent_grids, phis, pphi, pacc, phi, acc, chunks, zs);
+        return launch_kernel(k_accel<T, true>, n_chunks, kAccThreads, 0, s, L, parent_grids, phis, pphi, pacc, phi,
+                             acc, chunks, zs);
     else
-        return launch_kernel(k_accel<T, false>, n_chunks, kAccThreads, 0, s, L, parent_grids, phis, pphi, pacc, phi, acc, chunks, zs);
+        return launch_kernel(k_accel<T, false>, n_chunks, kAccThreads, 0, s, L, parent_grids, phis, pphi, pacc,
+                             phi, acc, chunks, zs);
 }
 
 template <typename T>
@@ -789,7 +792,8 @@ cudaError_t launch_interp(const LevelDev& L, const LevelDev* finer, const Partic
     if (P.n <= 0) return cudaSuccess;
     unsigned blocks = (unsigned)((P.n + 255) / 256);
     LevelDev F = finer ? *finer : L;
-    return launch_kernel(k_interp<T>, blocks, 256, 0, s, L, F, finer ? 1 : 0, P, half_dt, acc, reinterpret_cast<T*>(out));
+    return launch_kernel(k_interp<T>, blocks, 256, 0, s, L, F, finer ? 1 : 0, P, half_dt, acc,
+                         reinterpret_cast<T*>(out));
 }
 
 template <typename T>
@@ -797,7 +801,8 @@ cudaError_t launch_interp_levels(const LevelDev* levels, int nl, const Particles
                                  const void* const* const* accs, void* out, cudaStream_t s) {
     if (P.n <= 0 || nl <= 0) return cudaSuccess;
     unsigned blocks = (unsigned)((P.n + kIntThreads - 1) / kIntThreads);
-    return launch_kernel(k_interp_levels<T>, blocks, kIntThreads, 0, s, levels, nl, P, half_dt, accs, reinterpret_cast<T*>(out));
+    return launch_kernel(k_interp_levels<T>, blocks, kIntThreads, 0, s, levels, nl, P, half_dt, accs,
+                         reinterpret_cast<T*>(out));
 }
 
 template cudaError_t launch_accel<float>(const LevelDev&, const GridDev*, const void* const*,
