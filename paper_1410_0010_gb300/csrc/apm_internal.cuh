@@ -652,9 +652,15 @@ cudaError_t launch_fft_xi(const FftArgs& a, void* const* phis, cudaStream_t s);
 // M0 = M1 = L, and y + x inverse over one window plane (k_yx_fast) for grids
 // whose window fits the transform (W1 <= M1).
 enum { kFastYf = 0, kFastZ, kFastYi, kFastXf, kFastXi, kFastZg, kFastXy, kFastYx, kFastKernels };
+// threads of a plane kernel: 384, and 512 for the x + y forward where two planes
+// fit an SM (32 grids of L = 150: 368 -> 353 us; the inverse loses, 218 -> 244, as
+// does an isolated root of L = 192 with one plane per SM)
 constexpr int kFastXyThreads = 384;
 // the plane (L rows x L/2 + 1 columns) and the twiddles
 constexpr size_t fast_xy_smem(int L) { return (size_t)(L * (L / 2 + 1) + L) * sizeof(float2); }
+constexpr int fast_xy_threads(int kernel, int L) {
+    return kernel == kFastXy && 2 * (fast_xy_smem(L) + 1024) <= (size_t)227 * 1024 ? 512 : kFastXyThreads;
+}
 inline bool fast_xy_length(int L) { return fast_length(L, false) && fast_xy_smem(L) <= (size_t)kFftSmemLimit; }
 // plan 0 runs the fused planes for M0 = M1 = L from 70 to 192 (plan 2: wherever
 // a plane fits).  Measured, unfused against fused, one level's five passes in

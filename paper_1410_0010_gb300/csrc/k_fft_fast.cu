@@ -32,7 +32,7 @@ struct Kern {
     static constexpr bool row = kMode == kFastXf || kMode == kFastXi;
     // a fused plane kernel exists where the plane fits the shared-memory limit
     static constexpr bool ok = !kFused || fast_xy_smem(L) <= (size_t)kFftSmemLimit;
-    static constexpr int NT = kFused ? kFastXyThreads : fast_threads(A, B, Cc, kLines);
+    static constexpr int NT = kFused ? fast_xy_threads(kMode, L) : fast_threads(A, B, Cc, kLines);
     static constexpr size_t smem = kFused ? fast_xy_smem(L) : (row ? fast_row_smem(L, kF64) : fast_col_smem(L, kF64));
     static constexpr auto get() {
         if constexpr (kMode == kFastYf) return k_col_fast<P, 1, 0, kLines, NT, FT>;
