@@ -558,7 +558,10 @@ struct Particles {
 // step 10.2 -> 11.6 ms, that graph 99.5 -> 123 us.
 // The block index comes out of the same instruction sequence, so that every
 // address a kernel forms from it, and with it every load, depends on the wait
-// (loads through const __restrict__ pointers may otherwise be moved across it).
+// (loads through __restrict__ pointers may otherwise be moved across it).  The
+// exceptions are the level and pointer tables of the all-level kernels (levels,
+// gmfs, accs and the root's entry in them): no kernel writes those, and the
+// copies that do come before the predecessor's own wait or after its end.
 __device__ __forceinline__ unsigned begin_kernel() {
     unsigned block;
     asm volatile("griddepcontrol.wait;\n\tmov.u32 %0, %%ctaid.x;" : "=r"(block) : : "memory");

@@ -100,9 +100,10 @@ __global__ void __launch_bounds__(1024) k_order_scan_local(unsigned* __restrict_
 
 // exclusive scan of the chunk totals (at most 1024 chunks) in place, one CTA
 __global__ void __launch_bounds__(1024) k_order_scan_sums(unsigned* __restrict__ sums, int n) {
-    begin_kernel();
+    const unsigned block = begin_kernel();   // 0: its address keeps the load behind the wait
     __shared__ unsigned warp_tot[32];
-    const unsigned t = threadIdx.x < (unsigned)n ? sums[threadIdx.x] : 0u;
+    const unsigned i = block * blockDim.x + threadIdx.x;
+    const unsigned t = i < (unsigned)n ? sums[i] : 0u;
     unsigned v = t;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
 #pragma unroll
@@ -122,7 +123,7 @@ __global__ void __launch_bounds__(1024) k_order_scan_sums(unsigned* __restrict__
         warp_tot[lane] = w;
     }
     __syncthreads();
-    if (threadIdx.x < (unsigned)n) sums[threadIdx.x] = v - t + (warp > 0 ? warp_tot[warp - 1] : 0u);
+    if (i < (unsigned)n) sums[i] = v - t + (warp > 0 ? warp_tot[warp - 1] : 0u);
 }
 
 // perm[slot] = p with slot = (chunk offset + bin offset + rank)
