@@ -141,15 +141,22 @@ constexpr unsigned kNoCell = 0x80000000u;   // mass fields hold fewer than 2^31 
 // This lane's particle's charges, layer by layer: ((|M| wx) wy) wz for the 26
 // outer cells, every product rounded half up on the scale 2^63, the centre cell
 // |M| minus the others, all with the sign of M; the middle layer, which holds the
-// centre, comes last.  Masses in [0, 2^32) have 32-bit charges (the weights sum
-// to one): V = unsigned.
+// centre, comes last.  V = unsigned holds every charge of a mass in [2^9, 2^32)
+// (narrow_mass): none exceeds it, as the weights sum to one, and the centre cell's
+// is positive, as its weight is at least 1/8 (1/2 an axis) and the 26 others are
+// rounded up by less than 2 units each.  The centre of a smaller mass may be
+// negative (M = 1 on a cell corner: 7 charges of 1, centre -6).
+constexpr long long kMinNarrow = 512;
+__device__ __forceinline__ bool narrow_mass(long long M) {
+    return (unsigned long long)(M - kMinNarrow) < (1ULL << 32) - (unsigned long long)kMinNarrow;
+}
 __device__ __forceinline__ unsigned mul63w(unsigned a, unsigned long long b) { return wmul63_32(a, b); }
 __device__ __forceinline__ unsigned long long mul63w(unsigned long long a, unsigned long long b) {
     return wmul63(a, b);
 }
 template <typename V> struct LaneCharges {
     V mxy[9];        // (|M| wx) wy of cell a + 3 b
-    V centre;        // |M| minus the outer charges so far
+    V centre;        // |M| minus the outer charges so far (64 bits: modulo 2^64)
     bool negative;
     __device__ __forceinline__ void start(long long M, const unsigned long long w[3][3]) {
         negative = M < 0;
@@ -286,7 +293,7 @@ __device__ __forceinline__ bool deposit_level_warp(WarpCharges& s, const LevelDe
     ok = ok && candidates(L, ic, e0, e1);
     if (!__any_sync(kFull, ok)) return false;
     // one charge width for the whole warp (the 32-bit products round the same way)
-    const bool wide = __any_sync(kFull, ok && (unsigned long long)M >= (1ULL << 32));
+    const bool wide = __any_sync(kFull, ok && M != 0 && !narrow_mass(M));
     if (!ok) e1 = e0;
     // the candidate grids in turn (one on the root and almost everywhere else)
     for (; __any_sync(kFull, e0 < e1); ++e0) {
