@@ -220,7 +220,10 @@ __device__ __forceinline__ void send_layer(const WarpCharges& s, int lane, unsig
             const unsigned o = s.off[3 + b][k];
             unsigned long long q = s.lo[a + 3 * b][k];
             if (WIDE) q |= (unsigned long long)s.hi[a + 3 * b][k] << 32;
-            if ((out | o) < kNoCell) asm volatile("red.global.add.u64 [%0], %1;" ::"l"(base + (xz + o)), "l"(q));
+            // a particle on a cell face has charges of zero (19 of 27 on a corner): not
+            // sent (16.8 M corner particles on 256^3: 1.01 -> 0.92 ms)
+            if ((out | o) < kNoCell && q != 0)
+                asm volatile("red.global.add.u64 [%0], %1;" ::"l"(base + (xz + o)), "l"(q));
         }
     }
 }
