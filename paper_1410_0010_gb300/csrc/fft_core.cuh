@@ -394,41 +394,29 @@ __device__ __forceinline__ void load_twiddles(C<T>* dst, const C<T>* __restrict_
 // chip (the FP64 rate, measured; the 32-bit ones at 32).  For
 // -2^47 <= q < 2^47 the FP32 path splits q = h 2^23 + l with h in
 // [-2^24, 2^24) and 0 <= l < 2^23, both exact in FP32, so h 2^23 + l is rounded
-// once, by the FMA: the same bits as __ll2float_rn.  Larger values (a cell of
-// 1/32 of the unit mass or more with the default 52 fraction bits) take the
-// instruction.
+// once, by the FMA: the same bits as __ll2float_rn.  A larger q (a cell of 1/32
+// of the unit mass or more with the default 52 fraction bits) first loses its
+// low 17 bits to a sticky one (bit 17 set if any of them is: rounding to odd);
+// at least 30 bits are left, 6 more than the result holds, so the one rounding
+// that follows gives the same bits again.  No branch: the loads of a thread's
+// cells are issued together, and every field takes the same time: a 512^3 root
+// 1705 us, where a first pass for small cells and the instruction in a second
+// one for CTAs with a large one took 1717 and 1858; the x + y planes of 27 grids
+// of 128^3 306 us against 302 and 340.
 template <typename T> __device__ __forceinline__ T fixed_to_real(long long q, T scale);
 template <> __device__ __forceinline__ double fixed_to_real<double>(long long q, double scale) {
     return __ll2double_rn(q) * scale;
 }
-// -2^47 <= q < 2^47
-__device__ __forceinline__ bool fits48(long long q) { return (unsigned)((int)(q >> 32) + 0x8000) < 0x10000u; }
-__device__ __forceinline__ float fixed48_to_float(long long q) {
-    const int h = (int)(q >> 23);
-    const float l = __uint_as_float(0x4b000000u | ((unsigned)q & 0x7fffffu)) - 8388608.0f;
-    return __fmaf_rn((float)h, 8388608.0f, l);
-}
 template <> __device__ __forceinline__ float fixed_to_real<float>(long long q, float scale) {
-    return (fits48(q) ? fixed48_to_float(q) : __ll2float_rn(q)) * scale;
-}
-// two complex values (a + i b), (c + i d) at once (the load passes convert two
-// cells of two rows per thread).  WIDE false: without the test, *wide set where
-// one of the four needed the instruction (the pass is then done again); a branch
-// per value would keep the compiler from issuing a thread's loads together.
-template <typename T, bool WIDE>
-__device__ __forceinline__ void fixed4_to_real(long long a, long long b, long long c, long long d, T scale, C<T>& u,
-                                               C<T>& v, bool& wide) {
-    if constexpr (sizeof(T) == 8) {
-        u = mk<T>(__ll2double_rn(a) * scale, __ll2double_rn(b) * scale);
-        v = mk<T>(__ll2double_rn(c) * scale, __ll2double_rn(d) * scale);
-    } else if constexpr (WIDE) {
-        u = mk<T>(__ll2float_rn(a) * scale, __ll2float_rn(b) * scale);
-        v = mk<T>(__ll2float_rn(c) * scale, __ll2float_rn(d) * scale);
-    } else {
-        wide = wide || !(fits48(a) && fits48(b) && fits48(c) && fits48(d));
-        u = mk<T>(fixed48_to_float(a) * scale, fixed48_to_float(b) * scale);
-        v = mk<T>(fixed48_to_float(c) * scale, fixed48_to_float(d) * scale);
-    }
+    unsigned lo = (unsigned)q;
+    int hi = (int)(q >> 32);
+    const bool large = (unsigned)(hi + 0x8000) >= 0x10000u;   // outside [-2^47, 2^47)
+    const unsigned odd = __funnelshift_r(lo, (unsigned)hi, 17) | ((lo & 0x1ffffu) != 0u ? 1u : 0u);
+    lo = large ? odd : lo;
+    hi = large ? hi >> 17 : hi;
+    const int h = (int)__funnelshift_r(lo, (unsigned)hi, 23);
+    const float l = __uint_as_float(0x4b000000u | (lo & 0x7fffffu)) - 8388608.0f;
+    return __fmaf_rn((float)h, 8388608.0f, l) * (large ? scale * 131072.0f : scale);
 }
 
 // 2^-F in T, 1 <= F <= 62

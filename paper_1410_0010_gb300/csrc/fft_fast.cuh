@@ -416,10 +416,10 @@ struct NoIO {};
 // xf: GMF rows -> half spectra along x, A[z][y][kx] (the layout of k_xf).
 // Load pass: the CTA's rows are one contiguous int64 range, read with
 // consecutive threads on consecutive pairs of cells of a row pair and
-// converted (hardware int64 -> float rounding, exact power-of-two scale);
-// positions past G0 and missing rows are zero.  Then the forward stages in place, and the separation of the
-// two real rows, A_k = (Z_k + conj Z_{L-k}) / 2, B_k = (Z_k - conj Z_{L-k}) / 2i,
-// written with consecutive threads on consecutive kx.
+// converted (fixed_to_real); positions past G0 and missing rows are zero.  Then
+// the forward stages in place, and the separation of the two real rows,
+// A_k = (Z_k + conj Z_{L-k}) / 2, B_k = (Z_k - conj Z_{L-k}) / 2i, written with
+// consecutive threads on consecutive kx.
 template <class P, int NP, int NT, typename T>
 __global__ void __launch_bounds__(NT) k_xf_fast(const GridDev* __restrict__ grids, const Chunk* __restrict__ chunks,
                                                 const int64_t* const* __restrict__ gmf,
@@ -440,8 +440,7 @@ __global__ void __launch_bounds__(NT) k_xf_fast(const GridDev* __restrict__ grid
     const T scale = pow2_neg<T>(F);
     // element (x, line p) = (row 2p, row 2p + 1) at x; one thread per pair of
     // positions of a line, with 16-byte loads of both rows when G0 is even
-    auto load = [&](auto wide_c) -> bool {
-        bool wide = false;
+    {
         constexpr int HALF = (L + 1) / 2;
         const bool vec = !(G0 & 1) && !(reinterpret_cast<size_t>(in) & 15);
 #pragma unroll 4
@@ -472,17 +471,12 @@ __global__ void __launch_bounds__(NT) k_xf_fast(const GridDev* __restrict__ grid
                     if (x1) b1 = r0[G0 + 1];
                 }
             }
-            C<T> u, v;
-            fixed4_to_real<T, decltype(wide_c)::value>(a0, b0, a1, b1, scale, u, v, wide);
-            buf[x * PITCH + p] = u;
-            if (L % 2 == 0 || x + 1 < L) buf[(x + 1) * PITCH + p] = v;
+            buf[x * PITCH + p] = mk<T>(fixed_to_real<T>(a0, scale), fixed_to_real<T>(b0, scale));
+            if (L % 2 == 0 || x + 1 < L)
+                buf[(x + 1) * PITCH + p] = mk<T>(fixed_to_real<T>(a1, scale), fixed_to_real<T>(b1, scale));
         }
-        return wide;
-    };
-    if (__syncthreads_or(load(std::false_type{}))) {
-        load(std::true_type{});
-        __syncthreads();
     }
+    __syncthreads();
     const NoIO none;
     fast_dif_stage<T, P, 0, NP, NT, false, false, NoIO, NoIO, PITCH>(buf, tw, none, none);
     __syncthreads();
@@ -650,16 +644,13 @@ __global__ void __launch_bounds__(NT) k_xi_fast(const GridDev* __restrict__ grid
 // complex line p, line storage LS): one thread per pair of x positions of a
 // row pair, with 16-byte loads of both rows (consecutive threads on
 // consecutive positions) and one 16-byte shared store of the two complex
-// values; converted exactly (hardware int64 -> float rounding, power-of-two
-// scale).  Positions G0 .. L-1 and the row G1 of an odd G1 are zero.  LS is
+// values, converted by fixed_to_real.  Positions G0 .. L-1 and the row G1 of an odd G1 are zero.  LS is
 // even (2 (L/2 + 1)), so the stores are 16-byte aligned; with an odd G0 the
 // last pair writes position G0 (a zero), which lies inside the line storage
 // (LS >= L + 1) and is read by no x stage when G0 = L.
-// WIDE: see fixed4_to_real; returns whether a cell needs the wide conversion.
-template <int L, int NT, int LS, bool WIDE>
-__device__ __forceinline__ bool xy_load_plane(float2* buf, const int64_t* __restrict__ in, int G0, int G1, int nl,
+template <int L, int NT, int LS>
+__device__ __forceinline__ void xy_load_plane(float2* buf, const int64_t* __restrict__ in, int G0, int G1, int nl,
                                               float scale) {
-    bool wide = false;
     const int half = (G0 + 1) / 2;   // position pairs per row
     const bool vec = !(G0 & 1) && !(reinterpret_cast<size_t>(in) & 15);
     const int items = nl * half;
@@ -690,9 +681,9 @@ __device__ __forceinline__ bool xy_load_plane(float2* buf, const int64_t* __rest
                 b1 = x1 ? r0[G0 + 1] : 0;
             }
         }
-        float2 u, v;
-        fixed4_to_real<float, WIDE>(a0, b0, a1, b1, scale, u, v, wide);
-        *reinterpret_cast<float4*>(buf + p * LS + x) = make_float4(u.x, u.y, v.x, v.y);
+        *reinterpret_cast<float4*>(buf + p * LS + x) =
+            make_float4(fixed_to_real<float>(a0, scale), fixed_to_real<float>(b0, scale),
+                        fixed_to_real<float>(a1, scale), fixed_to_real<float>(b1, scale));
         xp += dx;
         p += dp;
         if (xp >= half) {
@@ -702,7 +693,6 @@ __device__ __forceinline__ bool xy_load_plane(float2* buf, const int64_t* __rest
     }
     for (int q = threadIdx.x >> 5; q < nl; q += NT / 32)
         for (int t = 2 * half + (threadIdx.x & 31); t < L; t += 32) buf[q * LS + t] = make_float2(0.f, 0.f);
-    return wide;
 }
 // the plane's spectrum rows are H = L / 2 + 1 long: every offset is a constant
 // from the butterfly's first
@@ -794,11 +784,8 @@ __global__ void __launch_bounds__(NT, 2) k_xy_fast(const GridDev* __restrict__ g
     // rows 2 nl .. L-1 are the y transform's zero padding
     for (int t = threadIdx.x + 2 * nl * H; t < L * H; t += NT) buf[t] = make_float2(0.f, 0.f);
     const int64_t* const in = gmf[ch.grid] + (long long)z * G1 * G0;
-    // the barrier is the twiddles' and the x lines' too
-    if (__syncthreads_or(xy_load_plane<L, NT, 2 * H, false>(buf, in, G0, G1, nl, pow2_neg<float>(F)))) {
-        xy_load_plane<L, NT, 2 * H, true>(buf, in, G0, G1, nl, pow2_neg<float>(F));
-        __syncthreads();
-    }
+    xy_load_plane<L, NT, 2 * H>(buf, in, G0, G1, nl, pow2_neg<float>(F));
+    __syncthreads();   // twiddles and x lines
     const NoIO none;
     xy_x_stage<P, 0, NT, 2 * H>(buf, tw, nl);
     __syncthreads();
