@@ -169,17 +169,19 @@ constexpr int fast_lines(bool f64) { return f64 ? 8 : 16; }
 // threads of a fast pass CTA for `lines` lines: whole warps.  Up to L = 96, of 3
 // to 6 warps the count whose stages leave the fewest threads without a butterfly
 // in their last trip; above, 4 or, where that fits the first stage's butterflies,
-// 5; and as many as give 24 warps per SM with as many CTAs as the shared memory
-// of their lines lets in (128 bytes of each of L elements and a pad; 8 warps for
-// L = 512).  The z pass of 32 grids of L = 150: 264 us with 2 warps, 178 with 3,
-// 181 with 4, 171 with 5; 8 spectral ones of 120: 155 with 3, 131 with 4; 343
-// grids of 36 to 84: all passes 531 with 2 or more, 498 with 3 or more, 515 with
-// 3 always; the x forward of a 512^3 root: 671 with 4, 449 with 8.
+// 5; FP32 above 192 8, FP64 there as many as give 24 warps per SM (its pipe
+// bounds it: up to 320 it takes the same time with 4 to 8).  The z pass of 32
+// grids of L = 150: 264 us with 2 warps, 178 with 3, 181 with 4, 171 with 5; 8
+// spectral ones of 120: 155 with 3, 131 with 4; 343 grids of 36 to 84: all passes
+// 531 with 2 or more, 498 with 3 or more, 515 with 3 always.  A periodic root's
+// five passes with 4, 6 and 8 warps: 200^3 147, 139, 129 us; 240^3 228, 242, 196;
+// 256^3 251, 253, 215; 320^3 549, 497, 460; 512^3 2133, 1879, 1692.
 constexpr int fast_threads(int r1, int r2, int r3, int lines) {
     const int L = r1 * r2 * r3;
     const int items[3] = {L / r1 * lines, L / r2 * lines, r3 > 1 ? L / r3 * lines : 0};
+    if (L > 192 && lines == 16) return 256;
     if (L > 96) {
-        const int ctas = 220 * 1024 / (L * 17 * 8);
+        const int ctas = 220 * 1024 / (L * 17 * 8);   // per SM, by their shared memory
         int nt = items[0] > 128 && items[0] <= 160 ? 160 : 128;
         while (nt < 256 && nt * ctas < 768) nt += 32;
         return nt;
