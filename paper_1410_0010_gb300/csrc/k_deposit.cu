@@ -47,9 +47,11 @@ __global__ void __launch_bounds__(256) k_gas_init(LevelDev L, const GridDev* __r
     const double scale = ldexp(1.0, F);
     const double vol = __dmul_rn(__dmul_rn(g.delta, g.delta), g.delta);
     // when delta is a power of two, 2^e, the two products are exact exponent
-    // shifts and rint((rho delta^3) 2^F) = rint(rho 2^(F + 3e)), which
-    // scaled_rint_small computes with one FP64 addition (the FP64 products remain
-    // for other cell sizes and for values beyond its range)
+    // shifts and rint((rho delta^3) 2^F) = rint(rho 2^(F + 3e)): one FP64 addition,
+    // or from 2^50 units up integer operations (scaled_rint), where the products and
+    // the conversion would bound the pass (256^3 cells of half a unit mass: 226 us,
+    // so 116; small ones 92).  The products remain for other cell sizes and beyond
+    // 2^62.
     const unsigned long long db = (unsigned long long)__double_as_longlong(g.delta);
     const int de = (int)((db >> 52) & 0x7FF);
     const bool pow2 = (db & 0xFFFFFFFFFFFFFULL) == 0 && de > 0 && de < 0x7FF;
@@ -81,7 +83,7 @@ __global__ void __launch_bounds__(256) k_gas_init(LevelDev L, const GridDev* __r
         }
         if (APM_IN_BOUNDS((long long)r * G0 + x, g.cells_gmf, L.status)) {
             bool ok = false;
-            long long v = pow2 ? scaled_rint_small(rho, K, ok) : 0;
+            long long v = pow2 ? scaled_rint(rho, K, ok) : 0;
             if (!ok) v = __double2ll_rn(__dmul_rn(__dmul_rn(rho, vol), scale));
             row[x] = v;
         }
