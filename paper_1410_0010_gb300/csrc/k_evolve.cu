@@ -10,19 +10,30 @@ namespace apm {
 namespace {
 
 // What bounds this kernel is the FP64 pipe (2 lanes per clock and SM, measured;
-// a conversion to FP64 counts like an operation), not its 108 bytes a particle:
-// 7 operations per axis took 140 us for 4.2 M particles, the 5 that are left 100.
+// a conversion to FP64 counts like an operation) next to its 108 bytes a particle
+// (144 with FP64 accelerations): 7 operations per axis took 185 us for 4.2 M
+// particles, the 5 that are left 137; FP64 accelerations, 6 to 5, 162 and 137.
 // An FP32 acceleration is widened by moving its bits, and the half in
 // ((v + v') / 2) dt goes into dt: halving is exact on either factor, so the
 // product is rounded the same way.  Warps with a particle outside the ordinary
-// range (a zero, subnormal, infinite or NaN acceleration, or a sum small enough
-// to lose a bit in the halving) take the written-out form.
+// range convert (a zero, subnormal, infinite or NaN acceleration) or halve the sum
+// itself (one small enough to lose a bit, or a dt without a half), by integer
+// operations: with FP64 ones there the compiler issues those of both sides (FP64
+// accelerations: 205 us).
 __device__ __forceinline__ bool ordinary(double) { return true; }
 __device__ __forceinline__ bool ordinary(float a) { return ((__float_as_uint(a) >> 23) & 0xffu) - 1u < 254u; }
 __device__ __forceinline__ double widen(double a) { return a; }
 __device__ __forceinline__ double widen(float a) {
     const unsigned b = __float_as_uint(a);
     return __hiloint2double((int)((b & 0x80000000u) | (((b & 0x7fffffffu) >> 3) + 0x38000000u)), (int)(b << 29));
+}
+
+// s / 2, rounded to nearest even where a subnormal result loses a bit
+__device__ __forceinline__ double halved_any(double s) {
+    const unsigned long long b = (unsigned long long)__double_as_longlong(s), sign = b & (1ULL << 63), m = b ^ sign;
+    if (m >= 0x7ffULL << 52) return s;                                  // infinite, NaN
+    if (m >= 2ULL << 52) return __longlong_as_double((long long)(b - (1ULL << 52)));
+    return __longlong_as_double((long long)(((m + ((m >> 1) & 1)) >> 1) | sign));
 }
 
 template <typename T>
@@ -56,13 +67,14 @@ __global__ void __launch_bounds__(256) k_kick_drift(long long n, double* __restr
         s[j] = __dadd_rn(v[j], vn[j]);
         plain = plain && ((unsigned)__double2hiint(s[j]) & 0x7fffffffu) >= (2u << 20);
     }
-    if (__all_sync(0xffffffffu, plain)) {
+    plain = __all_sync(0xffffffffu, plain);
+    if (!plain) {
 #pragma unroll
-        for (int j = 0; j < 3; ++j) qn[j] = __dadd_rn(q[j], __dmul_rn(s[j], half_dt));
-    } else {
-#pragma unroll
-        for (int j = 0; j < 3; ++j) qn[j] = __dadd_rn(q[j], __dmul_rn(__dmul_rn(s[j], 0.5), dt));
+        for (int j = 0; j < 3; ++j) s[j] = halved_any(s[j]);
     }
+    const double f = plain ? half_dt : dt;
+#pragma unroll
+    for (int j = 0; j < 3; ++j) qn[j] = __dadd_rn(q[j], __dmul_rn(s[j], f));
     if (!live) return;
     x[p] = qn[0];
     y[p] = qn[1];
