@@ -372,7 +372,7 @@ constexpr unsigned long long kOne63 = 1ULL << 63;
 // exponent and significand with integer operations; kNoFixed for larger or
 // non-finite values.
 constexpr long long kNoFixed = (long long)(1ULL << 63);
-static __device__ __noinline__ long long scaled_rint_any(double x, int K) {
+__device__ __forceinline__ long long scaled_rint_bits(double x, int K) {
     const unsigned long long b = (unsigned long long)__double_as_longlong(x);
     const int e = (int)((b >> 52) & 0x7FF);
     if (e == 0x7FF) return kNoFixed;
@@ -394,12 +394,14 @@ static __device__ __noinline__ long long scaled_rint_any(double x, int K) {
     }
     return (b >> 63) ? -(long long)r : (long long)r;
 }
+static __device__ __noinline__ long long scaled_rint_any(double x, int K) { return scaled_rint_bits(x, K); }
 // The same, ok cleared in the place of kNoFixed (scaled_rint_small: and beyond
-// its range, |x 2^K| < 2^51).  For |x 2^K| < 2^51 (every coordinate and mass of an ordinary
-// problem) one FP64 addition rounds: x + 1.5 2^(52-K) lies where an FP64 unit in
-// the last place is 2^-K, so its significand holds rint(x 2^K), ties to even.
-// That is 16 clocks of the FP64 pipe for a warp, where the integer route takes
-// about 40 instructions.
+// its range, |x 2^K| < 2^51).  For |x 2^K| < 2^51 (every coordinate and mass of an
+// ordinary problem) one FP64 addition rounds: x + 1.5 2^(52-K) lies where an FP64
+// unit in the last place is 2^-K, so its significand holds rint(x 2^K), ties to
+// even.  That is 16 clocks of the FP64 pipe for a warp, where the integer route
+// takes about 40 instructions; BITS takes that one, for kernels the FP64 pipe
+// bounds (the FP64 interpolation).
 __device__ __forceinline__ long long scaled_rint_small(double x, int K, bool& ok) {
     const int e = (__double2hiint(x) >> 20) & 0x7FF;   // |x| < 2^(e - 1022)
     ok = e + K < 1073 && K > -900 && K < 1000;
@@ -407,10 +409,13 @@ __device__ __forceinline__ long long scaled_rint_small(double x, int K, bool& ok
     const double t = __dadd_rn(x, __hiloint2double(chi, 0));
     return __double_as_longlong(t) - ((long long)chi << 32);
 }
+template <bool BITS = false>
 __device__ __forceinline__ long long scaled_rint(double x, int K, bool& ok) {
-    const long long v = scaled_rint_small(x, K, ok);
-    if (ok) return v;
-    const long long r = scaled_rint_any(x, K);
+    if constexpr (!BITS) {
+        const long long v = scaled_rint_small(x, K, ok);
+        if (ok) return v;
+    }
+    const long long r = BITS ? scaled_rint_bits(x, K) : scaled_rint_any(x, K);
     ok = r != kNoFixed;
     return ok ? r : 0;
 }
@@ -437,15 +442,16 @@ __device__ __forceinline__ double drift_raw(double x, double v, double half_dt) 
 // X = rint(x'/delta0 2^31), canonical: modulo the box on a periodic domain; on
 // an isolated domain a coordinate inside [0, box) that rounds onto the upper
 // face stays in the last cell
+template <bool BITS = false>
 __device__ __forceinline__ long long fixed_position(double xd, const LevelDev& L) {
     // a coordinate 2^31 root cells or more from the origin (or NaN) saturates at
     // -+2^62: far outside every box
     long long X;
     bool ok;
     if (L.delta0_pow2) {
-        X = scaled_rint(xd, L.pos_exp, ok);
+        X = scaled_rint<BITS>(xd, L.pos_exp, ok);
     } else {
-        X = scaled_rint(div_known(xd, L.delta0, L.inv_delta0, L.div_known != 0), 31, ok);
+        X = scaled_rint<BITS>(div_known(xd, L.delta0, L.inv_delta0, L.div_known != 0), 31, ok);
     }
     if (!ok) X = xd > 0.0 ? (1LL << 62) : -(1LL << 62);
     if (L.periodic) {

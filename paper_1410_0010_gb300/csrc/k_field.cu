@@ -433,11 +433,13 @@ __device__ __forceinline__ void interp_from(const LevelDev& L, const GridDev& g,
     out[2 * n + p] = a2;
 }
 
+template <typename T>
 __device__ __forceinline__ void particle_position(const LevelDev& L, const Particles& P, long long p,
                                                   double half_dt, long long X[3]) {
-    X[0] = fixed_position(drift_raw(P.x[p], P.vx[p], half_dt), L);
-    X[1] = fixed_position(drift_raw(P.y[p], P.vy[p], half_dt), L);
-    X[2] = fixed_position(drift_raw(P.z[p], P.vz[p], half_dt), L);
+    constexpr bool kBits = sizeof(T) == 8;
+    X[0] = fixed_position<kBits>(drift_raw(P.x[p], P.vx[p], half_dt), L);
+    X[1] = fixed_position<kBits>(drift_raw(P.y[p], P.vy[p], half_dt), L);
+    X[2] = fixed_position<kBits>(drift_raw(P.z[p], P.vz[p], half_dt), L);
 }
 
 // One level: the particles owned by a grid of L and by no grid of the finer
@@ -451,7 +453,7 @@ __global__ void __launch_bounds__(256) k_interp(LevelDev L, LevelDev F, int has_
     if (i >= P.n) return;
     const long long p = P.at(i);
     long long X[3];
-    particle_position(L, P, p, half_dt, X);
+    particle_position<T>(L, P, p, half_dt, X);
     long long ic[3];
     for (int j = 0; j < 3; ++j) ic[j] = X[j] >> L.frac_bits;
     int gi = find_owner(L, ic);
@@ -486,7 +488,7 @@ __global__ void __launch_bounds__(kIntThreads, APM_INT_MIN_CTAS) k_interp_levels
     if (i >= P.n) return;
     const long long p = P.at(i);
     long long X[3];
-    particle_position(levels[0], P, p, half_dt, X);
+    particle_position<T>(levels[0], P, p, half_dt, X);
     int own_l = -1, own_g = -1;
     for (int l = 0; l < nl; ++l) {
         long long ic[3];
