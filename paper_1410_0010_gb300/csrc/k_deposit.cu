@@ -170,12 +170,10 @@ template <typename V> struct LaneCharges {
             for (int b = 0; b < 3; ++b) mxy[a + 3 * b] = mul63w(mx, w[1][b]);
         }
     }
-    __device__ __forceinline__ void layer(WarpCharges& s, int lane, int c, const unsigned long long w[3][3]) {
+    // put(k, charge) for the cells k = a + 3 b of layer c
+    template <class PUT>
+    __device__ __forceinline__ void layer(int c, const unsigned long long w[3][3], PUT put) {
         const unsigned long long wz = c == 0 ? w[2][0] : (c == 1 ? w[2][1] : w[2][2]);
-        auto put = [&](int k, V v) {
-            s.lo[k][lane] = (unsigned)v;
-            if constexpr (sizeof(V) == 8) s.hi[k][lane] = (unsigned)(v >> 32);
-        };
 #pragma unroll
         for (int k = 0; k < 9; ++k) {
             if (k == 4 && c == 1) continue;
@@ -189,15 +187,17 @@ template <typename V> struct LaneCharges {
 };
 
 // the cells of this lane's cloud in grid g (centre cell ic) as summable offsets
+// (a centre cell beyond [-2, G + 1], an isolated root's particle outside the box,
+// folds like these do)
+__device__ __forceinline__ int local_centre(const GridDev& g, const long long ic[3], int j) {
+    return (int)min(max(ic[j] - g.lo[j], -2LL), (long long)g.G[j] + 1);
+}
 __device__ __forceinline__ void lane_cells(WarpCharges& s, int lane, const GridDev& g, const long long ic[3],
                                            unsigned* __restrict__ status) {
     const unsigned st[3] = {1u, (unsigned)g.G[0], (unsigned)g.G[0] * (unsigned)g.G[1]};
 #pragma unroll
     for (int j = 0; j < 3; ++j) {
-        const int G = g.G[j];
-        // a centre cell beyond [-2, G + 1] (an isolated root's particle outside
-        // the box) folds like these do
-        const int r = (int)min(max(ic[j] - g.lo[j], -2LL), (long long)G + 1);
+        const int G = g.G[j], r = local_centre(g, ic, j);
 #pragma unroll
         for (int k = 0; k < 3; ++k) {
             const int v = edge_rule(r + k - 1, G, g.mode);
@@ -246,7 +246,11 @@ __device__ __forceinline__ void send_clouds(WarpCharges& s, int lane, bool act, 
 #pragma unroll 1
     for (int k = 0; k < 3; ++k) {
         const int c = k == 0 ? 0 : 3 - k;   // 0, 2, 1
-        if (act) q.layer(s, lane, c, w);
+        if (act)
+            q.layer(c, w, [&](int j, V v) {
+                s.lo[j][lane] = (unsigned)v;
+                if constexpr (kWide) s.hi[j][lane] = (unsigned)(v >> 32);
+            });
         __syncwarp();
         send_layer<kWide>(s, lane, live, c);
         __syncwarp();
@@ -279,12 +283,145 @@ __device__ __forceinline__ bool candidates(const LevelDev& L, const long long ic
     return e0 != e1;
 }
 
-// The warp's deposit into the grids of one level: this lane's particle at
-// fixed-point position X with integer mass M (ok false: none).  Every lane of
-// the warp calls it.  False when this lane's particle is not a candidate of
+// ---- particles in bin order: a CTA's clouds gathered in a box ----
+// In bin order a CTA's particles lie close together, and where many share cells
+// (a halo's core) it adds their charges in shared memory and sends one reduction
+// per cell of the box around them, where the box of its clouds in one grid holds at
+// most kBoxPerParticle cells for each of its particles (and fits the row charges'
+// memory); elsewhere the warps send their rows.  A sum is two 32-bit words: of
+// 32-bit charges the low and the high halves (at most 128 particles add less than
+// 2^23 to either, and no carry is waited for), of 64-bit ones the low word, whose
+// carry goes to the high one.  Integer sums do not depend on the order: the same
+// field.  Rows only -> boxes, 1 M particles: a Plummer sphere on 256^3 281 -> 132
+// us, on 64^3 570 -> 114, on 64^3 with one nested level 864 -> 188, through three
+// levels 562 -> 344; at random places on 256^3 180 -> 181, on 64^3 139 -> 111.  With 6
+// cells for each particle the two nested ones take 531 and 482, with 18 the same.
+constexpr int kBoxCells = (int)(sizeof(WarpCharges) * (kDepThreads / 32) / 8);
+#ifndef APM_DEP_BOX
+#define APM_DEP_BOX 12
+#endif
+constexpr int kBoxPerParticle = APM_DEP_BOX;
+struct Box {
+    int lo[3], n[3];   // first cell (GMF-local, before the edge rule) and extents
+    int cells;         // 0: none
+    int gi;            // the grid
+};
+struct BoxShared {
+    int lo[kDepThreads / 32][4], hi[kDepThreads / 32][4], count[kDepThreads / 32];
+};
+// the box of the CTA's acting lanes at the centre cells r of grid gi (lanes with
+// other candidates beside it: one = false).  Every thread calls it.
+__device__ __forceinline__ Box cta_box(BoxShared& b, bool act, bool one, int gi, const int r[3]) {
+    constexpr unsigned kFull = 0xffffffffu;
+    const int warp = threadIdx.x >> 5;
+    const int v[4] = {r[0], r[1], r[2], one ? gi : -1};
+#pragma unroll
+    for (int j = 0; j < 4; ++j) {
+        const int lo = __reduce_min_sync(kFull, act ? v[j] : 0x7fffffff);
+        const int hi = __reduce_max_sync(kFull, act ? v[j] : -0x7fffffff);
+        if ((threadIdx.x & 31) == 0) {
+            b.lo[warp][j] = lo;
+            b.hi[warp][j] = hi;
+        }
+    }
+    const int count = __popc(__ballot_sync(kFull, act));
+    if ((threadIdx.x & 31) == 0) b.count[warp] = count;
+    __syncthreads();
+    int lo[4], hi[4], total = 0;
+#pragma unroll
+    for (int j = 0; j < 4; ++j) {
+        lo[j] = 0x7fffffff;
+        hi[j] = -0x7fffffff;
+#pragma unroll
+        for (int w = 0; w < kDepThreads / 32; ++w) {
+            lo[j] = min(lo[j], b.lo[w][j]);
+            hi[j] = max(hi[j], b.hi[w][j]);
+        }
+    }
+#pragma unroll
+    for (int w = 0; w < kDepThreads / 32; ++w) total += b.count[w];
+    __syncthreads();   // read by every warp
+    Box x;
+    x.gi = lo[3];
+    x.cells = 0;
+    if (total == 0 || lo[3] < 0 || lo[3] != hi[3]) return x;
+    long long cells = 1;
+#pragma unroll
+    for (int j = 0; j < 3; ++j) {
+        x.lo[j] = lo[j] - 1;
+        x.n[j] = hi[j] - lo[j] + 3;
+        cells *= x.n[j];   // extents below 2^21
+    }
+    if (cells <= min(kBoxCells, kBoxPerParticle * total)) x.cells = (int)cells;
+    return x;
+}
+// this lane's cloud (centre cell r) into the box
+template <typename V>
+__device__ __forceinline__ void box_add(unsigned* __restrict__ lo, unsigned* __restrict__ hi, const Box& x,
+                                        const int r[3], long long M, const unsigned long long w[3][3]) {
+    LaneCharges<V> q;
+    q.start(M, w);
+    const int n01 = x.n[0] * x.n[1];
+    const int first = (r[0] - 1 - x.lo[0]) + x.n[0] * (r[1] - 1 - x.lo[1]) + n01 * (r[2] - 1 - x.lo[2]);
+#pragma unroll 1
+    for (int k = 0; k < 3; ++k) {
+        const int c = k == 0 ? 0 : 3 - k;   // 0, 2, 1
+        q.layer(c, w, [&](int j, V v) {
+            const int at = first + c * n01 + (j % 3) + x.n[0] * (j / 3);
+            if constexpr (sizeof(V) == 4) {
+                if (v & 0xffffu) atomicAdd(lo + at, v & 0xffffu);
+                if (v >> 16) atomicAdd(hi + at, v >> 16);
+            } else {
+                const unsigned l = (unsigned)v;
+                const unsigned old = atomicAdd(lo + at, l);
+                const unsigned h = (unsigned)(v >> 32) + (old + l < old ? 1u : 0u);
+                if (h) atomicAdd(hi + at, h);
+            }
+        });
+    }
+}
+// every acting lane's cloud into the box, then one reduction per cell that is not
+// zero; words: kBoxCells low and high words.  Every thread calls it.
+__device__ __forceinline__ void box_deposit(unsigned* __restrict__ words, const Box& x, const GridDev& g, bool act,
+                                            const int r[3], long long M, const long long X[3], int P,
+                                            int64_t* __restrict__ out, unsigned* __restrict__ status) {
+    unsigned* const lo = words;
+    unsigned* const hi = words + x.cells;
+    for (int k = threadIdx.x; k < 2 * x.cells; k += kDepThreads) words[k] = 0u;
+    // one width of charges for the CTA
+    const bool wide = __syncthreads_or(act && M != 0 && !narrow_mass(M));
+    if (act && M != 0) {
+        unsigned long long w[3][3];
+#pragma unroll
+        for (int j = 0; j < 3; ++j) tsc_fixed(X[j], P, w[j]);
+        if (wide) box_add<unsigned long long>(lo, hi, x, r, M, w);
+        else box_add<unsigned>(lo, hi, x, r, M, w);
+    }
+    __syncthreads();
+    const unsigned G0 = g.G[0], G01 = (unsigned)g.G[0] * (unsigned)g.G[1];
+    for (int k = threadIdx.x; k < x.cells; k += kDepThreads) {
+        const unsigned long long v =
+            wide ? ((unsigned long long)hi[k] << 32 | lo[k]) : ((unsigned long long)hi[k] << 16) + lo[k];
+        if (v == 0) continue;
+        const int yz = k / x.n[0], cz = yz / x.n[1];
+        const int c0 = edge_rule(x.lo[0] + k - yz * x.n[0], g.G[0], g.mode);
+        const int c1 = edge_rule(x.lo[1] + yz - cz * x.n[1], g.G[1], g.mode);
+        const int c2 = edge_rule(x.lo[2] + cz, g.G[2], g.mode);
+        if ((c0 | c1 | c2) < 0) continue;
+        const unsigned at = (unsigned)c0 + G0 * (unsigned)c1 + G01 * (unsigned)c2;
+        if (APM_IN_BOUNDS(at, g.cells_gmf, status))
+            asm volatile("red.global.add.u64 [%0], %1;" ::"l"(out + at), "l"(v));
+    }
+    __syncthreads();   // the words are the warps' row charges too
+}
+
+// The deposit into the grids of one level: this lane's particle at fixed-point
+// position X with integer mass M (ok false: none).  Every lane of the warp calls
+// it, ORDERED every thread of the CTA.  False when this lane's particle is not a candidate of
 // the level (then it is none of a finer level's either: finer GMF boxes lie
 // inside the interiors of their parents).
-__device__ __forceinline__ bool deposit_level_warp(WarpCharges& s, const LevelDev& L, const long long X[3],
+template <bool ORDERED>
+__device__ __forceinline__ bool deposit_level_warp(WarpCharges* charges, BoxShared* box, const LevelDev& L, const long long X[3],
                                                    long long M, bool ok, bool outside,
                                                    int64_t* const* __restrict__ gmf,
                                                    unsigned* __restrict__ status) {
@@ -296,6 +433,19 @@ __device__ __forceinline__ bool deposit_level_warp(WarpCharges& s, const LevelDe
     for (int j = 0; j < 3; ++j) ic[j] = X[j] >> PB;
     int e0 = 0, e1 = 0;
     ok = ok && candidates(L, ic, e0, e1);
+    if constexpr (ORDERED) {
+        if (!__syncthreads_or(ok)) return false;
+        const int gi = !ok ? 0 : (L.is_root ? 0 : L.map.dep_list[e0]);
+        const GridDev& g = L.g[gi];
+        const int r[3] = {local_centre(g, ic, 0), local_centre(g, ic, 1), local_centre(g, ic, 2)};
+        const Box x = cta_box(*box, ok, e1 - e0 == 1, gi, r);
+        if (x.cells > 0) {
+            if (ok && g.mode == 1 && outside) atomicOr(status, kStOutOfBox);
+            box_deposit(reinterpret_cast<unsigned*>(charges), x, L.g[x.gi], ok, r, M, X, PB, gmf[x.gi], status);
+            return ok;
+        }
+    }
+    WarpCharges& s = charges[threadIdx.x >> 5];
     if (!__any_sync(kFull, ok)) return false;
     // one charge width for the whole warp (the 32-bit products round the same way)
     const bool wide = __any_sync(kFull, ok && M != 0 && !narrow_mass(M));
@@ -367,36 +517,44 @@ __device__ __forceinline__ long long first_slot(const Particles& P, unsigned b) 
     return (long long)b * kDepThreads;
 }
 
-// One level, in the caller's order.
+// One level.  ORDERED: in bin order.
+template <bool ORDERED>
 __global__ void __launch_bounds__(kDepThreads, APM_DEP_MIN_CTAS) k_deposit(LevelDev L, Particles P, double half_dt,
                                                  double box, int F,
                                                  int64_t* const* __restrict__ gmf,
                                                  unsigned* __restrict__ status) {
     const unsigned block = begin_kernel();
     __shared__ WarpCharges charges[kDepThreads / 32];
+    __shared__ BoxShared cta[1];
     const long long i = first_slot(P, block) + threadIdx.x;
     long long X[3] = {0, 0, 0}, M = 0;
     bool outside = false;
     const bool ok = i < P.n && particle_of_level(L, P, i, half_dt, box, F, X, &M, &outside, status);
-    deposit_level_warp(charges[threadIdx.x >> 5], L, X, M, ok, outside, gmf, status);
+    deposit_level_warp<ORDERED>(charges, cta, L, X, M, ok, outside, gmf, status);
 }
 
 // Every level in one pass over the particles: the position and mass are
 // converted once, then deposited level by level from the root down while the
 // particle is a candidate.  levels: the LevelDev of each level; gmfs[l]: the
 // GMF pointer table of level l.
+template <bool ORDERED>
 __global__ void __launch_bounds__(kDepThreads, APM_DEP_MIN_CTAS) k_deposit_levels(
     const LevelDev* __restrict__ levels, int nl, Particles P, double half_dt, double box, int F,
     int64_t* const* const* __restrict__ gmfs, unsigned* __restrict__ status) {
     const unsigned block = begin_kernel();
     __shared__ WarpCharges charges[kDepThreads / 32];
+    __shared__ BoxShared cta[1];
     const long long i = first_slot(P, block) + threadIdx.x;
     long long X[3] = {0, 0, 0}, M = 0;
     bool outside = false, ok = false;
     if (i < P.n) ok = particle_fixed(levels[0], P, P.at(i), half_dt, box, F, X, &M, &outside, status);
     for (int l = 0; l < nl; ++l) {
-        ok = deposit_level_warp(charges[threadIdx.x >> 5], levels[l], X, M, ok, l == 0 && outside, gmfs[l], status);
-        if (!__any_sync(0xffffffffu, ok)) break;
+        ok = deposit_level_warp<ORDERED>(charges, cta, levels[l], X, M, ok, l == 0 && outside, gmfs[l], status);
+        if constexpr (ORDERED) {   // the CTA's box needs all its warps
+            if (!__syncthreads_or(ok)) break;
+        } else {
+            if (!__any_sync(0xffffffffu, ok)) break;
+        }
     }
 }
 
@@ -411,10 +569,10 @@ cudaError_t launch_gas_init(const LevelDev& L, const GridDev* parent_grids,
 }
 
 // In bin order the CTAs that run together would add into the same few cells
-// where many particles share them; a golden-ratio stride through the CTAs
-// spreads them over the bins, and each CTA keeps its own bin's locality.  The
-// Plummer sphere 690 -> 417 us (caller's order 396), the random particles 647
-// -> 707 (926).
+// where many particles share them and no box gathers them; a golden-ratio stride
+// through the CTAs spreads them over the bins, and each CTA keeps its own bin's
+// locality.  A Plummer sphere of 1 M through three nested levels 413 -> 344 us
+// (caller's order 551); random places on 256^3 166 -> 182 (246).
 static Particles deposit_order(Particles P, unsigned blocks) {
     P.stride = 0;
     if (P.perm && blocks > 2) {
@@ -436,8 +594,8 @@ cudaError_t launch_deposit(const LevelDev& L, const Particles& P, double half_dt
                            int F, int64_t* const* gmf, unsigned* status, cudaStream_t s) {
     if (P.n <= 0) return cudaSuccess;
     unsigned blocks = (unsigned)((P.n + kDepThreads - 1) / kDepThreads);
-    return launch_kernel(k_deposit, blocks, kDepThreads, 0, s, L, deposit_order(P, blocks), half_dt, box, F, gmf,
-                         status);
+    return launch_kernel(P.perm ? k_deposit<true> : k_deposit<false>, blocks, kDepThreads, 0, s, L,
+                         deposit_order(P, blocks), half_dt, box, F, gmf, status);
 }
 
 cudaError_t launch_deposit_levels(const LevelDev* levels, int nl, const Particles& P, double half_dt,
@@ -445,8 +603,8 @@ cudaError_t launch_deposit_levels(const LevelDev* levels, int nl, const Particle
                                   cudaStream_t s) {
     if (P.n <= 0 || nl <= 0) return cudaSuccess;
     unsigned blocks = (unsigned)((P.n + kDepThreads - 1) / kDepThreads);
-    return launch_kernel(k_deposit_levels, blocks, kDepThreads, 0, s, levels, nl, deposit_order(P, blocks),
-                         half_dt, box, F, gmfs, status);
+    return launch_kernel(P.perm ? k_deposit_levels<true> : k_deposit_levels<false>, blocks, kDepThreads, 0, s, levels,
+                         nl, deposit_order(P, blocks), half_dt, box, F, gmfs, status);
 }
 
 }  // namespace apm

@@ -231,8 +231,9 @@ class Solver:
 
     def set_deposit_tiles(self, on):
         """True: while a particle order is current, the deposits visit the
-        particles in it too (bit-identical; pays for particles in no spatial
-        order).  Default off."""
+        particles in it too, and gather the charges of those that share cells
+        (bit-identical; pays for clustered particles, and for unordered ones
+        on a large field).  Default off."""
         check(lib().apm_set_deposit_tiles(self._ctx, 1 if on else 0), "apm_set_deposit_tiles")
 
     def fft_shapes(self, level):
