@@ -335,12 +335,13 @@ apm_status apm_set_deposit_tiles(apm_ctx* ctx, int32_t on);
  *             200, 216, 224, 240, 250, 256, 288, 300, 320, 360, 384, 400, 480
  *             and 512, FP64 the same ones from 70 up; FP32 grids with
  *             M0 = M1 from 70 to 192 run the x and y transforms of a whole z
- *             plane in one kernel (the y pass then has no work for them; the
- *             inverse needs the window no taller than M1, which excludes a
- *             periodic root); 1: every grid runs the runtime-planned kernel;
- *             2 (x forward and x inverse only): as 0, with the plane kernels
- *             for every FP32 grid with M0 = M1 whose M x (M/2 + 1) plane fits
- *             200 KB;
+ *             plane in one kernel where the y pass has plan 0 too (it then has
+ *             no work for them; the inverse needs the window no taller than
+ *             M1, which excludes a periodic root); 1: every grid runs the
+ *             runtime-planned kernel; 2 (x forward and x inverse only): as 0,
+ *             with the plane kernels for every FP32 grid with M0 = M1 whose
+ *             M x (M/2 + 1) plane fits 200 KB, whatever the y pass's plan; 3
+ *             (the same two): as 0, without the plane kernels;
  *  max_radix  the largest stage radix of the runtime plans: 16 (FP32
  *             default; composite radices in registers) or 8 (FP64: always 8);
  *  packing    0: the grids of a level enter each work list in hierarchy order;
@@ -363,9 +364,12 @@ typedef struct {
  * while timing every candidate shape of each FFT pass in turn (budgets
  * 512..8192 (FP32) or 256..4096 (FP64) by powers of two, 128 or 256 threads;
  * the fastest of five timed launches after a warm one, CUDA events on
- * `stream`), then, over the whole level's passes, each pass's plan (FP32),
- * the packing and the runtime plans' largest radix (FP32), one at a time, and
- * keeps the fastest choices for the context's later calls.  phi_short
+ * `stream`; none on a pass whose grids all run compile-time plans, which have
+ * one shape), then, over the whole level's passes, each pass's plan (FP32),
+ * the plane kernels against the unfused passes (FP32), the packing and the
+ * runtime plans' largest radix (FP32), one at a time and where it changes a
+ * kernel, and keeps the fastest choices for the context's later calls (FP64
+ * keeps plan 0, and with it its bits).  phi_short
  * holds the level's potential on return.  Synchronises `stream` and the
  * device several times: APM_E_STATE while `stream` is being captured. */
 apm_status apm_autotune_level(apm_ctx* ctx, int32_t level, const int64_t* const* gmf,

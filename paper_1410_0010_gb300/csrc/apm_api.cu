@@ -356,6 +356,37 @@ int fast_kernel(int q, int kind, int comp) {
     }
 }
 
+// the transform length of pass q on grid g
+int pass_length(int q, const GridDev& g) {
+    return q == kPassXf || q == kPassXi ? g.M[0] : (q == kPassZ ? g.M[2] : g.M[1]);
+}
+
+// The kernel of pass q on grid g with the passes' plans `plan`: L, the
+// compile-time plan of its length; -L, the fused planes; kSkip, nothing (its x
+// pass runs the planes); 0, the runtime-planned kernel.  A spectral gradient's
+// components run the z pass on the same work list (k_col_fast MODE 3, or k_col
+// MODE 3).
+constexpr int kSkip = INT_MIN;
+int pass_kind(int q, bool f64, const GridDev& g, const int* plan) {
+    const bool fwd = q == kPassXf || q == kPassYf;
+    const int x_pass = fwd ? kPassXf : kPassXi, y_pass = fwd ? kPassYf : kPassYi;
+    if (!fft_fast_enabled()) return 0;
+    // the bulk-copy wait that is made to run out is the runtime x forward's
+    if (fwd && fault_wait() && q == kPassXf) return 0;
+    // the fused planes: plan 2 on the x pass, or plan 0 on the x and the y pass and
+    // a length of fast_xy_default (plan 3: never).  The forward stores row pair p
+    // in plane rows 2p, 2p + 1: an odd G1 needs G1 < M1.  The inverse needs the
+    // window's row pairs to be distinct rows of the transform (a periodic root,
+    // whose window is taller than M1, is excluded) and its rows no longer than the
+    // transform's.
+    const bool asked = plan[x_pass] == 2 || (plan[x_pass] == 0 && plan[y_pass] == 0 && fast_xy_default(g.M[0]));
+    if (q != kPassZ && !f64 && asked && g.M[0] == g.M[1] && fast_xy_length(g.M[0]) && !(fwd && fault_wait()) &&
+        (fwd ? 2 * ((g.G[1] + 1) / 2) <= g.M[1] : 2 * ((g.W[1] + 1) / 2) <= g.M[1] && g.W[0] <= g.M[0]))
+        return q == x_pass ? -g.M[0] : kSkip;
+    const int len = pass_length(q, g);
+    return plan[q] != 1 && fast_length(len, f64) ? len : 0;
+}
+
 // Work list of FFT pass q over the grids of a level for a buffer budget and a
 // CTA size: each grid's lines per CTA (halved until the CTA fits its shared
 // memory), one chunk per CTA.  The lines batch whole lines, so the shape never
@@ -369,43 +400,9 @@ apm_status build_pass(apm_ctx* c, const Level& L, int q, int budget, int threads
     P.count.assign(ng, 0);
     P.seg_of.assign(ng, 0);
     P.seg.clear();
-    // the kernel of each grid: the compile-time plan of its length, if there is
-    // one (not for the x-forward pass while its bulk-copy
-    // wait is made to run out); a spectral gradient's components run the z pass
-    // on the same work list (k_col_fast MODE 3, or k_col MODE 3)
-    std::vector<int> fast(ng, 0), lens(ng, 0);
+    std::vector<int> fast(ng);
+    for (int k = 0; k < ng; ++k) fast[k] = pass_kind(q, f64, L.hg[k], L.plan);
     const bool row = q == kPassXf || q == kPassXi;
-    // with plan 2 on the x-forward pass (or plan 0 and a length of
-    // fast_xy_default), a grid with M0 = M1 whose plane fits runs the fused x + y
-    // forward (k_xy_fast) as its x-forward segment (kind -L) and has no y-forward
-    // work (kind kSkip); other grids run plan 0
-    constexpr int kSkip = INT_MIN;
-    auto fuses = [&](int x_pass, int len) {
-        return L.plan[x_pass] == 2 || (L.plan[x_pass] == 0 && fast_xy_default(len));
-    };
-    // (the kernel stores row pair p in plane rows 2p, 2p + 1: an odd G1 needs
-    // G1 < M1, so that the pairs fit the M1 rows of the plane)
-    auto fused_xy = [&](const GridDev& g) {
-        return !f64 && fuses(kPassXf, g.M[0]) && fft_fast_enabled() && !fault_wait() && g.M[0] == g.M[1] &&
-               fast_xy_length(g.M[0]) && 2 * ((g.G[1] + 1) / 2) <= g.M[1];
-    };
-    // ... and the fused y + x inverse (k_yx_fast) as its x-inverse segment when
-    // the window's row pairs are distinct rows of the transform (2 ceil(W1/2)
-    // <= M1: a periodic root, whose window is taller than M1, is excluded) and
-    // its rows no longer than the transform's
-    auto fused_yx = [&](const GridDev& g) {
-        return !f64 && fuses(kPassXi, g.M[0]) && fft_fast_enabled() && g.M[0] == g.M[1] && fast_xy_length(g.M[0]) &&
-               2 * ((g.W[1] + 1) / 2) <= g.M[1] && g.W[0] <= g.M[0];
-    };
-    for (int k = 0; k < ng; ++k) {
-        const GridDev& g = L.hg[k];
-        lens[k] = row ? g.M[0] : (q == kPassZ ? g.M[2] : g.M[1]);
-        if (L.plan[q] != 1 && fft_fast_enabled() && fast_length(lens[k], f64) &&
-            !(q == kPassXf && fault_wait()))
-            fast[k] = lens[k];
-        if ((q == kPassXf || q == kPassYf) && fused_xy(g)) fast[k] = q == kPassXf ? -lens[k] : kSkip;
-        if ((q == kPassXi || q == kPassYi) && fused_yx(g)) fast[k] = q == kPassXi ? -lens[k] : kSkip;
-    }
     std::vector<int> kinds(fast);
     std::sort(kinds.begin(), kinds.end());
     kinds.erase(std::unique(kinds.begin(), kinds.end()), kinds.end());
@@ -433,7 +430,7 @@ apm_status build_pass(apm_ctx* c, const Level& L, int q, int budget, int threads
         for (int k : order) {
             if (fast[k] != kind) continue;
             const GridDev& g = L.hg[k];
-            const int len = lens[k];
+            const int len = pass_length(q, g);
             if (kind < 0) {             // fused x + y passes: one chunk per z (window) plane
                 P.lines[k] = fast_lines(f64);
                 P.first[k] = (int)list.size();
@@ -1395,6 +1392,12 @@ apm_status apm_autotune_level(apm_ctx* c, int32_t level, const int64_t* const* g
         *ms = best;
         return APM_OK;
     };
+    // every grid of pass q runs a compile-time plan
+    auto all_planned = [&](int q) {
+        for (const GridDev& g : L.hg)
+            if (pass_kind(q, f64, g, L.plan) == 0) return false;
+        return true;
+    };
     // the launch shapes are those of the runtime-planned kernels: tune them with
     // every pass on that kernel, then choose each pass's plan below
     const int plan0[kFftPasses] = {L.plan[0], L.plan[1], L.plan[2], L.plan[3], L.plan[4]};
@@ -1417,7 +1420,8 @@ apm_status apm_autotune_level(apm_ctx* c, int32_t level, const int64_t* const* g
                 PassPlan cand;
                 if ((st = build_pass(c, L, q, budgets[bi], t, f64, cand)) != APM_OK) break;
                 float ms = 0;
-                const bool same = cand.lines == L.pass[q].lines && cand.threads == L.pass[q].threads;
+                // compile-time plans have one shape: there is nothing to compare
+                const bool same = all_planned(q) || (cand.lines == L.pass[q].lines && cand.threads == L.pass[q].threads);
                 if (!same && (st = time_pass(q, cand, &ms)) == APM_OK && ms < best_ms) {
                     best_ms = ms;
                     dfree(c, L.pass[q].d);
@@ -1469,6 +1473,13 @@ apm_status apm_autotune_level(apm_ctx* c, int32_t level, const int64_t* const* g
         *ms = best;
         return APM_OK;
     };
+    // whether the plans `alt` run the kernels that L.plan does
+    auto same_kernels = [&](const int* alt) {
+        for (int q = 0; q < kFftPasses; ++q)
+            for (const GridDev& g : L.hg)
+                if (pass_kind(q, f64, g, alt) != pass_kind(q, f64, g, L.plan)) return false;
+        return true;
+    };
     // one knob at a time: keep the candidate when it is faster, else restore
     auto try_knob = [&](auto set, auto restore) -> apm_status {
         float base = 0, cand = 0;
@@ -1481,38 +1492,45 @@ apm_status apm_autotune_level(apm_ctx* c, int32_t level, const int64_t* const* g
         return rebuild();
     };
     if (st == APM_OK && !f64) {
-        // each pass: the compile-time plan (where its lengths have one) against
-        // the tuned runtime-planned kernel
+        // each pass: the compile-time plan (where its lengths have one; on the x
+        // passes without the planes) against the tuned runtime-planned kernel
         for (int q = 0; q < kFftPasses && st == APM_OK; ++q) {
             bool any_fast = false;
-            for (int k = 0; k < (int)L.hg.size(); ++k) {
-                const GridDev& g = L.hg[k];
-                const int len = (q == kPassXf || q == kPassXi) ? g.M[0] : (q == kPassZ ? g.M[2] : g.M[1]);
-                any_fast = any_fast || fast_length(len, f64);
-            }
+            for (const GridDev& g : L.hg) any_fast = any_fast || fast_length(pass_length(q, g), f64);
+            const bool x = q == kPassXf || q == kPassXi;
             if (any_fast && fft_fast_enabled())
-                st = try_knob([&] { L.plan[q] = 0; }, [&] { L.plan[q] = 1; });
+                st = try_knob([&] { L.plan[q] = x ? 3 : 0; }, [&] { L.plan[q] = 1; });
             else
                 L.plan[q] = plan0[q];
         }
         if (st == APM_OK) st = rebuild();
-        // the fused plane kernels: x + y forward, y + x inverse (grids with
-        // M0 = M1 whose plane fits)
-        bool any_fuse = false;
-        for (const GridDev& g : L.hg) any_fuse = any_fuse || (g.M[0] == g.M[1] && fast_xy_length(g.M[0]));
-        if (any_fuse && fft_fast_enabled()) {
-            for (int q : {(int)kPassXf, (int)kPassXi}) {
-                if (st != APM_OK) break;
+        // the fused plane kernels, x + y forward and y + x inverse, against the
+        // choice so far: for every grid they fit, then for the lengths plan 0 takes
+        // them for, where those are other kernels
+        for (int q : {(int)kPassXf, (int)kPassXi})
+            for (int p : {2, 0}) {
+                int alt[kFftPasses];
+                std::copy(L.plan, L.plan + kFftPasses, alt);
+                alt[q] = p;
+                if (st != APM_OK || same_kernels(alt)) continue;
                 const int old = L.plan[q];
-                st = try_knob([&] { L.plan[q] = 2; }, [&] { L.plan[q] = old; });
+                st = try_knob([&] { L.plan[q] = p; }, [&] { L.plan[q] = old; });
             }
+        // the default's number for the default's kernels
+        for (int q : {(int)kPassXf, (int)kPassXi}) {
+            int alt[kFftPasses];
+            std::copy(L.plan, L.plan + kFftPasses, alt);
+            alt[q] = 0;
+            if (st == APM_OK && same_kernels(alt)) L.plan[q] = 0;
         }
     }
     if (st == APM_OK && L.hg.size() > 1) {
         const int old = L.packing;
         st = try_knob([&] { L.packing = 1 - old; }, [&] { L.packing = old; });
     }
-    if (st == APM_OK && !f64) {
+    bool any_runtime = false;
+    for (int q = 0; q < kFftPasses; ++q) any_runtime = any_runtime || !all_planned(q);
+    if (st == APM_OK && !f64 && any_runtime) {
         const int old = L.max_radix, alt = old == 16 ? 8 : 16;
         st = try_knob([&] { replan_level(L, alt); }, [&] { replan_level(L, old); });
     }
@@ -1575,7 +1593,7 @@ apm_status apm_set_fft_shapes(apm_ctx* c, int32_t level, const apm_fft_shapes* s
     for (int q = 0; q < kFftPasses; ++q) {
         const int t = shapes->threads[q];
         if (shapes->budget[q] < 1 || (t != 128 && t != 256)) return APM_E_INVALID;
-        const int pmax = (q == kPassXf || q == kPassXi) ? 2 : 1;   // 2: fused with the y pass
+        const int pmax = (q == kPassXf || q == kPassXi) ? 3 : 1;   // 2: fused with the y pass, 3: never fused
         if (shapes->plan[q] < 0 || shapes->plan[q] > pmax) return APM_E_INVALID;
     }
     if ((shapes->packing != 0 && shapes->packing != 1) ||
