@@ -1017,6 +1017,7 @@ apm_status apm_set_hierarchy(apm_ctx* c, const apm_grid* grids, int32_t n) {
         D.frac_bits = kPosBits - L.level;
         D.span = (long long)N0 << kPosBits;
         D.box = cfg.box;
+        D.root_cells = (double)grids[0].dims[0] * grids[0].dims[1] * grids[0].dims[2];
         D.periodic = periodic ? 1 : 0;
         D.status = c->d_status;
         if (L.level > 0) {
@@ -1188,7 +1189,8 @@ apm_status apm_deposit_all(apm_ctx* c, const apm_particles* particles, double ha
     Particles P = to_dev(particles);
     if (c->dep_tiles) use_order(c, P);
     Trace t(c, K_DEPOSIT, s);
-    return cuda_status(launch_deposit_levels(c->d_levels, nl, P, half_dt, c->cfg.box, c->cfg.mass_frac_bits,
+    return cuda_status(launch_deposit_levels(c->d_levels, nl, c->levels[0].dev.root_cells, P, half_dt, c->cfg.box,
+                                             c->cfg.mass_frac_bits,
                                              (int64_t* const* const*)(c->d_tabs + (size_t)R_GMF * nl),
                                              c->d_status, s));
 }

@@ -355,6 +355,7 @@ struct LevelDev {
     int frac_bits;         // 31 - level: fraction bits of a position on this level
     long long span;        // N0 2^31: the box in fixed-point units
     double box;
+    double root_cells;     // cells of the root
     int periodic;
     int div_known;         // div_known() may divide by delta0 with inv_delta0
     int pos_exp;           // delta0 = 2^(31 - pos_exp) when delta0_pow2: X = rint(x 2^pos_exp)
@@ -548,6 +549,7 @@ struct Particles {
     const double *x, *y, *z, *vx, *vy, *vz, *m;
     const int* perm = nullptr;   // processing order (launch_order): slot i visits particle perm[i]
     unsigned stride = 0;         // the deposit's walk through its CTAs in that order (deposit_order)
+    bool spread = false;         // ... and its lanes' slots (thread_slot)
     __device__ __forceinline__ long long at(long long i) const { return perm ? (long long)perm[i] : i; }
 };
 
@@ -613,8 +615,8 @@ cudaError_t launch_gas_init(const LevelDev& L, const GridDev* parent_grids,
 cudaError_t launch_deposit(const LevelDev& L, const Particles& P, double half_dt, double box,
                            int F, int64_t* const* gmf, unsigned* status, cudaStream_t s);
 // every level in one pass: levels[nl] and gmfs[nl] in device memory
-cudaError_t launch_deposit_levels(const LevelDev* levels, int nl, const Particles& P, double half_dt,
-                                  double box, int F, int64_t* const* const* gmfs, unsigned* status,
+cudaError_t launch_deposit_levels(const LevelDev* levels, int nl, double root_cells, const Particles& P,
+                                  double half_dt, double box, int F, int64_t* const* const* gmfs, unsigned* status,
                                   cudaStream_t s);
 
 // FFT passes of one level (T = float or double)

@@ -510,11 +510,15 @@ __device__ __forceinline__ bool particle_of_level(const LevelDev& L, const Parti
     return ok;
 }
 
-// the first slot of this CTA: in the caller's order CTA after CTA; in bin order
-// spread over the bins (deposit_stride, coprime to the number of CTAs)
-__device__ __forceinline__ long long first_slot(const Particles& P, unsigned b) {
+// this thread's slot: in the caller's order CTA after CTA; in bin order spread over
+// the bins (deposit_stride, coprime to the number of CTAs).  spread: the warp's 32
+// slots transposed, lane 8 j + p taking slot 4 p + j, so that the 8 clouds an
+// instruction sends are every fourth one
+__device__ __forceinline__ long long thread_slot(const Particles& P, unsigned b) {
     if (P.stride) b = (unsigned)((unsigned long long)b * P.stride % gridDim.x);
-    return (long long)b * kDepThreads;
+    unsigned t = threadIdx.x;
+    if (P.spread) t = (t & ~31u) | (t & 7u) << 2 | (t >> 3 & 3u);
+    return (long long)b * kDepThreads + t;
 }
 
 // One level.  ORDERED: in bin order.
@@ -526,7 +530,7 @@ __global__ void __launch_bounds__(kDepThreads, APM_DEP_MIN_CTAS) k_deposit(Level
     const unsigned block = begin_kernel();
     __shared__ WarpCharges charges[kDepThreads / 32];
     __shared__ BoxShared cta[1];
-    const long long i = first_slot(P, block) + threadIdx.x;
+    const long long i = thread_slot(P, block);
     long long X[3] = {0, 0, 0}, M = 0;
     bool outside = false;
     const bool ok = i < P.n && particle_of_level(L, P, i, half_dt, box, F, X, &M, &outside, status);
@@ -544,7 +548,7 @@ __global__ void __launch_bounds__(kDepThreads, APM_DEP_MIN_CTAS) k_deposit_level
     const unsigned block = begin_kernel();
     __shared__ WarpCharges charges[kDepThreads / 32];
     __shared__ BoxShared cta[1];
-    const long long i = first_slot(P, block) + threadIdx.x;
+    const long long i = thread_slot(P, block);
     long long X[3] = {0, 0, 0}, M = 0;
     bool outside = false, ok = false;
     if (i < P.n) ok = particle_fixed(levels[0], P, P.at(i), half_dt, box, F, X, &M, &outside, status);
@@ -573,8 +577,16 @@ cudaError_t launch_gas_init(const LevelDev& L, const GridDev* parent_grids,
 // through the CTAs spreads them over the bins, and each CTA keeps its own bin's
 // locality.  A Plummer sphere of 1 M through three nested levels 413 -> 344 us
 // (caller's order 551); random places on 256^3 166 -> 182 (246).
-static Particles deposit_order(Particles P, unsigned blocks) {
+// In the caller's order, where there are two particles or more to a root cell,
+// neighbouring ones stored in spatial order share cells, and an instruction's
+// reductions into one cell wait for one another: it sends every fourth particle
+// instead.  A lattice of 8 to a cell on 128^3 1252 -> 1019 us, of 64 to a cell on
+// 64^3 2248 -> 1437, of 4 to a cell on 128^3 608 -> 545; of one to a cell on 256^3
+// 1031 either way, and below that the neighbours' shared sectors are worth more (one
+// to 8 cells there 168 -> 194).  In no spatial order it makes no difference.
+static Particles deposit_order(Particles P, unsigned blocks, double cells) {
     P.stride = 0;
+    P.spread = !P.perm && (double)P.n >= 2.0 * cells;
     if (P.perm && blocks > 2) {
         auto gcd = [](unsigned a, unsigned b) {
             while (b) {
@@ -595,16 +607,16 @@ cudaError_t launch_deposit(const LevelDev& L, const Particles& P, double half_dt
     if (P.n <= 0) return cudaSuccess;
     unsigned blocks = (unsigned)((P.n + kDepThreads - 1) / kDepThreads);
     return launch_kernel(P.perm ? k_deposit<true> : k_deposit<false>, blocks, kDepThreads, 0, s, L,
-                         deposit_order(P, blocks), half_dt, box, F, gmf, status);
+                         deposit_order(P, blocks, L.root_cells), half_dt, box, F, gmf, status);
 }
 
-cudaError_t launch_deposit_levels(const LevelDev* levels, int nl, const Particles& P, double half_dt,
-                                  double box, int F, int64_t* const* const* gmfs, unsigned* status,
+cudaError_t launch_deposit_levels(const LevelDev* levels, int nl, double root_cells, const Particles& P,
+                                  double half_dt, double box, int F, int64_t* const* const* gmfs, unsigned* status,
                                   cudaStream_t s) {
     if (P.n <= 0 || nl <= 0) return cudaSuccess;
     unsigned blocks = (unsigned)((P.n + kDepThreads - 1) / kDepThreads);
     return launch_kernel(P.perm ? k_deposit_levels<true> : k_deposit_levels<false>, blocks, kDepThreads, 0, s, levels,
-                         nl, deposit_order(P, blocks), half_dt, box, F, gmfs, status);
+                         nl, deposit_order(P, blocks, root_cells), half_dt, box, F, gmfs, status);
 }
 
 }  // namespace apm
