@@ -133,8 +133,10 @@ static_assert(kDepThreads % 32 == 0, "the deposit works by whole warps");
 // 1 M through three nested levels 0.75 -> 0.40.
 constexpr int kChargePitch = 40;
 struct WarpCharges {
-    unsigned lo[9][kChargePitch];      // charge of cell a + 3 b of the layer, of each lane's particle
-    unsigned hi[9][kChargePitch];      // ... high words of wide charges
+    union {                            // charge of cell a + 3 b of the layer, of each lane's particle
+        unsigned narrow[9][kChargePitch];
+        unsigned long long wide[9][kChargePitch];
+    };
     unsigned off[9][kChargePitch];     // cx[3], G0 cy[3], G0 G1 cz[3]; kNoCell: outside
     int64_t* base[32];                 // the mass field of each lane's grid
 };
@@ -220,8 +222,7 @@ __device__ __forceinline__ void send_layer(const WarpCharges& s, int lane, unsig
 #pragma unroll
         for (int b = 0; b < 3; ++b) {
             const unsigned o = s.off[3 + b][k];
-            unsigned long long q = s.lo[a + 3 * b][k];
-            if (WIDE) q |= (unsigned long long)s.hi[a + 3 * b][k] << 32;
+            const unsigned long long q = WIDE ? s.wide[a + 3 * b][k] : s.narrow[a + 3 * b][k];
             // a particle on a cell face has charges of zero (19 of 27 on a corner): not
             // sent (16.8 M corner particles on 256^3: 1.01 -> 0.92 ms)
             if ((out | o) < kNoCell && q != 0)
@@ -248,8 +249,8 @@ __device__ __forceinline__ void send_clouds(WarpCharges& s, int lane, bool act, 
         const int c = k == 0 ? 0 : 3 - k;   // 0, 2, 1
         if (act)
             q.layer(c, w, [&](int j, V v) {
-                s.lo[j][lane] = (unsigned)v;
-                if constexpr (kWide) s.hi[j][lane] = (unsigned)(v >> 32);
+                if constexpr (kWide) s.wide[j][lane] = v;
+                else s.narrow[j][lane] = v;
             });
         __syncwarp();
         send_layer<kWide>(s, lane, live, c);
