@@ -25,14 +25,20 @@ constexpr int kMode = APM_FAST_MODE;
 constexpr bool kFused = kMode == kFastXy || kMode == kFastYx;
 constexpr int kLines = fast_lines(kF64);
 
+// The plan of radices A, B, Cc.  FP64 takes 75 in three stages: 15 x 5 has 40 first
+// butterflies in a CTA, one warp and a quarter, and the pipe that bounds it takes as
+// long for the quarter as for a warp (8 grids of L = 75: 627 -> 514 us).
+template <int A, int B, int Cc>
+using PlanOf = typename std::conditional<kF64 && A * B * Cc == 75, FastPlan<3, 5, 5>, FastPlan<A, B, Cc>>::type;
+
 template <int A, int B, int Cc>
 struct Kern {
-    using P = FastPlan<A, B, Cc>;
+    using P = PlanOf<A, B, Cc>;
     static constexpr int L = A * B * Cc;
     static constexpr bool row = kMode == kFastXf || kMode == kFastXi;
     // a fused plane kernel exists where the plane fits the shared-memory limit
     static constexpr bool ok = !kFused || fast_xy_smem(L) <= (size_t)kFftSmemLimit;
-    static constexpr int NT = kFused ? fast_xy_threads(kMode, L) : fast_threads(A, B, Cc, kLines);
+    static constexpr int NT = kFused ? fast_xy_threads(kMode, L) : fast_threads(P::R1, P::R2, P::R3, kLines);
     static constexpr size_t smem = kFused ? fast_xy_smem(L) : (row ? fast_row_smem(L, kF64) : fast_col_smem(L, kF64));
     static constexpr auto get() {
         if constexpr (kMode == kFastYf) return k_col_fast<P, 1, 0, kLines, NT, FT>;
