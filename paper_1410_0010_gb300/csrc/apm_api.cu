@@ -1045,25 +1045,6 @@ apm_status apm_set_hierarchy(apm_ctx* c, const apm_grid* grids, int32_t n) {
             std::vector<int> doff, dlist, ooff, olist;
             build_csr(dep, lo, shift, nt, doff, dlist);
             build_csr(own, lo, shift, nt, ooff, olist);
-            // dilated occupancy: a particle whose FP32-estimated tile has no
-            // occupied neighbour cannot touch any GMF box of the level
-            std::vector<unsigned char> occ((size_t)nt[0] * nt[1] * nt[2], 0);
-            for (int z = 0; z < nt[2]; ++z)
-                for (int y = 0; y < nt[1]; ++y)
-                    for (int x = 0; x < nt[0]; ++x) {
-                        long long t = x + (long long)nt[0] * (y + (long long)nt[1] * z);
-                        if (doff[t + 1] == doff[t]) continue;
-                        for (int dz = -1; dz <= 1; ++dz)
-                            for (int dy = -1; dy <= 1; ++dy)
-                                for (int dx = -1; dx <= 1; ++dx) {
-                                    int X = x + dx, Y = y + dy, Z = z + dz;
-                                    if (X < 0 || Y < 0 || Z < 0 || X >= nt[0] || Y >= nt[1] || Z >= nt[2]) continue;
-                                    occ[X + (size_t)nt[0] * (Y + (size_t)nt[1] * Z)] = 1;
-                                }
-                    }
-            unsigned char* d_occ;
-            if ((st = upload(c, &d_occ, occ)) != APM_OK) return st;
-            D.map.occ = d_occ;
             int *d_doff, *d_dlist, *d_ooff, *d_olist;
             if ((st = upload(c, &d_doff, doff)) != APM_OK) return st;
             if ((st = upload(c, &d_dlist, dlist)) != APM_OK) return st;

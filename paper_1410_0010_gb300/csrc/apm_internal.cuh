@@ -334,7 +334,6 @@ struct TileMap {
     const int* dep_list;
     const int* own_off;   // grids whose interior meets the tile
     const int* own_list;
-    const unsigned char* occ;  // 1 if the tile or one of its 26 neighbours has a dep entry
 };
 
 struct Chunk { int grid; int tile; };   // one CTA of a batched pass
@@ -529,16 +528,9 @@ __device__ __forceinline__ bool mbar_wait_bounded(unsigned long long* bar, unsig
 }
 constexpr unsigned kWaitPolls = 1u << 20;
 
-// wmul63 for a < 2^32: with b = bh 2^32 + bl, (a b + 2^62) >> 63 equals
-// (a bh + ((a bl) >> 32) + 2^30) >> 31 (the low 32 bits of a bl cannot carry
-// into the result); two 32 x 32 -> 64 products
-__device__ __forceinline__ unsigned long long wmul63_small(unsigned long long a, unsigned long long b) {
-    const unsigned a32 = (unsigned)a;
-    const unsigned long long hi = (unsigned long long)a32 * (unsigned)(b >> 32);
-    const unsigned long long lo = (unsigned long long)a32 * (unsigned)b;
-    return (hi + (lo >> 32) + (1ULL << 30)) >> 31;
-}
-// ... and its 32-bit result: a weight is at most 1, so the product is below 2^32
+// wmul63 for a < 2^32 and a 32-bit result (a weight is at most 1): with
+// b = bh 2^32 + bl, (a b + 2^62) >> 63 equals (a bh + ((a bl) >> 32) + 2^30) >> 31
+// (the low 32 bits of a bl cannot carry into the result)
 __device__ __forceinline__ unsigned wmul63_32(unsigned a, unsigned long long b) {
     const unsigned long long hi = (unsigned long long)a * (unsigned)(b >> 32) + (1ULL << 30);
     return (unsigned)((hi + __umulhi(a, (unsigned)b)) >> 31);
