@@ -552,10 +552,10 @@ struct Particles {
 // before it on its stream, so the launch itself overlaps that one's end; each
 // begins with begin_kernel(), which waits until everything before it is complete
 // and visible (nothing is read or written early, whatever comes before: a kernel
-// of the caller's, a copy, another stream joined by an event).  The 9 launches of
-// an isolated 96^3 root's solve 59.7 -> 52.7 us, a 1 M Plummer step of three
-// nested levels 826 -> 765, 32 grids of 128^3 886 -> 871, a two-level 64^3 step
-// replayed as a graph 97.6 -> 95.9.  Letting the next kernel's CTAs in early
+// of the caller's, a copy, another stream joined by an event).  The 3 launches of
+// an isolated 96^3 root's solve 51.3 -> 44.9 us, a 1 M Plummer step of three
+// nested levels 808 -> 746, 32 grids of 128^3 742 -> 734, a two-level 64^3 step
+// replayed as a graph 94.0 -> 91.4.  Letting the next kernel's CTAs in early
 // (griddepcontrol.launch_dependents) costs more than it gives: the cosmological
 // step 10.2 -> 11.6 ms, that graph 99.5 -> 123 us.
 // The block index comes out of the same instruction sequence, so that every
