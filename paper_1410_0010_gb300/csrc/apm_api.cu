@@ -1044,6 +1044,8 @@ apm_status apm_set_hierarchy(apm_ctx* c, const apm_grid* grids, int32_t n) {
             for (int j = 0; j < 3; ++j) nt[j] = (int)(((hi[j] - lo[j]) + (1LL << shift) - 1) >> shift);
             std::vector<int> doff, dlist, ooff, olist;
             build_csr(dep, lo, shift, nt, doff, dlist);
+            for (size_t t = 0; t + 1 < doff.size(); ++t)
+                if (doff[t + 1] - doff[t] > 1) D.overlap = 1;
             build_csr(own, lo, shift, nt, ooff, olist);
             int *d_doff, *d_dlist, *d_ooff, *d_olist;
             if ((st = upload(c, &d_doff, doff)) != APM_OK) return st;
@@ -1170,8 +1172,10 @@ apm_status apm_deposit_all(apm_ctx* c, const apm_particles* particles, double ha
     Particles P = to_dev(particles);
     if (c->dep_tiles) use_order(c, P);
     Trace t(c, K_DEPOSIT, s);
-    return cuda_status(launch_deposit_levels(c->d_levels, nl, c->levels[0].dev.root_cells, P, half_dt, c->cfg.box,
-                                             c->cfg.mass_frac_bits,
+    bool overlap = false;
+    for (const Level& L : c->levels) overlap = overlap || L.dev.overlap != 0;
+    return cuda_status(launch_deposit_levels(c->d_levels, nl, c->levels[0].dev.root_cells, overlap, P, half_dt,
+                                             c->cfg.box, c->cfg.mass_frac_bits,
                                              (int64_t* const* const*)(c->d_tabs + (size_t)R_GMF * nl),
                                              c->d_status, s));
 }

@@ -356,6 +356,7 @@ struct LevelDev {
     double box;
     double root_cells;     // cells of the root
     int periodic;
+    int overlap;           // a tile lists more than one deposit candidate
     int div_known;         // div_known() may divide by delta0 with inv_delta0
     int pos_exp;           // delta0 = 2^(31 - pos_exp) when delta0_pow2: X = rint(x 2^pos_exp)
     unsigned* status;      // the context's device status word (bounds-checked builds)
@@ -607,7 +608,7 @@ cudaError_t launch_gas_init(const LevelDev& L, const GridDev* parent_grids,
 cudaError_t launch_deposit(const LevelDev& L, const Particles& P, double half_dt, double box,
                            int F, int64_t* const* gmf, unsigned* status, cudaStream_t s);
 // every level in one pass: levels[nl] and gmfs[nl] in device memory
-cudaError_t launch_deposit_levels(const LevelDev* levels, int nl, double root_cells, const Particles& P,
+cudaError_t launch_deposit_levels(const LevelDev* levels, int nl, double root_cells, bool overlap, const Particles& P,
                                   double half_dt, double box, int F, int64_t* const* const* gmfs, unsigned* status,
                                   cudaStream_t s);
 

@@ -129,8 +129,8 @@ static_assert(kDepThreads % 32 == 0, "the deposit works by whole warps");
 // particles (stores) and on 3 x 8 (loads) fall into distinct banks.
 // All levels, before (one particle per thread, x neighbours' columns merged in
 // registers) -> now: 16.8 M lattice particles on 512^3 with two refined levels
-// 1.82 -> 1.46 ms; 4.2 M random ones on 256^3 1.23 -> 0.93; a Plummer sphere of
-// 1 M through three nested levels 0.75 -> 0.40.
+// 1.82 -> 1.43 ms; 4.2 M random ones on 256^3 1.23 -> 0.78; a Plummer sphere of
+// 1 M through three nested levels 0.96 -> 0.54.
 constexpr int kChargePitch = 40;
 struct WarpCharges {
     union {                            // charge of cell a + 3 b of the layer, of each lane's particle
@@ -262,6 +262,71 @@ __device__ __noinline__ void send_wide_clouds(WarpCharges& s, int lane, bool act
                                               long long z, int P) {
     send_clouds<unsigned long long>(s, lane, act, M, x, y, z, P);
 }
+
+// This lane's cloud straight into the candidate grids [e0, e1) (list null: the
+// root), one reduction per cell; UNROLL of the three layers
+template <typename V, int UNROLL>
+__device__ __forceinline__ void send_direct(const GridDev* __restrict__ grids, const int* __restrict__ list, int e0, int e1,
+                                         long long M, long long x, long long y, long long z, int P,
+                                         int64_t* const* __restrict__ gmf, unsigned* __restrict__ status) {
+    const long long ic[3] = {x >> P, y >> P, z >> P};
+    unsigned long long w[3][3];
+    tsc_fixed(x, P, w[0]);
+    tsc_fixed(y, P, w[1]);
+    tsc_fixed(z, P, w[2]);
+    for (int e = e0; e < e1; ++e) {
+        const int gi = list ? list[e] : 0;
+        const GridDev& g = grids[gi];
+        const unsigned st[3] = {1u, (unsigned)g.G[0], (unsigned)g.G[0] * (unsigned)g.G[1]};
+        unsigned off[3][3];
+        bool touches = true;
+#pragma unroll
+        for (int j = 0; j < 3; ++j) {
+            const int G = g.G[j], r = local_centre(g, ic, j);
+            touches = touches && (g.mode != 0 || (r >= -1 && r <= G));
+#pragma unroll
+            for (int k = 0; k < 3; ++k) {
+                const int v = edge_rule(r + k - 1, G, g.mode);
+                off[j][k] = v >= 0 && APM_IN_BOUNDS(v, G, status) ? st[j] * (unsigned)v : kNoCell;
+            }
+        }
+        if (!touches) continue;   // listed by its tile only
+        int64_t* __restrict__ const out = gmf[gi];
+        LaneCharges<V> q;
+        q.start(M, w);
+#pragma unroll UNROLL
+        for (int k = 0; k < 3; ++k) {
+            const int c = k == 0 ? 0 : 3 - k;   // 0, 2, 1
+            const unsigned oz = c == 0 ? off[2][0] : (c == 1 ? off[2][1] : off[2][2]);
+            q.layer(c, w, [&](int j, V v) {
+                const unsigned ox = off[0][j % 3], oy = off[1][j / 3];
+                if ((ox | oy | oz) < kNoCell && v != 0)
+                    asm volatile("red.global.add.u64 [%0], %1;" ::"l"(out + (ox + oy + oz)), "l"((unsigned long long)v));
+            });
+        }
+    }
+}
+
+__device__ __forceinline__ bool candidates(const LevelDev& L, const long long ic[3], int& e0, int& e1);
+// the cloud of a lane with more candidates on level L into those after the first
+__device__ __forceinline__ void deposit_rest(const LevelDev& L, const long long X[3], long long M,
+                                             int64_t* const* __restrict__ gmf, unsigned* __restrict__ status) {
+    const int P = L.frac_bits;
+    const long long ic[3] = {X[0] >> P, X[1] >> P, X[2] >> P};
+    int e0, e1;
+    candidates(L, ic, e0, e1);
+    // (64-bit charges for every mass: the narrow ones round the same way)
+    send_direct<unsigned long long, 1>(L.g, L.map.dep_list, e0 + 1, e1, M, X[0], X[1], X[2], P, gmf, status);
+}
+
+// How a launch sends its clouds: in rows; in rows, and straight into the candidate
+// grids after the first, on levels with overlapping borders (rows for them would be
+// mostly empty: 200000 random particles over 8 touching grids 72 -> 70 us, with
+// 64-bit charges 92 -> 86); in bin order, like that where no box gathers them; all
+// straight, which is the shorter way where a launch leaves most schedulers a warp or
+// none.  A loop over the candidates in the rows' kernel spills registers there (1 M
+// random particles on 256^3 246 us with it, 227 without; a lattice on 192^3 103, 98).
+enum DepositWay { kRows, kRowsOverlap, kOrdered, kDirect };
 
 // the candidate grids [e0, e1) of level L's tile lists for the centre cell ic
 // (the root: [0, 1)); false when there is none
@@ -418,14 +483,15 @@ __device__ __forceinline__ void box_deposit(unsigned* __restrict__ words, const 
 
 // The deposit into the grids of one level: this lane's particle at fixed-point
 // position X with integer mass M (ok false: none).  Every lane of the warp calls
-// it, ORDERED every thread of the CTA.  False when this lane's particle is not a candidate of
+// it, kOrdered every thread of the CTA.  False when this lane's particle is not a candidate of
 // the level (then it is none of a finer level's either: finer GMF boxes lie
 // inside the interiors of their parents).
-template <bool ORDERED>
-__device__ __forceinline__ bool deposit_level_warp(WarpCharges* charges, BoxShared* box, const LevelDev& L, const long long X[3],
-                                                   long long M, bool ok, bool outside,
+template <DepositWay WAY>
+__device__ __forceinline__ bool deposit_level_warp(WarpCharges* charges, BoxShared* box, const LevelDev& L,
+                                                   const long long X[3], long long M, bool ok, bool outside, bool& more,
                                                    int64_t* const* __restrict__ gmf,
                                                    unsigned* __restrict__ status) {
+    more = false;
     constexpr unsigned kFull = 0xffffffffu;
     const int lane = threadIdx.x & 31;
     const int PB = L.frac_bits;
@@ -434,7 +500,7 @@ __device__ __forceinline__ bool deposit_level_warp(WarpCharges* charges, BoxShar
     for (int j = 0; j < 3; ++j) ic[j] = X[j] >> PB;
     int e0 = 0, e1 = 0;
     ok = ok && candidates(L, ic, e0, e1);
-    if constexpr (ORDERED) {
+    if constexpr (WAY == kOrdered) {
         if (!__syncthreads_or(ok)) return false;
         const int gi = !ok ? 0 : (L.is_root ? 0 : L.map.dep_list[e0]);
         const GridDev& g = L.g[gi];
@@ -446,25 +512,30 @@ __device__ __forceinline__ bool deposit_level_warp(WarpCharges* charges, BoxShar
             return ok;
         }
     }
-    WarpCharges& s = charges[threadIdx.x >> 5];
     if (!__any_sync(kFull, ok)) return false;
     // one charge width for the whole warp (the 32-bit products round the same way)
     const bool wide = __any_sync(kFull, ok && M != 0 && !narrow_mass(M));
     if (!ok) e1 = e0;
-    // the candidate grids in turn (one on the root and almost everywhere else)
-    for (; __any_sync(kFull, e0 < e1); ++e0) {
-        const bool act = e0 < e1;
-        if (act) {
-            const int gi = L.is_root ? 0 : L.map.dep_list[e0];
-            const GridDev& g = L.g[gi];
-            if (g.mode == 1 && outside) atomicOr(status, kStOutOfBox);
-            lane_cells(s, lane, g, ic, status);
-            s.base[lane] = gmf[gi];
+    if (ok && outside) atomicOr(status, kStOutOfBox);
+    const int* const list = L.is_root ? nullptr : L.map.dep_list;
+    if constexpr (WAY == kDirect) {
+        if (e0 < e1 && M != 0) {
+            if (wide) send_direct<unsigned long long, 3>(L.g, list, e0, e1, M, X[0], X[1], X[2], PB, gmf, status);
+            else send_direct<unsigned, 3>(L.g, list, e0, e1, M, X[0], X[1], X[2], PB, gmf, status);
         }
-        // a particle without mass sends nothing
-        if (wide) send_wide_clouds(s, lane, act && M != 0, M, X[0], X[1], X[2], PB);
-        else send_clouds<unsigned>(s, lane, act && M != 0, M, X[0], X[1], X[2], PB);
+        return ok;
     }
+    WarpCharges& s = charges[threadIdx.x >> 5];
+    const bool act = e0 < e1;
+    if (act) {
+        const int gi = list ? list[e0] : 0;
+        lane_cells(s, lane, L.g[gi], ic, status);
+        s.base[lane] = gmf[gi];
+    }
+    // a particle without mass sends nothing
+    if (wide) send_wide_clouds(s, lane, act && M != 0, M, X[0], X[1], X[2], PB);
+    else send_clouds<unsigned>(s, lane, act && M != 0, M, X[0], X[1], X[2], PB);
+    more = e0 + 1 < e1 && M != 0;
     return ok;
 }
 
@@ -522,9 +593,10 @@ __device__ __forceinline__ long long thread_slot(const Particles& P, unsigned b)
     return (long long)b * kDepThreads + t;
 }
 
-// One level.  ORDERED: in bin order.
-template <bool ORDERED>
-__global__ void __launch_bounds__(kDepThreads, APM_DEP_MIN_CTAS) k_deposit(LevelDev L, Particles P, double half_dt,
+constexpr int dep_min_ctas(DepositWay way) { return way == kDirect ? 4 : APM_DEP_MIN_CTAS; }
+// One level.
+template <DepositWay WAY>
+__global__ void __launch_bounds__(kDepThreads, dep_min_ctas(WAY)) k_deposit(LevelDev L, Particles P, double half_dt,
                                                  double box, int F,
                                                  int64_t* const* __restrict__ gmf,
                                                  unsigned* __restrict__ status) {
@@ -535,15 +607,17 @@ __global__ void __launch_bounds__(kDepThreads, APM_DEP_MIN_CTAS) k_deposit(Level
     long long X[3] = {0, 0, 0}, M = 0;
     bool outside = false;
     const bool ok = i < P.n && particle_of_level(L, P, i, half_dt, box, F, X, &M, &outside, status);
-    deposit_level_warp<ORDERED>(charges, cta, L, X, M, ok, outside, gmf, status);
+    bool more;
+    deposit_level_warp<WAY>(charges, cta, L, X, M, ok, outside, more, gmf, status);
+    if ((WAY == kRowsOverlap || WAY == kOrdered) && more) deposit_rest(L, X, M, gmf, status);
 }
 
 // Every level in one pass over the particles: the position and mass are
 // converted once, then deposited level by level from the root down while the
 // particle is a candidate.  levels: the LevelDev of each level; gmfs[l]: the
 // GMF pointer table of level l.
-template <bool ORDERED>
-__global__ void __launch_bounds__(kDepThreads, APM_DEP_MIN_CTAS) k_deposit_levels(
+template <DepositWay WAY>
+__global__ void __launch_bounds__(kDepThreads, dep_min_ctas(WAY)) k_deposit_levels(
     const LevelDev* __restrict__ levels, int nl, Particles P, double half_dt, double box, int F,
     int64_t* const* const* __restrict__ gmfs, unsigned* __restrict__ status) {
     const unsigned block = begin_kernel();
@@ -553,12 +627,22 @@ __global__ void __launch_bounds__(kDepThreads, APM_DEP_MIN_CTAS) k_deposit_level
     long long X[3] = {0, 0, 0}, M = 0;
     bool outside = false, ok = false;
     if (i < P.n) ok = particle_fixed(levels[0], P, P.at(i), half_dt, box, F, X, &M, &outside, status);
+    unsigned rest = 0;   // levels (at most 21) with more candidates for this lane
     for (int l = 0; l < nl; ++l) {
-        ok = deposit_level_warp<ORDERED>(charges, cta, levels[l], X, M, ok, l == 0 && outside, gmfs[l], status);
-        if constexpr (ORDERED) {   // the CTA's box needs all its warps
+        bool more;
+        ok = deposit_level_warp<WAY>(charges, cta, levels[l], X, M, ok, l == 0 && outside, more, gmfs[l], status);
+        if (more) rest |= 1u << l;
+        if constexpr (WAY == kOrdered) {   // the CTA's box needs all its warps
             if (!__syncthreads_or(ok)) break;
         } else {
             if (!__any_sync(0xffffffffu, ok)) break;
+        }
+    }
+    // after the levels, so that no call stands in their loop
+    if constexpr (WAY == kRowsOverlap || WAY == kOrdered) {
+        for (; rest; rest &= rest - 1) {
+            const int l = __ffs(rest) - 1;
+            deposit_rest(levels[l], X, M, gmfs[l], status);
         }
     }
 }
@@ -582,9 +666,10 @@ cudaError_t launch_gas_init(const LevelDev& L, const GridDev* parent_grids,
 // neighbouring ones stored in spatial order share cells, and an instruction's
 // reductions into one cell wait for one another: it sends every fourth particle
 // instead.  A lattice of 8 to a cell on 128^3 1252 -> 1019 us, of 64 to a cell on
-// 64^3 2248 -> 1437, of 4 to a cell on 128^3 608 -> 545; of one to a cell on 256^3
-// 1031 either way, and below that the neighbours' shared sectors are worth more (one
-// to 8 cells there 168 -> 194).  In no spatial order it makes no difference.
+// 64^3 2248 -> 1437, of 4 to a cell on 128^3 608 -> 545 (947, 1366 and 504 now); of
+// one to a cell on 256^3 1031 either way, and below that the neighbours' shared
+// sectors are worth more (one to 8 cells there 168 -> 194).  In no spatial order it
+// makes no difference.
 static Particles deposit_order(Particles P, unsigned blocks, double cells) {
     P.stride = 0;
     P.spread = !P.perm && (double)P.n >= 2.0 * cells;
@@ -603,21 +688,36 @@ static Particles deposit_order(Particles P, unsigned blocks, double cells) {
     return P;
 }
 
+// Straight up to 16384 particles (64-bit charges on an isolated 32^3 root 12.4 us in
+// rows, 10.4 so; 20000 on a 60^3 root 12.4 in rows and 14.0 so), four times as many
+// where levels overlap (8586 over 8 touching grids 33 us in rows and 23 so, 60000 39
+// and 37, with 64-bit charges 41 and 25, 46 and 39).
+constexpr long long kDirectParticles = 16384;
+static DepositWay deposit_way(const Particles& P, bool overlap) {
+    if (P.perm) return kOrdered;
+    if (P.n <= (overlap ? 4 * kDirectParticles : kDirectParticles)) return kDirect;
+    return overlap ? kRowsOverlap : kRows;
+}
+
 cudaError_t launch_deposit(const LevelDev& L, const Particles& P, double half_dt, double box,
                            int F, int64_t* const* gmf, unsigned* status, cudaStream_t s) {
     if (P.n <= 0) return cudaSuccess;
     unsigned blocks = (unsigned)((P.n + kDepThreads - 1) / kDepThreads);
-    return launch_kernel(P.perm ? k_deposit<true> : k_deposit<false>, blocks, kDepThreads, 0, s, L,
+    void (*const kernels[])(LevelDev, Particles, double, double, int, int64_t* const*, unsigned*) = {
+        k_deposit<kRows>, k_deposit<kRowsOverlap>, k_deposit<kOrdered>, k_deposit<kDirect>};
+    return launch_kernel(kernels[deposit_way(P, L.overlap != 0)], blocks, kDepThreads, 0, s, L,
                          deposit_order(P, blocks, L.root_cells), half_dt, box, F, gmf, status);
 }
 
-cudaError_t launch_deposit_levels(const LevelDev* levels, int nl, double root_cells, const Particles& P,
+cudaError_t launch_deposit_levels(const LevelDev* levels, int nl, double root_cells, bool overlap, const Particles& P,
                                   double half_dt, double box, int F, int64_t* const* const* gmfs, unsigned* status,
                                   cudaStream_t s) {
     if (P.n <= 0 || nl <= 0) return cudaSuccess;
     unsigned blocks = (unsigned)((P.n + kDepThreads - 1) / kDepThreads);
-    return launch_kernel(P.perm ? k_deposit_levels<true> : k_deposit_levels<false>, blocks, kDepThreads, 0, s, levels,
-                         nl, deposit_order(P, blocks, root_cells), half_dt, box, F, gmfs, status);
+    void (*const kernels[])(const LevelDev*, int, Particles, double, double, int, int64_t* const* const*, unsigned*) = {
+        k_deposit_levels<kRows>, k_deposit_levels<kRowsOverlap>, k_deposit_levels<kOrdered>, k_deposit_levels<kDirect>};
+    return launch_kernel(kernels[deposit_way(P, overlap)], blocks, kDepThreads, 0, s, levels, nl,
+                         deposit_order(P, blocks, root_cells), half_dt, box, F, gmfs, status);
 }
 
 }  // namespace apm

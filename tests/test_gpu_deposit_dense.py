@@ -1,9 +1,10 @@
-"""Two particles or more to a root cell: the deposit's lanes take every fourth
-particle of the warp's 32 (any order gives the same field).  Bit-exact against the
-oracle for particles stored in x order, 2 to 40 to a cell and just below two, of 32-
-and 64-bit charges, some of zero mass, with a ragged last warp, on the root, a
-refined level and in the overlapping borders of two grids, in the caller's order and
-the bins'."""
+"""The deposit's arrangements by the number of particles: straight up to 16384 (65536
+where grids' borders overlap), in rows above, the candidate grids after the first
+straight, and with two or more particles to a root cell every fourth one of a warp's
+32 to an instruction (any order gives the same field).  Bit-exact against the oracle on
+both sides of each line, for particles stored in x order, of 32- and 64-bit charges,
+some of zero mass, with a ragged last warp, on the root, a refined level and in the
+overlapping borders of two and of four grids, in the caller's order and the bins'."""
 import numpy as np
 import pytest
 
@@ -12,21 +13,23 @@ from apm_inputs import GridDesc
 
 pytestmark = pytest.mark.gpu
 
-GRIDS = [GridDesc(0, -1, (0, 0, 0), (12, 12, 12)), GridDesc(1, 0, (6, 6, 8), (6, 12, 8)),
-         GridDesc(1, 0, (12, 6, 6), (6, 10, 12))]
+OVERLAP = [GridDesc(0, -1, (0, 0, 0), (24, 24, 24)), GridDesc(1, 0, (12, 12, 12), (12, 12, 12)),
+           GridDesc(1, 0, (24, 12, 12), (8, 12, 13)), GridDesc(1, 0, (12, 24, 12), (12, 9, 12)),
+           GridDesc(1, 0, (24, 24, 14), (9, 10, 8))]
+ONE = OVERLAP[:2]
 
 
 @pytest.mark.parametrize("periodic", [False, True])
 @pytest.mark.parametrize("masses", ["narrow", "wide", "mixed"])
-@pytest.mark.parametrize("per_cell", [2, 8, 40])
-def test_dense_particles_bit_exact(per_cell, masses, periodic):
+@pytest.mark.parametrize("GRIDS,n", [(g, n) for g in (ONE, OVERLAP) for n in
+                                     (1, 33, 16384, 16385, 27647, 27648)] + [(OVERLAP, 65536), (OVERLAP, 65537)])
+def test_arrangements_bit_exact(GRIDS, n, masses, periodic):   # 2 * 24^3 = 27648
     import torch
 
     from paper_1410_0010_gb300.solver import Particles, Solver
-    rng = np.random.default_rng(per_cell)
-    n = {2: 3455, 8: 3456, 40: 4001}[per_cell]      # 2 * 12^3 = 3456
-    x = (np.arange(n) + rng.random(n)) / (12 * per_cell) % 1.0      # rows along x, wrapped
-    row = (np.arange(n) / (12 * per_cell)).astype(int)
+    rng = np.random.default_rng(n)
+    x = (np.arange(n) + rng.random(n)) / 96 % 1.0       # rows along x, four to a cell
+    row = np.arange(n) // 96
     pos = np.array([x, (row * 0.618 + 0.3) % 1.0, (row * 0.381 + 0.25) % 1.0])
     m = (1 + rng.random(n)) * 2.0 ** (-24 if masses == "narrow" else -6)
     if masses == "mixed":

@@ -58,10 +58,11 @@ def _points(n, rng):
 @pytest.mark.parametrize("periodic", [False, True])
 @pytest.mark.parametrize("company", ["light", "heavy"])
 @pytest.mark.parametrize("frac", [52, 8])
-def test_small_masses_bit_exact(frac, company, periodic):
+@pytest.mark.parametrize("times", [32, 256])   # 2304 and 18432 particles: straight and in rows
+def test_small_masses_bit_exact(times, frac, company, periodic):
     rng = np.random.default_rng(frac + periodic)
     edges = [255, 256, 511, 512, 513, 2 ** 32 - 1, 2 ** 32, 2 ** 32 + 1]
-    units = np.repeat(np.concatenate([np.arange(1, 65), edges]), 32)
+    units = np.repeat(np.concatenate([np.arange(1, 65), edges]), times)
     pos = _points(len(units), rng)
     order = np.arange(len(units))               # whole warps of one mass
     if company == "heavy":                      # each warp a mixture, with wide and negative masses

@@ -31,9 +31,10 @@ def _kernels(src):
 
 
 BODIES = {name: body for src in _sources().values() for name, body in _kernels(src)}
-LAUNCHED = sorted(set(re.findall(r"\bk_\w+", " ".join(
-    m for src in _sources().values()
-    for m in re.findall(r"(?:launch_kernel\(|return )(k_\w+)[<,]", src)))))
+# launched by name, returned by a chooser, or listed by a way of their own (k_deposit<kRows>)
+LAUNCHED = sorted({m for src in _sources().values() for pattern in (r"(?:launch_kernel\(|return )(k_\w+)[<,]",
+                                                                    r"\b(k_\w+)<k[A-Z]\w*>")
+                   for m in re.findall(pattern, src)})
 
 
 def test_the_launched_kernels_are_found():
