@@ -316,8 +316,8 @@ apm_status apm_order_particles(apm_ctx* ctx, const apm_particles* particles, dou
  * the bins; a CTA whose particles share cells adds their charges in shared memory
  * and sends one reduction per cell.  The field is bit-identical to the caller's
  * order's.  It pays for clustered particles (1 M of a Plummer sphere through
- * three nested levels: 0.55 -> 0.34 ms) and for those in no spatial order on a
- * field larger than L2 (4.2 M at random places on 256^3: 0.86 -> 0.69 ms); for
+ * three nested levels: 0.54 -> 0.34 ms) and for those in no spatial order on a
+ * field larger than L2 (4.2 M at random places on 256^3: 0.78 -> 0.69 ms); for
  * others the caller's order is faster.  APM_E_INVALID for another value. */
 apm_status apm_set_deposit_tiles(apm_ctx* ctx, int32_t on);
 

@@ -124,7 +124,7 @@ static_assert(kDepThreads % 32 == 0, "the deposit works by whole warps");
 // time, lane 8 a + p the cell a of particle p in each (y, z) row.  The kernel
 // waits on latency: a layer at a time takes 4.6 KB of shared memory a warp and
 // 64 registers a thread, 32 warps per SM (all 27 charges at once: 20 warps and
-// 1.74 ms where this takes 1.46).  Integer addition is exact and associative:
+// 1.74 ms where this took 1.46).  Integer addition is exact and associative:
 // the field does not depend on the arrangement.  Pitch 40: lanes on 32
 // particles (stores) and on 3 x 8 (loads) fall into distinct banks.
 // All levels, before (one particle per thread, x neighbours' columns merged in
@@ -661,7 +661,7 @@ cudaError_t launch_gas_init(const LevelDev& L, const GridDev* parent_grids,
 // where many particles share them and no box gathers them; a golden-ratio stride
 // through the CTAs spreads them over the bins, and each CTA keeps its own bin's
 // locality.  A Plummer sphere of 1 M through three nested levels 413 -> 344 us
-// (caller's order 551); random places on 256^3 166 -> 182 (246).
+// (caller's order 544); random places on 256^3 166 -> 182 (227).
 // In the caller's order, where there are two particles or more to a root cell,
 // neighbouring ones stored in spatial order share cells, and an instruction's
 // reductions into one cell wait for one another: it sends every fourth particle
