@@ -147,7 +147,8 @@ inline void fft_plan_reversed(const FftPlan1D& f, FftPlan1D* r) {
 // takes the smallest one >= N + 20; an isolated root of N cells takes 2 N) and
 // the usual longer ones; the rest runs the runtime-planned kernels.  The lists
 // are four groups so that they compile in parallel.  FP64 takes groups 1 to 3:
-// below 70 points a transform is too short for the FP64 pipe to bound it.
+// below 70 points it runs the runtime-planned kernels, as it always has (no plan was
+// measured there).
 #define APM_FAST_LENGTHS_0(X) \
     X(36, 6, 6, 1) X(40, 8, 5, 1) X(42, 7, 6, 1) X(45, 9, 5, 1) X(48, 8, 6, 1) X(49, 7, 7, 1) \
     X(50, 10, 5, 1) X(54, 9, 6, 1) X(56, 8, 7, 1) X(60, 10, 6, 1) X(63, 9, 7, 1) X(64, 8, 8, 1)
